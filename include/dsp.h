@@ -263,7 +263,11 @@ dsp_status dsp_get_cursor(const dsp_grid *g, int64_t *cursor, int64_t *n_steps);
  * diagonal (EXACT and STRANG_XY: the real diagonal cos(theta), so a step of
  * the product costs 8 multiply-adds instead of 12; MAGNUS4: cos|n|) and divide
  * the product by the square root of its determinant, so the applied operator
- * is unitary to FP32 rounding. */
+ * is unitary to FP32 rounding.  Where G > 1, EXACT and MAGNUS4 evaluate the
+ * operator of 16, 8 or 4 aligned steps at once, from the expansion of their
+ * product in what A changes inside the group (its coefficients are formed once
+ * per pulse), as long as the terms it drops, summed over the run, stay below
+ * 4e-6; pulses too rough for that take the steps one by one as above. */
 typedef struct {
     int32_t nx, ny, precision, scheme, valley;
     int32_t cos_degree, sinc_degree;
@@ -273,12 +277,13 @@ typedef struct {
     int32_t group_steps;
     int32_t row_begin;  /* first global row (0 unless the grid is a band)      */
     int32_t ny_total;   /* rows of the full grid (ny unless the grid is a band) */
-    int32_t row_strips; /* 1: evolve launches tile the grid in row strips of 4 rows
-                           x 256 columns (nx a multiple of 256; FP32_MIXED every
-                           scheme, FP64 EXACT and STRANG_XY), sharing each step's
-                           momentum work across a strip; 0: contiguous tiles of
-                           1024 points.  n_tiles counts the tiles of the tiling
-                           in use. */
+    int32_t row_strips; /* 1: evolve launches that go step by step tile the grid in
+                           row strips of 4 rows x 256 columns (nx a multiple of 256;
+                           FP32_MIXED every scheme, FP64 EXACT and STRANG_XY),
+                           sharing each step's momentum work across a strip; 0: in
+                           contiguous tiles of 1024 points.  n_tiles counts those
+                           tiles.  Launches on expanded groups take 32 columns x 1,
+                           2 or 4 rows per warp on any grid. */
     int32_t tan_degree; /* see above */
 } dsp_grid_info;
 /* Fills *info for the grid's current pulse (the fields above; bookkeeping,
@@ -299,10 +304,17 @@ dsp_status dsp_test_withhold_next_copy(dsp_grid *g);
  * STRANG_XY) evolve on row strips: a CTA owns 4 rows x 256 columns and shares
  * the per-step momentum work across them; a launch of one such grid whose last
  * wave of CTAs would be at most half full runs its last strips 2 rows high.
- * tiling = 1: that automatic choice (the default); 0: contiguous 1024-point
- * tiles; 2: row strips, all 4 rows high.  Every tiling gives bitwise the same
+ * Expanded step groups evolve on warps of 4, 2 or 1 rows, by what fills the chip.
+ * tiling = 1: those automatic choices (the default); 0: contiguous 1024-point
+ * tiles, warps of 1 row; 2: row strips and warps, all 4 rows high.  Every tiling gives bitwise the same
  * map and density; the hook exists so that a test can show it. */
 dsp_status dsp_test_tiling(dsp_grid *g, int32_t tiling);
+
+/* Test hook (not in the paper) on the step groups of the pulses set after it.  on =
+ * 1 (the default): a group's product of step operators may be evaluated from its
+ * expansion (see dsp_get_info); 0: always step by step.  The two agree up to
+ * rounding; the hook exists so that a test can show it. */
+dsp_status dsp_test_expansion(dsp_grid *g, int32_t on);
 
 /* Copies the raw spinor state (dsp_state_bytes bytes) to the host, or back
  * from the host, with the step cursor, for checkpoint / resume.  Synchronise.
@@ -382,7 +394,8 @@ typedef struct {
 #define DSP_REQ_CANCELLED 4
 
 /* hbm_budget_bytes > 0: admission limit on the sum of device footprints
- * (state + table + map + partial sums) of the active requests; max_active
+ * (state + table + map + partial sums; the expanded step groups of a request, at
+ * most 67 bytes a step, are not counted) of the active requests; max_active
  * >= 1; chunk_steps >= 1: steps per batched launch, rounded down to a multiple
  * of 16 when it is 16 or more (a request's result is then bitwise the same alone
  * or in any mix, see dsp_evolve).

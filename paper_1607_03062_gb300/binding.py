@@ -41,7 +41,7 @@ EXPORTS = (
     "dsp_server_query", "dsp_server_cancel", "dsp_server_destroy", "dsp_density_noalloc",
     "dsp_get_info", "dsp_solve_segmented", "dsp_sample_pulse_gauss",
     "dsp_test_withhold_next_copy", "dsp_create_band", "dsp_set_keep_final_state",
-    "dsp_test_tiling",
+    "dsp_test_tiling", "dsp_test_expansion",
 )
 
 
@@ -128,6 +128,7 @@ def lib() -> ctypes.CDLL:
                 "dsp_sample_pulse_gauss": (i32, [ctypes.POINTER(PulseSpec), i64, p, p, p, pd]),
                 "dsp_test_withhold_next_copy": (i32, [p]),
                 "dsp_test_tiling": (i32, [p, i32]),
+                "dsp_test_expansion": (i32, [p, i32]),
             }
             for name, (res, args) in sig.items():
                 fn = getattr(L, name)
@@ -313,6 +314,12 @@ def test_tiling(h: int, tiling):
     contiguous tiles, 2 row strips without the last-wave split (the results
     are bitwise the same in every case)."""
     _check(lib().dsp_test_tiling(ctypes.c_void_p(h), int(tiling)), "test_tiling")
+
+
+def test_expansion(h: int, on: bool):
+    """Test hook on the step groups of the pulses set after it: True (the default)
+    lets a group be evaluated from its expansion, False keeps to single steps."""
+    _check(lib().dsp_test_expansion(ctypes.c_void_p(h), 1 if on else 0), "test_expansion")
 
 
 def status_string(code: int) -> str:

@@ -1,7 +1,7 @@
 """Builds the in-tree CUDA library ``_build/libdsp.so`` for sm_103a.
 
-The translation units (the FP32-mixed evolve kernel on contiguous tiles; the
-row-strip kernel, compiled once per scheme and strip height; the other kernels;
+The translation units (the FP32-mixed evolve kernels on expanded step groups and on
+contiguous tiles; the row-strip kernel, compiled once per scheme and strip height; the other kernels;
 the host API; the allocation-free density) are compiled in parallel with nvcc,
 then linked into one shared library with the CUDA runtime linked statically.  Host code is compiled without floating-point
 contraction, so the host-side arithmetic (pulse tables, projection nodes) rounds
@@ -34,7 +34,8 @@ def _nvcc() -> str:
 
 def sources() -> list[str]:
     return [os.path.join(CSRC, f) for f in ("dsp_mixed.cu", "dsp_strip.cu", "dsp_kernels.cu",
-                                            "dsp_api.cpp", "dsp_noalloc.cu")]
+                                            "dsp_group.cu", "dsp_api.cpp",
+                                            "dsp_noalloc.cu")]
 
 
 # dsp_strip.cu is compiled once per scheme (EXACT, STRANG_XY, MAGNUS4) and strip height

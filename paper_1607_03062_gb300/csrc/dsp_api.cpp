@@ -71,6 +71,12 @@ struct dsp_grid {
     int32_t level = 0;
     double theta_max = 0.0;
     int32_t group = 1;  // FP32_MIXED: steps multiplied per update (choose_group)
+    // FP32_MIXED expanded groups: device memory (the caller's table, the sums and the
+    // groups' entries: GroupMemory) and whether the pulse may use them
+    void *groups = nullptr;
+    size_t groups_cap = 0;  // bytes
+    bool by_groups = false;
+    bool expand = true;  // test hook, see dsp_test_expansion
     int32_t tdeg = 0;   // FP32_MIXED: tan series degree of the step groups (choose_tan_degree)
     bool withhold_next = false;  // test hook, see dsp_test_withhold_next_copy
     bool fresh = true;      // state not yet written on the device
@@ -190,6 +196,22 @@ double theta_max(const dsp_grid *g, const double *a_mid, int64_t n, double dt)
     return dt * m;
 }
 
+// SMs of the device, looked up once for the process (152 where there is none to ask).
+int sm_count()
+{
+    static const int sms = [] {
+        int dev = 0, n = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+            n < 1) {
+            cudaGetLastError();
+            return 152;
+        }
+        return n;
+    }();
+    return sms;
+}
+
 dsp_status check_usable(const dsp_grid *g)
 {
     if (!g)
@@ -212,6 +234,35 @@ int32_t strip_tiles(const dsp_grid *g)
                                 ((static_cast<int64_t>(g->ny) + dsp::kStripHeight - 1) /
                                  dsp::kStripHeight));
 }
+
+// The largest expanded group whose angle is within the wide level's (an index of
+// group_size; kNumGroupSizes: none).
+int32_t first_group_size(double theta_max)
+{
+    int32_t i = 0;
+    while (i < dsp::kNumGroupSizes && dsp::group_size(i) * theta_max > dsp::kGroupAngleWide)
+        ++i;
+    return i;
+}
+
+// Layout of a grid's expanded-group memory: the caller's table in FP64, the sums, the
+// entries of every group size.
+struct GroupMemory {
+    size_t raw_bytes, entry_bytes;
+    explicit GroupMemory(const dsp_grid *g) : GroupMemory(g->scheme, g->n_steps) {}
+    GroupMemory(int32_t scheme, int64_t n)
+        : raw_bytes((scheme == DSP_SCHEME_MAGNUS4 ? 32 : 16) * static_cast<size_t>(n)),
+          entry_bytes(0)
+    {
+        for (int i = 0; i < dsp::kNumGroupSizes; ++i)
+            entry_bytes += sizeof(dsp::GroupEntry) * static_cast<size_t>(n / dsp::group_size(i));
+    }
+    static constexpr size_t kSums = 64;
+    size_t total() const { return raw_bytes + kSums + entry_bytes; }
+    unsigned char *sums(void *base) const { return static_cast<unsigned char *>(base) + raw_bytes; }
+    unsigned char *entries(void *base) const { return sums(base) + kSums; }
+};
+static_assert(sizeof(dsp::GroupSums) <= GroupMemory::kSums, "the sums' slot");
 
 ReqDesc make_desc(const dsp_grid *g, int64_t begin, int64_t end, bool project, void *map)
 {
@@ -261,6 +312,16 @@ ReqDesc make_desc(const dsp_grid *g, int64_t begin, int64_t end, bool project, v
     r.tdeg = g->tdeg;
     r.withhold_first_copy = g->withhold_next ? 1 : 0;
     r.table_steps = g->table_cap;
+    if (g->by_groups && end > begin) {
+        const GroupMemory m(g);
+        r.by_groups = 1;
+        r.groups.entries = reinterpret_cast<const dsp::GroupEntry *>(m.entries(g->groups));
+        r.groups.sums = reinterpret_cast<const dsp::GroupSums *>(m.sums(g->groups));
+        r.groups.n_steps = g->n_steps;
+        r.groups.eps = static_cast<float>(dsp::group_size(0) * g->theta_max);
+        r.groups.first = first_group_size(g->theta_max);
+    }
+    r.group_rows = g->tiling == 0 ? 1 : g->tiling == 2 ? 4 : 0;
     return r;
 }
 
@@ -339,14 +400,101 @@ std::vector<ReqDesc> split_last_wave(const ReqDesc &r, int precision)
     return out;
 }
 
+// Rows per warp of a launch on expanded groups: 4 (two packed row pairs per lane)
+// unless the chip's schedulers are filled better by lower warps.  A scheduler
+// takes about cost[H] issue cycles per group and warp of H rows (the lane operations
+// of dsp_group.cu, two cycles per packed one, and the column part); warps are spread
+// evenly over the schedulers and the fullest one ends the launch.
+int group_rows(const std::vector<const ReqDesc *> &reqs)
+{
+    static const int schedulers = 4 * sm_count();
+    struct Shape {
+        int rows;
+        double cost;
+    };
+    constexpr Shape shapes[3] = {{4, 1.0}, {2, 0.53}, {1, 0.32}};
+    int best = 4;
+    double best_t = 0.0;
+    for (const Shape &sh : shapes) {
+        int64_t warps = 0;
+        for (const ReqDesc *r : reqs)
+            warps += ((r->nx + 31) / 32) * static_cast<int64_t>((r->ny + sh.rows - 1) / sh.rows);
+        const double load = static_cast<double>(warps) / schedulers;
+        const double t = sh.cost * (load <= 8.0 ? std::ceil(load) : load);
+        if (sh.rows == 4 || t < 0.97 * best_t) {
+            best = sh.rows;
+            best_t = t;
+        }
+    }
+    for (const ReqDesc *r : reqs)
+        if (r->group_rows > 0)
+            best = r->group_rows;
+    return best;
+}
+
+// Queues the evolution of the requests whose groups may be evaluated expanded.
+cudaError_t launch_groups(const std::vector<const ReqDesc *> &reqs, cudaStream_t stream)
+{
+    const int rows = group_rows(reqs);
+    size_t i = 0;
+    while (i < reqs.size()) {
+        std::unique_ptr<EvolveArgs> a(new EvolveArgs());
+        std::memset(a.get(), 0, sizeof(EvolveArgs));
+        int tiles = 0, n = 0;
+        for (; i < reqs.size() && n < dsp::kMaxReqPerLaunch; ++i, ++n) {
+            ReqDesc &r = a->r[n];
+            r = *reqs[i];
+            r.store_state = 1;
+            r.project = 0;
+            r.tile_begin = tiles;
+            r.n_tiles = static_cast<int32_t>(((r.nx + 31) / 32) *
+                                             static_cast<int64_t>((r.ny + rows - 1) / rows));
+            tiles += r.n_tiles;
+        }
+        a->nreq = n;
+        a->total_tiles = tiles;
+        // one warp per CTA while that spreads the warps over more SMs
+        const int warps = tiles <= 2 * sm_count() ? 1 : dsp::kGroupWarps;
+        const cudaError_t e = dsp::launch_evolve_group(*a, rows, warps, stream);
+        if (e != cudaSuccess)
+            return e;
+    }
+    return cudaSuccess;
+}
+
 // Queues launches advancing several requests of one precision.  Requests go to
 // their kernel -- FP64 or FP32_MIXED, on contiguous tiles or on row strips, or
 // the projection kernel when every request only projects -- and are split into
 // launches of at most kMaxReqPerLaunch.  Each request reports device errors in
 // its own error word (ReqDesc::err).  A launch of one grid on row strips has its
 // last wave split (split_last_wave).
-cudaError_t launch_requests(const std::vector<ReqDesc> &reqs, int precision, cudaStream_t stream)
+cudaError_t launch_requests(const std::vector<ReqDesc> &given, int precision, cudaStream_t stream)
 {
+    // A request of a pair runs on expanded groups or, where its pulse's sums say no,
+    // step by step: both launches are queued and one of them returns at once.  Its
+    // projection is a launch of its own over the state they leave.
+    std::vector<ReqDesc> reqs, after;
+    std::vector<const ReqDesc *> grouped;
+    for (const ReqDesc &r : given) {
+        reqs.push_back(r);
+        if (!r.by_groups)
+            continue;
+        grouped.push_back(&r);
+        reqs.back().store_state = 1;
+        reqs.back().project = 0;
+        if (r.project) {
+            after.push_back(r);
+            ReqDesc &p = after.back();
+            p.step_begin = p.step_end;
+            p.by_groups = p.fresh = p.store_state = p.strips = 0;
+            p.n_tiles = static_cast<int32_t>((r.n_points + dsp::kTilePoints - 1) / dsp::kTilePoints);
+        }
+    }
+    if (!grouped.empty()) {
+        const cudaError_t e = launch_groups(grouped, stream);
+        if (e != cudaSuccess)
+            return e;
+    }
     bool proj = !reqs.empty();
     for (const ReqDesc &r : reqs)
         proj = proj && project_only(r);
@@ -392,7 +540,7 @@ cudaError_t launch_requests(const std::vector<ReqDesc> &reqs, int precision, cud
                 return e;
         }
     }
-    return cudaSuccess;
+    return after.empty() ? cudaSuccess : launch_requests(after, precision, stream);
 }
 
 cudaError_t launch_finalizes(const std::vector<dsp::FinDesc> &fins, cudaStream_t stream)
@@ -609,6 +757,10 @@ void free_grid_memory(dsp_grid *g)
         cudaFree(g->nodes);
     if (g->seg_buf)
         cudaFree(g->seg_buf);
+    if (g->groups)
+        cudaFree(g->groups);
+    g->groups = nullptr;
+    g->groups_cap = 0;
     g->seg_buf = nullptr;
     g->seg_cap = 0;
     g->state = g->table = g->own_map = nullptr;
@@ -708,7 +860,6 @@ dsp_status prepare_pulse(dsp_grid *g, const double *a_mid, int64_t n_steps, doub
     dsp_status s = validate_pulse_args(g, a_mid, n_samples, dt, a_in, a_out, &tmax);
     if (s != DSP_OK)
         return s;
-    build_table(g, a_mid, n_steps, dt, host);
     g->has_pulse = true;
     g->n_steps = n_steps;
     g->cursor = 0;
@@ -721,11 +872,41 @@ dsp_status prepare_pulse(dsp_grid *g, const double *a_mid, int64_t n_steps, doub
     g->level = choose_level(g->precision, tmax, n_steps);
     g->tdeg = g->precision == DSP_FP32_MIXED ? choose_tan_degree(g->scheme, tmax, n_steps) : 0;
     g->group = choose_group(g->precision, g->scheme, g->tdeg, tmax);
+    // groups that the grid's piece rule allows may be evaluated expanded: then the
+    // device makes the per-step table too, from the caller's
+    g->by_groups = g->expand && g->group > 1 && g->scheme != DSP_SCHEME_STRANG_XY &&
+                   first_group_size(tmax) < dsp::kNumGroupSizes;
+    if (g->by_groups) {
+        host.resize(GroupMemory(g).raw_bytes);
+        std::memcpy(host.data(), a_mid, host.size());
+    } else {
+        build_table(g, a_mid, n_steps, dt, host);
+    }
     g->fresh = true;
     g->projected = false;
     g->state_stale = false;
     build_nodes(g, nodes);
     return DSP_OK;
+}
+
+// Queues the expansion of the grid's groups (and its per-step table) from the
+// caller's table, which is in the grid's group memory already.
+cudaError_t prep_groups(const dsp_grid *g, cudaStream_t stream)
+{
+    const GroupMemory m(g);
+    dsp::PrepArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.raw = static_cast<const double *>(g->groups);
+    a.n_steps = g->n_steps;
+    a.sdt = (g->valley > 0 ? 1.0 : -1.0) * g->dt;
+    a.scheme = g->scheme;
+    a.first = first_group_size(g->theta_max);
+    a.eps = static_cast<float>(dsp::group_size(0) * g->theta_max);
+    a.table = g->table;
+    a.entries = reinterpret_cast<dsp::GroupEntry *>(m.entries(g->groups));
+    a.sums = reinterpret_cast<dsp::GroupSums *>(m.sums(g->groups));
+    const cudaError_t e = cudaMemsetAsync(a.sums, 0, sizeof(dsp::GroupSums), stream);
+    return e == cudaSuccess ? dsp::launch_prep_groups(a, stream) : e;
 }
 
 dsp_status set_pulse_impl(dsp_grid *g, const double *a_mid, int64_t n_steps, double dt,
@@ -738,6 +919,25 @@ dsp_status set_pulse_impl(dsp_grid *g, const double *a_mid, int64_t n_steps, dou
     if (s != DSP_OK)
         return s;
     cudaError_t e = cudaSuccess;
+    const size_t gbytes = staged.by_groups ? GroupMemory(&staged).total() : 0;
+    if (gbytes > g->groups_cap) {
+        if (g->groups) {
+            e = cudaStreamSynchronize(g->stream);  // the old groups may still be read
+            if (e == cudaSuccess)
+                e = cudaFree(g->groups);
+            g->groups = nullptr;
+            g->groups_cap = 0;
+            g->by_groups = false;  // the pulse before goes on step by step
+        }
+        if (e == cudaSuccess)
+            e = cudaMalloc(&g->groups, gbytes);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            g->groups = nullptr;
+            return e == cudaErrorMemoryAllocation ? DSP_E_NOMEM : latch_cuda(g, e);
+        }
+        g->groups_cap = gbytes;
+    }
     if (n_steps > g->table_cap) {
         if (g->table) {
             e = cudaStreamSynchronize(g->stream);  // old table may still be read
@@ -755,7 +955,13 @@ dsp_status set_pulse_impl(dsp_grid *g, const double *a_mid, int64_t n_steps, dou
         g->table_cap = n_steps;
     }
     if (n_steps > 0) {
-        e = cudaMemcpyAsync(g->table, host.data(), host.size(), cudaMemcpyHostToDevice, g->stream);
+        e = cudaMemcpyAsync(staged.by_groups ? g->groups : g->table, host.data(), host.size(),
+                            cudaMemcpyHostToDevice, g->stream);
+        if (e == cudaSuccess && staged.by_groups) {
+            staged.table = g->table;
+            staged.groups = g->groups;
+            e = prep_groups(&staged, g->stream);
+        }
         if (e != cudaSuccess)
             return latch_cuda(g, e);
     }
@@ -764,6 +970,8 @@ dsp_status set_pulse_impl(dsp_grid *g, const double *a_mid, int64_t n_steps, dou
         return latch_cuda(g, e);
     staged.table = g->table;
     staged.table_cap = g->table_cap;
+    staged.groups = g->groups;
+    staged.groups_cap = g->groups_cap;
     *g = staged;
     return DSP_OK;
 }
@@ -953,17 +1161,7 @@ dsp_status dsp_solve_segmented(dsp_grid *g, int32_t segments, void *map_dev, dou
         // segments are short and latency bound, and the FP64 combine grows with S: one
         // segment-tile per two SMs.  At least 16 steps a segment.  (Measured on the 64^2
         // x 2000-step case, 4 tiles: S = 38 / 19 beat S = 76 by 8% / 40%.)
-        // looked up once for the process (a thread-safe static initialisation)
-        static const int sms = [] {
-            int dev = 0, n = 0;
-            if (cudaGetDevice(&dev) != cudaSuccess ||
-                cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-                n < 1) {
-                cudaGetLastError();
-                return 152;
-            }
-            return n;
-        }();
+        const int sms = sm_count();
         const int64_t ctas = g->precision == DSP_FP64 ? sms : (sms + 1) / 2;
         S = (ctas + g->n_tiles - 1) / g->n_tiles;
         S = std::min<int64_t>(S, g->n_steps / 16);
@@ -1149,6 +1347,17 @@ dsp_status dsp_test_tiling(dsp_grid *g, int32_t tiling)
     if (tiling < 0 || tiling > 2)
         return DSP_E_INVALID;
     g->tiling = tiling;
+    return DSP_OK;
+}
+
+dsp_status dsp_test_expansion(dsp_grid *g, int32_t on)
+{
+    dsp_status s = check_usable(g);
+    if (s != DSP_OK)
+        return s;
+    if (on != 0 && on != 1)
+        return DSP_E_INVALID;
+    g->expand = on != 0;
     return DSP_OK;
 }
 
@@ -1433,7 +1642,8 @@ struct ServerReq {
     std::vector<double> a_mid;
     int32_t state = DSP_REQ_QUEUED;
     dsp_grid g{};             // pointers borrowed from `block`
-    void *block = nullptr;    // one pool allocation: state | table | partials | scalars | map
+    void *block = nullptr;    // one pool allocation: state | table, nodes, groups | partials |
+                              // scalars | map
     void *map_dev = nullptr;
     int64_t footprint = 0;
     int64_t finish_iter = -1;  // iteration whose launch holds the last steps
@@ -1513,13 +1723,24 @@ dsp_status server_admit(dsp_server *s, ServerReq *r)
     if (st != DSP_OK)
         return st;
     r->g.keep_final_state = false;  // a finished request's state is never read again
-    // table (padded to 16 bytes) and projection nodes, uploaded in one copy
+    // One copy uploads the table (padded to 16 bytes) and the projection nodes; for
+    // expanded groups the nodes and the caller's table, from which the device makes
+    // the rest: block holds table | nodes | group memory, the last two from o_nodes.
     const size_t tb = table_bytes(p.precision, p.scheme, p.n_steps);
-    host.resize(tb + node_bytes(&r->g), 0);
-    std::memcpy(host.data() + tb, nodes.data(), node_bytes(&r->g));
+    const size_t nb = (node_bytes(&r->g) + 15) & ~static_cast<size_t>(15);
+    const bool by_groups = r->g.by_groups;
+    std::vector<unsigned char> up((by_groups ? 0 : tb) + nb, 0);
+    std::memcpy(up.data() + (by_groups ? 0 : tb), nodes.data(), node_bytes(&r->g));
+    if (by_groups)
+        up.insert(up.end(), host.begin(), host.end());
+    else if (!host.empty())
+        std::memcpy(up.data(), host.data(), host.size());
+    host.swap(up);
+    const size_t o_up = by_groups ? tb : 0;  // where the upload lands after o_table
+    const size_t region = tb + nb + (by_groups ? GroupMemory(&r->g).total() : 0);
     const size_t pts = static_cast<size_t>(r->g.n_points);
     const size_t o_table = align256(32 * pts);
-    const size_t o_part = o_table + align256(host.size());
+    const size_t o_part = o_table + align256(region);
     const size_t o_scal = o_part + align256(8 * static_cast<size_t>(r->g.n_parts));
     const size_t o_map = o_scal + align256(sizeof(DeviceScalars));
     const size_t total = o_map + align256(map_elem_bytes(p.precision) * pts);
@@ -1537,6 +1758,7 @@ dsp_status server_admit(dsp_server *s, ServerReq *r)
     r->g.table = b + o_table;
     r->g.table_cap = p.n_steps;
     r->g.nodes = reinterpret_cast<float2 *>(b + o_table + tb);
+    r->g.groups = by_groups ? b + o_table + tb + nb : nullptr;
     r->g.partials = reinterpret_cast<double *>(b + o_part);
     r->g.scal = reinterpret_cast<DeviceScalars *>(b + o_scal);
     r->map_dev = b + o_map;
@@ -1564,8 +1786,9 @@ dsp_status server_admit(dsp_server *s, ServerReq *r)
             s->staging_cap = host.size();
         }
         std::memcpy(s->staging, host.data(), host.size());
-        if (cudaMemcpyAsync(r->g.table, s->staging, host.size(), cudaMemcpyHostToDevice,
+        if (cudaMemcpyAsync(b + o_table + o_up, s->staging, host.size(), cudaMemcpyHostToDevice,
                             s->copy_stream) != cudaSuccess ||
+            (by_groups && prep_groups(&r->g, s->copy_stream) != cudaSuccess) ||
             cudaEventRecord(s->upload_done, s->copy_stream) != cudaSuccess ||
             cudaStreamWaitEvent(s->stream, s->upload_done, 0) != cudaSuccess)
             return server_fail(s, DSP_E_CUDA);

@@ -455,6 +455,40 @@ __device__ __forceinline__ bool table_range_ok(const ReqDesc &R, int64_t first, 
 #endif
 }
 
+// Entries of all group sizes before size i (kNumGroupSizes: all of them).
+__host__ __device__ __forceinline__ int64_t group_entries_before(int64_t n_steps, int i)
+{
+    int64_t n = 0;
+    for (int k = 0; k < i; ++k)
+        n += n_steps / group_size(k);
+    return n;
+}
+
+// The group size a run takes (an index of group_size, kNumGroupSizes: step by
+// step) and whether its groups are evaluated at the wide level.
+struct GroupPick {
+    int size;
+    bool wide;
+};
+__device__ __forceinline__ GroupPick pick_plan(const GroupTable &t)
+{
+    constexpr unsigned long long budget =
+        static_cast<unsigned long long>(kPlanBudget / kPlanUnit);
+    for (int i = t.first; i < kNumGroupSizes; ++i)
+        if (t.n_steps >= group_size(i) && __ldg(&t.sums->wide[i]) <= budget) {
+            const float eps = t.eps / static_cast<float>(1 << i);
+            return {i, !(eps <= static_cast<float>(kGroupAngleLite) &&
+                         __ldg(&t.sums->lite[i]) <= budget)};
+        }
+    return {kNumGroupSizes, true};
+}
+// A step-by-step kernel leaves a request of a pair to the expanded groups where the
+// plan picked them.
+__device__ __forceinline__ bool left_to_groups(const ReqDesc &R)
+{
+    return R.by_groups && pick_plan(R.groups).size < kNumGroupSizes;
+}
+
 // Bounds-check builds verify a CTA's tile index; a bad one sets kErrBounds.
 __device__ __forceinline__ bool tile_ok(const ReqDesc &R, int tile, int *err)
 {

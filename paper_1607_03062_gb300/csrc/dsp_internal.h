@@ -20,7 +20,7 @@ constexpr int kGranule = 256;
 // Spinors per thread (independent momenta advanced together for ILP).
 constexpr int kSpinorsPerThread = 2;
 constexpr int kThreads = kTilePoints / kSpinorsPerThread;
-// Requests one evolve launch can carry in its parameter block (96 x 232 bytes:
+// Requests one evolve launch can carry in its parameter block (96 x 280 bytes:
 // within the 32 KB kernel-parameter limit).
 constexpr int kMaxReqPerLaunch = 96;
 // Device-side error bits (the launch's error word).
@@ -70,6 +70,60 @@ constexpr double kSecSeries[kTanTerms] = {1.0,
 constexpr int kNumTanDegrees = 5;
 constexpr int kTanDegrees[kNumTanDegrees] = {1, 2, 3, 4, 6};
 
+// Expanded step groups (dsp_group.cu): the coefficients of one group, in FP32.
+//   v[0..3]   sum of s dt A_x over the group as hi + lo; m1_y, n3_y
+//   v[4..7]   n5_y, u2_y, u4_y, K_xx
+//   v[8..11]  K_yx; sum of s dt A_y as hi + lo; C
+//   v[12..15] m1_x, n3_x, n5_x, u2_x
+//   v[16..19] u4_x, K_xy, K_yy, 0
+struct GroupEntry {
+    float v[20];
+};
+// Largest group angle G theta_max of each level of the expansion.  In an exact CPU
+// emulation of the kernel's FP32 arithmetic against FP64 steps (2-norm error of
+// |c+|^2 over 600 points; step-by-step chains, then lite or wide): 2048^2 sin^2
+// pulse, angle 0.16: 4.2e-7, 2.8e-7; paper pulse, 0.55: 5.7e-7, 2.1e-7; Gaussian
+// pulse, 0.63: 2.5e-7, 1.7e-7; 64^2 sin^2 pulse, 0.49: 9.4e-8, 5.8e-8.
+constexpr double kGroupAngleLite = 0.25, kGroupAngleWide = 0.72;
+constexpr int kGroupWarps = 4;  // most warps per CTA of the expanded-group kernel
+constexpr int kNumGroupSizes = 3;
+// Group sizes 16, 8, 4 (i = 0, 1, 2).
+__host__ __device__ constexpr int group_size(int i) { return 16 >> i; }
+
+// What a run's groups come to, on the device: per group size the sums of what the
+// wide and the lite level drop (kPlanUnit fixed point, so the sum does not depend
+// on its order).
+struct GroupSums {
+    unsigned long long wide[kNumGroupSizes], lite[kNumGroupSizes];
+};
+constexpr double kPlanUnit = 0x1p-50;
+// Bound on those sums, a worst case in which every group errs in the same direction.
+// FP32_MIXED's target is 1e-5 per point.
+constexpr double kPlanBudget = 4e-6;
+
+// The groups of a pulse: entries of each size, one size after the other, and the
+// sums.  The kernels pick the largest size whose sum is in the budget (pick_plan),
+// or none: then the run goes step by step.
+struct GroupTable {
+    const GroupEntry *entries;
+    const GroupSums *sums;
+    int64_t n_steps;
+    float eps;          // group_size(0) * theta_max
+    int32_t first;      // first group size within kGroupAngleWide (kNumGroupSizes: none)
+};
+
+struct PrepArgs {
+    const double *raw;  // the caller's table: (A_x, A_y) per step, MAGNUS4 two per step
+    int64_t n_steps;
+    double sdt;         // valley * dt
+    int32_t scheme;
+    int32_t first;
+    float eps;
+    void *table;        // per-step table the kernels read (ReqDesc::table)
+    GroupEntry *entries;
+    GroupSums *sums;    // zeroed
+};
+
 struct ReqDesc {
     // Per step, s = valley (valley K- steps as K+ on -P: its operator is K+'s at -P):
     //   EXACT, STRANG_XY: s*dt*A at the step midpoint, as float2 (FP32_MIXED) or
@@ -117,6 +171,10 @@ struct ReqDesc {
     int32_t tail_split;  // 1: a launch of this request alone may split its last wave
                          // (host only; see split_last_wave)
     int64_t table_steps;          // entries in the table (checked by bounds-check builds)
+    GroupTable groups;   // FP32_MIXED expanded groups (entries null: none)
+    int32_t by_groups;   // 1: this launch is one of a pair, on expanded groups or step by
+                         // step: the kernel that the plan does not pick does nothing
+    int32_t group_rows;  // rows per warp asked for by the tiling hook; 0: by size
 };
 
 // Steps are grouped (G = 16, 8, 4 or 2, the largest allowed) when G * theta_max
@@ -203,6 +261,11 @@ cudaError_t launch_evolve_mixed(const EvolveArgs &args, cudaStream_t stream);
 // args has that scheme and strip_h).
 cudaError_t launch_evolve_strip(const EvolveArgs &args, int scheme, int strip_h,
                                 cudaStream_t stream);
+// FP32_MIXED on expanded groups (every request has by_groups, and n_tiles counts its
+// tiles of 32 columns x rows); `warps` tiles per CTA.  Does not project.
+cudaError_t launch_evolve_group(const EvolveArgs &args, int rows, int warps, cudaStream_t stream);
+// Per-step table, group entries and sums of a pulse from the caller's table.
+cudaError_t launch_prep_groups(const PrepArgs &args, cudaStream_t stream);
 // CTAs of the 4-row strip kernel of a precision (and FP32_MIXED scheme) that one
 // SM holds at once.
 cudaError_t strip_ctas_per_sm(int precision, int scheme, int *ctas);

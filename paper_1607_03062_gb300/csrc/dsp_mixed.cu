@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(kMixedThreads, kMixedMinBlocks)
     const int r = find_request(args);
     const ReqDesc &R = args.r[r];
     const int tile = static_cast<int>(blockIdx.x) - R.tile_begin;
-    if (!tile_ok(R, tile, R.err))
+    if (!tile_ok(R, tile, R.err) || left_to_groups(R))
         return;
     if (R.scheme == 0)
         body_mixed<0>(R, tile, smem, bars, R.err);

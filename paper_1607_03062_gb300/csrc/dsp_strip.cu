@@ -598,7 +598,7 @@ __global__ void __launch_bounds__(kStripThreads, kMixedMinBlocks)
     const int r = find_request(args);
     const ReqDesc &R = args.r[r];
     const int tile = static_cast<int>(blockIdx.x) - R.tile_begin;
-    if (!tile_ok(R, tile, R.err))
+    if (!tile_ok(R, tile, R.err) || left_to_groups(R))
         return;
     body_strip<SCHEME, NP>(R, tile, smem, bars, R.err);
 }

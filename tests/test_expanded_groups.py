@@ -1,0 +1,107 @@
+"""FP32-mixed step groups evaluated from their expansion (EXACT and MAGNUS4): against the FP64
+oracle, against the same steps taken one by one, and bitwise across the kernel's warp tiles, at
+grid sizes around its 32-column, 4-row tiles.
+
+Tolerance between the two paths: each is within its own rounding of the FP64 steps (a few 1e-7 at
+these step counts, below 1e-6), and the expansion drops at most 4e-6 in sum over a run: 6e-6."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1607_03062_gb300 import binding as B
+from paper_1607_03062_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+PATHS = 6e-6
+# (nx, ny): one point; a column short of a tile; a column and a row over; whole tiles; odd
+SIZES = [(1, 1), (31, 3), (33, 5), (64, 8), (97, 43)]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    from paper_1607_03062_gb300 import build
+    build.build()
+    B.lib()
+    torch.cuda.set_device(0)
+
+
+def solve(size, table, scheme="exact", valley=1, expand=True, tiling=1, pieces=None, rows=None):
+    a, a_in, a_out, dt = table
+    g = B.Grid(size[0], size[1], (-3.0, 5.0), (-2.5, 3.5), "fp32_mixed", scheme, valley, rows=rows)
+    B.test_expansion(g.h, expand)
+    B.test_tiling(g.h, tiling)
+    g.set_pulse(a, dt, a_in, a_out)
+    for p in pieces or []:
+        g.evolve(p)
+    m, n = g.solve()
+    torch.cuda.synchronize()
+    out = m.double().cpu().numpy().copy()
+    g.close()
+    return out, n
+
+
+# steps -> the largest group within the wide level's angle: 16, 16, 8 and 4 (theta_max ~ 160 /
+# steps); a count that is no multiple of 16 leaves steps alone at the end
+@pytest.mark.parametrize("size", SIZES)
+@pytest.mark.parametrize("scheme,steps", [("exact", 24005), ("exact", 5000), ("exact", 2403),
+                                          ("exact", 1501), ("magnus4", 6007), ("magnus4", 2600)])
+def test_expansion_against_oracle_and_single_steps(orc, size, scheme, steps):
+    pulse = W.sin2_pulse(2.0, 1.2, 4.0, eps=0.6)
+    sample, oracle_table = ((B.sample_pulse_gauss, orc.pulse_table_gauss) if scheme == "magnus4"
+                            else (B.sample_pulse, orc.pulse_table))
+    valley = -1 if steps % 2 else 1
+    a, a_in, a_out, dt = oracle_table(pulse, steps)
+    ref, _, _, nref = orc.solve_grid(size[0], size[1], (-3.0, 5.0), (-2.5, 3.5), a, dt, a_in,
+                                     a_out, scheme=scheme, valley=valley)
+    tab = sample(pulse, steps)
+    m, n = solve(size, tab, scheme, valley)
+    assert np.abs(m - ref).max() <= 1e-5 and abs(n - nref) <= 1e-4 * nref
+    m1, _ = solve(size, tab, scheme, valley, expand=False)
+    assert np.abs(m - m1).max() <= PATHS
+    for tiling in (0, 2):  # one row per warp, four rows per warp
+        m2, n2 = solve(size, tab, scheme, valley, tiling=tiling)
+        assert np.array_equal(m, m2) and n == n2
+    # pieces on multiples of 16 meet the same groups; others change rounding only
+    m2, n2 = solve(size, tab, scheme, valley, pieces=[16, 640, 16 * 33])
+    assert np.array_equal(m, m2) and n == n2
+    m2, _ = solve(size, tab, scheme, valley, pieces=[3, 6, 1, 700])
+    assert np.abs(m - m2).max() <= PATHS
+
+
+@pytest.mark.parametrize("kind", ["noise", "step", "spikes"])
+def test_rough_tables_meet_the_oracle(orc, kind):
+    """Potentials that jump from step to step: what the expansion would drop is over its bound
+    for the larger jumps, and the run goes step by step; either way it meets the oracle."""
+    rng = np.random.default_rng(3)
+    for amp in (1e-3, 0.05, 1.0):
+        n = 1777
+        a = np.zeros((n, 2))
+        if kind == "noise":
+            a = amp * rng.standard_normal((n, 2)).clip(-3, 3)
+        elif kind == "step":
+            a[n // 3:] = amp
+        else:
+            a[rng.integers(0, n, 40)] = amp
+        a_in, a_out, dt = np.zeros(2), a[-1].copy(), 0.003
+        ref, _, _, nref = orc.solve_grid(65, 19, (-3.0, 5.0), (-2.5, 3.5), a, dt, a_in, a_out)
+        m, nd = solve((65, 19), (a, a_in, a_out, dt))
+        assert np.abs(m - ref).max() <= 1e-5
+        m1, _ = solve((65, 19), (a, a_in, a_out, dt), expand=False)
+        assert np.abs(m - m1).max() <= PATHS
+
+
+def test_bands_and_segments_on_expanded_groups():
+    """A row band holds the full grid's points bitwise, and the time-parallel solve agrees."""
+    tab = B.sample_pulse(W.sin2_pulse(2.0, 1.2, 4.0, eps=0.6), 9001)
+    full, _ = solve((70, 45), tab)
+    band, _ = solve((70, 45), tab, rows=(7, 30))
+    assert np.array_equal(band, full[7:30])
+    a, a_in, a_out, dt = tab
+    for segments in (0, 7):
+        g = B.Grid(70, 45, (-3.0, 5.0), (-2.5, 3.5), "fp32_mixed")
+        g.set_pulse(a, dt, a_in, a_out)
+        m, _ = g.solve_segmented(segments)
+        torch.cuda.synchronize()
+        assert np.abs(m.double().cpu().numpy() - full).max() <= PATHS
+        g.close()
