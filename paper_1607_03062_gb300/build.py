@@ -1,7 +1,8 @@
 """Builds the in-tree CUDA library ``_build/libdsp.so`` for sm_103a.
 
 The translation units (the FP32-mixed evolve kernels on expanded step groups and on
-contiguous tiles; the row-strip kernel, compiled once per scheme and strip height; the other kernels;
+contiguous tiles; the row-strip kernel, compiled once per scheme and strip height; the FP64 evolve kernels;
+projection and density;
 the host API; the allocation-free density) are compiled in parallel with nvcc,
 then linked into one shared library with the CUDA runtime linked statically.  Host code is compiled without floating-point
 contraction, so the host-side arithmetic (pulse tables, projection nodes) rounds
@@ -34,7 +35,7 @@ def _nvcc() -> str:
 
 def sources() -> list[str]:
     return [os.path.join(CSRC, f) for f in ("dsp_mixed.cu", "dsp_strip.cu", "dsp_kernels.cu",
-                                            "dsp_group.cu", "dsp_api.cpp",
+                                            "dsp_group.cu", "dsp_f64.cu", "dsp_api.cpp",
                                             "dsp_noalloc.cu")]
 
 

@@ -219,8 +219,9 @@ dsp_status check_usable(const dsp_grid *g)
     return g->latched;
 }
 
-// Grids whose rows split into whole 256-column strips evolve on row-strip tiles
-// (ReqDesc::strips): FP32_MIXED in every scheme, FP64 in EXACT and STRANG_XY.
+// FP32_MIXED grids whose rows split into whole 256-column strips go step by step on
+// row-strip tiles (ReqDesc::strips).  (FP64 by size: f64_lanes; the flag is what
+// dsp_get_info reports.)
 // Every point's arithmetic is the same on either tiling.
 bool use_strips(const dsp_grid *g)
 {
@@ -301,7 +302,6 @@ ReqDesc make_desc(const dsp_grid *g, int64_t begin, int64_t end, bool project, v
     r.fresh = g->fresh ? 1 : 0;
     r.project = project ? 1 : 0;
     r.n_tiles = g->n_tiles;
-    // a projection of the state on the device runs on contiguous tiles
     r.strips = use_strips(g) && !(read_only && project) ? 1 : 0;
     r.strip_h = dsp::kStripHeight;
     r.strip_row0 = 0;
@@ -321,7 +321,7 @@ ReqDesc make_desc(const dsp_grid *g, int64_t begin, int64_t end, bool project, v
         r.groups.eps = static_cast<float>(dsp::group_size(0) * g->theta_max);
         r.groups.first = first_group_size(g->theta_max);
     }
-    r.group_rows = g->tiling == 0 ? 1 : g->tiling == 2 ? 4 : 0;
+    r.rows = g->tiling == 0 ? 1 : g->tiling == 2 ? 4 : 0;
     return r;
 }
 
@@ -344,16 +344,16 @@ bool project_only(const ReqDesc &r)
 // wave takes about half as long.  Grids of at most half a wave are all 2-row
 // strips.  Every point's arithmetic, and every granule, is unchanged: only
 // which CTA computes which rows.  Returns the descriptors to launch.
-std::vector<ReqDesc> split_last_wave(const ReqDesc &r, int precision)
+std::vector<ReqDesc> split_last_wave(const ReqDesc &r)
 {
     std::vector<ReqDesc> out(1, r);
     if (!r.strips || !r.tail_split || r.strip_h != dsp::kStripHeight)
         return out;
-    // per kernel: [0] FP64, [1 + scheme] FP32_MIXED; looked up once for the process
-    // (handles may be used from different host threads, so under a lock)
+    // per scheme, looked up once for the process (handles may be used from different
+    // host threads, so under a lock)
     static std::mutex cache_mutex;
-    static int sms[4] = {0, 0, 0, 0}, per_sm[4] = {0, 0, 0, 0};
-    const int p = precision == DSP_FP64 ? 0 : 1 + r.scheme;
+    static int sms[3] = {0, 0, 0}, per_sm[3] = {0, 0, 0};
+    const int p = r.scheme;
     int n_sm = 0, n_per_sm = 0;
     {
         std::lock_guard<std::mutex> lock(cache_mutex);
@@ -362,7 +362,7 @@ std::vector<ReqDesc> split_last_wave(const ReqDesc &r, int precision)
             if (cudaGetDevice(&dev) != cudaSuccess ||
                 cudaDeviceGetAttribute(&sms[p], cudaDevAttrMultiProcessorCount, dev) !=
                     cudaSuccess ||
-                dsp::strip_ctas_per_sm(precision == DSP_FP64 ? 0 : 1, r.scheme, &per_sm[p]) !=
+                dsp::strip_ctas_per_sm(r.scheme, &per_sm[p]) !=
                     cudaSuccess ||
                 per_sm[p] < 1) {
                 cudaGetLastError();
@@ -400,14 +400,67 @@ std::vector<ReqDesc> split_last_wave(const ReqDesc &r, int precision)
     return out;
 }
 
-// Rows per warp of a launch on expanded groups: 4 (two packed row pairs per lane)
-// unless the chip's schedulers are filled better by lower warps.  A scheduler
-// takes about cost[H] issue cycles per group and warp of H rows (the lane operations
-// of dsp_group.cu, two cycles per packed one, and the column part); warps are spread
-// evenly over the schedulers and the fullest one ends the launch.
-int group_rows(const std::vector<const ReqDesc *> &reqs)
+// A projection-only descriptor of a request's state.
+ReqDesc projection_of(const ReqDesc &r)
 {
-    static const int schedulers = 4 * sm_count();
+    ReqDesc p = r;
+    p.step_begin = p.step_end;
+    p.by_groups = p.fresh = p.store_state = p.strips = 0;
+    p.n_tiles = static_cast<int32_t>((r.n_points + dsp::kTilePoints - 1) / dsp::kTilePoints);
+    return p;
+}
+
+// Fills a launch from reqs[i...] (at most kMaxReqPerLaunch; tiles(r) each) and returns
+// the next i.
+template <typename Tiles>
+size_t fill_launch(const std::vector<ReqDesc> &reqs, size_t i, EvolveArgs &a, Tiles tiles)
+{
+    std::memset(&a, 0, sizeof(EvolveArgs));
+    for (; i < reqs.size() && a.nreq < dsp::kMaxReqPerLaunch; ++i) {
+        ReqDesc &r = a.r[a.nreq++];
+        r = reqs[i];
+        r.tile_begin = a.total_tiles;
+        r.n_tiles = static_cast<int32_t>(tiles(r));
+        a.total_tiles += r.n_tiles;
+    }
+    return i;
+}
+
+cudaError_t launch_projections(const std::vector<ReqDesc> &reqs, int precision,
+                               cudaStream_t stream)
+{
+    std::unique_ptr<EvolveArgs> a(new EvolveArgs());
+    for (size_t i = 0; i < reqs.size();) {
+        i = fill_launch(reqs, i, *a, [](const ReqDesc &r) { return r.n_tiles; });
+        const cudaError_t e = dsp::launch_project(*a, precision, stream);
+        if (e != cudaSuccess)
+            return e;
+    }
+    return cudaSuccess;
+}
+
+int64_t row_tiles(const ReqDesc &r, int rows)
+{
+    return ((static_cast<int64_t>(r.nx) + 31) / 32) * ((r.ny + rows - 1) / rows);
+}
+
+// Warps per CTA: one while that spreads a launch's warps over more SMs.
+int warps_per_cta(int64_t tiles, int most) { return tiles <= 2 * sm_count() ? 1 : most; }
+
+// The time a launch of `warps` warps of `cost` takes: they are spread evenly over the
+// schedulers, and the fullest one ends the launch.
+double launch_time(int64_t warps, double cost)
+{
+    const double load = static_cast<double>(warps) / (4 * sm_count());
+    return cost * (load <= 8.0 ? std::ceil(load) : load + 0.5);
+}
+
+// Rows per warp of a launch on expanded groups: 4 (two packed row pairs per lane)
+// unless lower warps fill the chip's schedulers better.  Costs: issue cycles of a warp
+// per group (the lane operations of dsp_group.cu, two cycles per packed one, and the
+// column part), relative to 4 rows.
+int group_rows(const std::vector<ReqDesc> &reqs)
+{
     struct Shape {
         int rows;
         double cost;
@@ -417,130 +470,150 @@ int group_rows(const std::vector<const ReqDesc *> &reqs)
     double best_t = 0.0;
     for (const Shape &sh : shapes) {
         int64_t warps = 0;
-        for (const ReqDesc *r : reqs)
-            warps += ((r->nx + 31) / 32) * static_cast<int64_t>((r->ny + sh.rows - 1) / sh.rows);
-        const double load = static_cast<double>(warps) / schedulers;
-        const double t = sh.cost * (load <= 8.0 ? std::ceil(load) : load);
+        for (const ReqDesc &r : reqs)
+            warps += row_tiles(r, sh.rows);
+        const double t = launch_time(warps, sh.cost);
         if (sh.rows == 4 || t < 0.97 * best_t) {
             best = sh.rows;
             best_t = t;
         }
     }
-    for (const ReqDesc *r : reqs)
-        if (r->group_rows > 0)
-            best = r->group_rows;
+    for (const ReqDesc &r : reqs)
+        if (r.rows > 0)
+            best = r.rows;
     return best;
 }
 
 // Queues the evolution of the requests whose groups may be evaluated expanded.
-cudaError_t launch_groups(const std::vector<const ReqDesc *> &reqs, cudaStream_t stream)
+cudaError_t launch_groups(const std::vector<ReqDesc> &reqs, cudaStream_t stream)
 {
     const int rows = group_rows(reqs);
-    size_t i = 0;
-    while (i < reqs.size()) {
-        std::unique_ptr<EvolveArgs> a(new EvolveArgs());
-        std::memset(a.get(), 0, sizeof(EvolveArgs));
-        int tiles = 0, n = 0;
-        for (; i < reqs.size() && n < dsp::kMaxReqPerLaunch; ++i, ++n) {
-            ReqDesc &r = a->r[n];
-            r = *reqs[i];
-            r.store_state = 1;
-            r.project = 0;
-            r.tile_begin = tiles;
-            r.n_tiles = static_cast<int32_t>(((r.nx + 31) / 32) *
-                                             static_cast<int64_t>((r.ny + rows - 1) / rows));
-            tiles += r.n_tiles;
-        }
-        a->nreq = n;
-        a->total_tiles = tiles;
-        // one warp per CTA while that spreads the warps over more SMs
-        const int warps = tiles <= 2 * sm_count() ? 1 : dsp::kGroupWarps;
-        const cudaError_t e = dsp::launch_evolve_group(*a, rows, warps, stream);
+    std::unique_ptr<EvolveArgs> a(new EvolveArgs());
+    for (size_t i = 0; i < reqs.size();) {
+        i = fill_launch(reqs, i, *a, [&](const ReqDesc &r) { return row_tiles(r, rows); });
+        const cudaError_t e = dsp::launch_evolve_group(
+            *a, rows, warps_per_cta(a->total_tiles, dsp::kGroupWarps), stream);
         if (e != cudaSuccess)
             return e;
     }
     return cudaSuccess;
 }
 
-// Queues launches advancing several requests of one precision.  Requests go to
-// their kernel -- FP64 or FP32_MIXED, on contiguous tiles or on row strips, or
-// the projection kernel when every request only projects -- and are split into
-// launches of at most kMaxReqPerLaunch.  Each request reports device errors in
-// its own error word (ReqDesc::err).  A launch of one grid on row strips has its
-// last wave split (split_last_wave).
-cudaError_t launch_requests(const std::vector<ReqDesc> &given, int precision, cudaStream_t stream)
+// Shape of an FP64 launch (launch_evolve_f64's lanes) by the FP64 instructions of its
+// fullest scheduler (dsp_f64.cu): per warp and step 65 for 4 rows x 32 columns, 18, 9
+// or 6 flat on 1, 2 or 4 lanes per point (EXACT); STRANG_XY ~70 and 36, whose series
+// are FP64 and shared along rows and columns.
+int f64_lanes(const std::vector<ReqDesc> &reqs, int scheme)
 {
-    // A request of a pair runs on expanded groups or, where its pulse's sums say no,
-    // step by step: both launches are queued and one of them returns at once.  Its
-    // projection is a launch of its own over the state they leave.
-    std::vector<ReqDesc> reqs, after;
-    std::vector<const ReqDesc *> grouped;
-    for (const ReqDesc &r : given) {
-        reqs.push_back(r);
-        if (!r.by_groups)
+    if (scheme == DSP_SCHEME_MAGNUS4)
+        return 1;
+    struct Shape {
+        int lanes;
+        double exact, strang;
+    };
+    constexpr Shape shapes[4] = {{0, 65.0, 70.0}, {1, 18.0, 36.0}, {2, 9.0, 0.0}, {4, 6.0, 0.0}};
+    int best = 0;
+    double best_t = 0.0;
+    for (const Shape &sh : shapes) {
+        const double cost = scheme == DSP_SCHEME_EXACT ? sh.exact : sh.strang;
+        if (cost == 0.0)
             continue;
-        grouped.push_back(&r);
-        reqs.back().store_state = 1;
-        reqs.back().project = 0;
-        if (r.project) {
-            after.push_back(r);
-            ReqDesc &p = after.back();
-            p.step_begin = p.step_end;
-            p.by_groups = p.fresh = p.store_state = p.strips = 0;
-            p.n_tiles = static_cast<int32_t>((r.n_points + dsp::kTilePoints - 1) / dsp::kTilePoints);
+        int64_t warps = 0;
+        for (const ReqDesc &r : reqs)
+            warps += sh.lanes == 0 ? row_tiles(r, 4)
+                                   : (r.n_points + 32 / sh.lanes - 1) / (32 / sh.lanes);
+        const double t = launch_time(warps, cost);
+        if (sh.lanes == 0 || t < 0.98 * best_t) {
+            best = sh.lanes;
+            best_t = t;
         }
     }
-    if (!grouped.empty()) {
-        const cudaError_t e = launch_groups(grouped, stream);
-        if (e != cudaSuccess)
-            return e;
-    }
-    bool proj = !reqs.empty();
     for (const ReqDesc &r : reqs)
-        proj = proj && project_only(r);
-    std::vector<ReqDesc> split;
-    if (!proj && reqs.size() == 1)
-        split = split_last_wave(reqs[0], precision);
-    const std::vector<ReqDesc> &all = split.empty() ? reqs : split;
-    // kernel kinds: 0 contiguous tiles; 1 + 2 scheme + (strip_h == 2): row strips
-    const auto kind_of = [&](const ReqDesc &r) {
-        return proj || !r.strips ? 0 : 1 + 2 * r.scheme + (r.strip_h == 2 ? 1 : 0);
-    };
-    for (int kind = 0; kind < 7; ++kind) {
-        std::vector<const ReqDesc *> sel;
-        for (const ReqDesc &r : all)
-            if (kind_of(r) == kind)
-                sel.push_back(&r);
-        size_t i = 0;
-        while (i < sel.size()) {
-            std::unique_ptr<EvolveArgs> a(new EvolveArgs());
-            std::memset(a.get(), 0, sizeof(EvolveArgs));
-            int tiles = 0;
-            int n = 0;
-            while (i < sel.size() && n < dsp::kMaxReqPerLaunch) {
-                a->r[n] = *sel[i];
-                a->r[n].tile_begin = tiles;
-                tiles += sel[i]->n_tiles;
-                ++n;
-                ++i;
-            }
-            a->nreq = n;
-            a->total_tiles = tiles;
-            cudaError_t e;
-            if (proj)
-                e = dsp::launch_project(*a, precision, stream);
-            else if (precision == DSP_FP64)
-                e = kind == 0 ? dsp::launch_evolve_f64(*a, stream)
-                              : dsp::launch_evolve_f64_strip(*a, stream);
-            else if (kind == 0)
-                e = dsp::launch_evolve_mixed(*a, stream);
-            else
-                e = dsp::launch_evolve_strip(*a, (kind - 1) / 2, (kind - 1) % 2 ? 2 : 4, stream);
+        if (r.rows > 0)
+            best = r.rows == 4 ? 0 : 1;
+    return best;
+}
+
+// Queues the evolution of FP64 requests, one launch per scheme (and 96 requests).
+cudaError_t launch_f64(const std::vector<ReqDesc> &reqs, cudaStream_t stream)
+{
+    std::unique_ptr<EvolveArgs> a(new EvolveArgs());
+    for (int scheme = 0; scheme < 3; ++scheme) {
+        std::vector<ReqDesc> sel;
+        for (const ReqDesc &r : reqs)
+            if (r.scheme == scheme)
+                sel.push_back(r);
+        const int lanes = f64_lanes(sel, scheme);
+        for (size_t i = 0; i < sel.size();) {
+            i = fill_launch(sel, i, *a, [&](const ReqDesc &r) {
+                return lanes == 0 ? row_tiles(r, 4) : (r.n_points + 32 / lanes - 1) / (32 / lanes);
+            });
+            const cudaError_t e = dsp::launch_evolve_f64(
+                *a, lanes, warps_per_cta(a->total_tiles, dsp::kF64Warps), stream);
             if (e != cudaSuccess)
                 return e;
         }
     }
-    return after.empty() ? cudaSuccess : launch_requests(after, precision, stream);
+    return cudaSuccess;
+}
+
+// Queues the FP32_MIXED step-by-step launches: on contiguous tiles or on row strips,
+// one kernel per scheme and strip height; a launch of one grid on row strips has its
+// last wave split (split_last_wave).
+cudaError_t launch_steps_mixed(const std::vector<ReqDesc> &reqs, cudaStream_t stream)
+{
+    std::vector<ReqDesc> split;
+    if (reqs.size() == 1)
+        split = split_last_wave(reqs[0]);
+    const std::vector<ReqDesc> &all = split.empty() ? reqs : split;
+    std::unique_ptr<EvolveArgs> a(new EvolveArgs());
+    // kernel kinds: 0 contiguous tiles; 1 + 2 scheme + (strip_h == 2): row strips
+    for (int kind = 0; kind < 7; ++kind) {
+        std::vector<ReqDesc> sel;
+        for (const ReqDesc &r : all)
+            if ((r.strips ? 1 + 2 * r.scheme + (r.strip_h == 2 ? 1 : 0) : 0) == kind)
+                sel.push_back(r);
+        for (size_t i = 0; i < sel.size();) {
+            i = fill_launch(sel, i, *a, [](const ReqDesc &r) { return r.n_tiles; });
+            const cudaError_t e =
+                kind == 0 ? dsp::launch_evolve_mixed(*a, stream)
+                          : dsp::launch_evolve_strip(*a, (kind - 1) / 2, (kind - 1) % 2 ? 2 : 4,
+                                                     stream);
+            if (e != cudaSuccess)
+                return e;
+        }
+    }
+    return cudaSuccess;
+}
+
+// Queues launches advancing several requests of one precision; each request reports
+// device errors in its own error word (ReqDesc::err).  The step-by-step FP32_MIXED
+// kernels project in the same launch; the FP64 kernels and the expanded groups leave
+// the projection to a launch of its own over the state they store.  A request whose
+// groups may be evaluated expanded is queued twice: on expanded groups and step by
+// step, and the launch that its pulse's sums do not pick returns at once.
+cudaError_t launch_requests(const std::vector<ReqDesc> &given, int precision, cudaStream_t stream)
+{
+    std::vector<ReqDesc> steps, grouped, after;
+    for (const ReqDesc &r : given) {
+        if (project_only(r)) {
+            after.push_back(projection_of(r));
+            continue;
+        }
+        steps.push_back(r);
+        if (precision == DSP_FP64 || r.by_groups) {
+            steps.back().store_state = 1;
+            steps.back().project = 0;
+            if (r.by_groups)
+                grouped.push_back(steps.back());
+            if (r.project)
+                after.push_back(projection_of(r));
+        }
+    }
+    cudaError_t e = launch_groups(grouped, stream);
+    if (e == cudaSuccess)
+        e = precision == DSP_FP64 ? launch_f64(steps, stream) : launch_steps_mixed(steps, stream);
+    return e == cudaSuccess ? launch_projections(after, precision, stream) : e;
 }
 
 cudaError_t launch_finalizes(const std::vector<dsp::FinDesc> &fins, cudaStream_t stream)

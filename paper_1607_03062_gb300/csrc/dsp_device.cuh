@@ -423,7 +423,6 @@ constexpr int kGroupUnroll = DSP_GROUP_UNROLL;  // chain loop inside one group (
 constexpr int kMixedSpt = DSP_MIXED_SPT;
 constexpr int kMixedThreads = kTilePoints / kMixedSpt;
 constexpr int kMixedMinBlocks = DSP_MIXED_MINB;  // resident CTAs per SM the registers allow
-constexpr int kF64Threads = kThreads;
 static_assert(kTilePoints % kMixedSpt == 0, "a CTA owns one whole tile");
 static_assert(kMixedSpt % 2 == 0, "FP32x2 pairs of spinors");
 

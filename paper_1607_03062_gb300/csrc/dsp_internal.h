@@ -17,9 +17,6 @@ constexpr int kStripHeight = 4;
 // Points per density partial sum (a granule: point index / kGranule); every CTA
 // shape covers whole granules.
 constexpr int kGranule = 256;
-// Spinors per thread (independent momenta advanced together for ILP).
-constexpr int kSpinorsPerThread = 2;
-constexpr int kThreads = kTilePoints / kSpinorsPerThread;
 // Requests one evolve launch can carry in its parameter block (96 x 280 bytes:
 // within the 32 KB kernel-parameter limit).
 constexpr int kMaxReqPerLaunch = 96;
@@ -86,6 +83,7 @@ struct GroupEntry {
 // pulse, 0.63: 2.5e-7, 1.7e-7; 64^2 sin^2 pulse, 0.49: 9.4e-8, 5.8e-8.
 constexpr double kGroupAngleLite = 0.25, kGroupAngleWide = 0.72;
 constexpr int kGroupWarps = 4;  // most warps per CTA of the expanded-group kernel
+constexpr int kF64Warps = 4;    // most warps per CTA of the FP64 kernels
 constexpr int kNumGroupSizes = 3;
 // Group sizes 16, 8, 4 (i = 0, 1, 2).
 __host__ __device__ constexpr int group_size(int i) { return 16 >> i; }
@@ -161,7 +159,7 @@ struct ReqDesc {
                      // sec) series, one of kTanDegrees
     int32_t withhold_first_copy;  // test hook: announce chunk 0 but never copy it, so the
                                   // bounded wait for it runs out (no fault, no hang)
-    int32_t strips;  // 1: row strips (nx a multiple of kStripWidth): CTA tile b is rows
+    int32_t strips;  // FP32_MIXED, 1: row strips (nx a multiple of kStripWidth): CTA tile b is rows
                      // strip_row0 + strip_h (b / (nx / 256)) .. + strip_h - 1, columns
                      // 256 (b % (nx / 256)) .. + 255; 0: CTA tile b is points
                      // 1024 b .. 1024 b + 1023
@@ -174,7 +172,7 @@ struct ReqDesc {
     GroupTable groups;   // FP32_MIXED expanded groups (entries null: none)
     int32_t by_groups;   // 1: this launch is one of a pair, on expanded groups or step by
                          // step: the kernel that the plan does not pick does nothing
-    int32_t group_rows;  // rows per warp asked for by the tiling hook; 0: by size
+    int32_t rows;  // rows per warp asked for by the tiling hook (4, 1); 0: by size
 };
 
 // Steps are grouped (G = 16, 8, 4 or 2, the largest allowed) when G * theta_max
@@ -251,11 +249,12 @@ struct CombineArgs {
     int32_t row0;  // global row index of the grid's first row
 };
 
-// Evolve launches, one kernel per kind of request: FP64 or FP32_MIXED, on
-// contiguous tiles (strips == 0) or on row strips (strips == 1).  Every request
-// in args must be of that kind.
-cudaError_t launch_evolve_f64(const EvolveArgs &args, cudaStream_t stream);
-cudaError_t launch_evolve_f64_strip(const EvolveArgs &args, cudaStream_t stream);
+// Evolve launches, one kernel per kind of request.  FP64: `lanes` 0 tiles of 32
+// columns x 4 rows (no MAGNUS4), 1, 2 or 4 lanes per point on tiles of 32 / lanes
+// consecutive points (2, 4: EXACT only); n_tiles counts those, `warps` tiles per CTA.
+// Does not project.
+cudaError_t launch_evolve_f64(const EvolveArgs &args, int lanes, int warps, cudaStream_t stream);
+// FP32_MIXED on contiguous tiles.
 cudaError_t launch_evolve_mixed(const EvolveArgs &args, cudaStream_t stream);
 // FP32_MIXED row strips: one kernel per scheme and strip height (every request in
 // args has that scheme and strip_h).
@@ -266,9 +265,8 @@ cudaError_t launch_evolve_strip(const EvolveArgs &args, int scheme, int strip_h,
 cudaError_t launch_evolve_group(const EvolveArgs &args, int rows, int warps, cudaStream_t stream);
 // Per-step table, group entries and sums of a pulse from the caller's table.
 cudaError_t launch_prep_groups(const PrepArgs &args, cudaStream_t stream);
-// CTAs of the 4-row strip kernel of a precision (and FP32_MIXED scheme) that one
-// SM holds at once.
-cudaError_t strip_ctas_per_sm(int precision, int scheme, int *ctas);
+// CTAs of a scheme's 4-row strip kernel that one SM holds at once.
+cudaError_t strip_ctas_per_sm(int scheme, int *ctas);
 // Projection only, of states already on the device: every request in args has
 // step_begin == step_end, project == 1, fresh == 0 and a node table.
 cudaError_t launch_project(const EvolveArgs &args, int precision, cudaStream_t stream);
