@@ -194,7 +194,7 @@ __device__ __forceinline__ void strip64_step(F64Point (&pt)[H], double tx, doubl
 // MAGNUS4 flat 1.  The projection is the projection kernel's, on the state these
 // leave.
 //
-// Measured: 64^2 x 2000 steps 9.48 -> 1.29 ms (1024-point CTAs held 4 of 152 SMs;
+// Measured: 64^2 x 2000 steps 9.48 -> 1.08 ms (1024-point CTAs held 4 of 152 SMs;
 // flat 4 holds 512 warps), 300 x 257 x 1700 steps 8.10 -> 4.20 ms.
 // ---------------------------------------------------------------------------
 
@@ -292,57 +292,149 @@ __device__ __forceinline__ float shfl_x(float v, int mask)
     return __shfl_xor_sync(0xffffffffu, v, mask);
 }
 
-// sum_{k=K..D} c_k x^(k-K) in double-float as horner_df, of the cos series (odd =
-// false: c_k = (-1)^k/(2k)!, to DC) or the sinc one (odd: (-1)^k/(2k + 1)!, to DS);
-// the shorter one starts from zero coefficients, which changes nothing.
-template <int DC, int DS, int K>
-__device__ __forceinline__ void horner_either(bool odd, float xh, float xl, float &th, float &tl)
+// sum_{k=K..D} c_k x^(k-K) in double-float as horner_df, for U steps at once, of the cos
+// series (odd = false: c_k = (-1)^k/(2k)!, to DC) or the sinc one (odd: (-1)^k/(2k +
+// 1)!, to DS); the shorter one starts from zero coefficients, which changes nothing.
+template <int DC, int DS, int K, int U>
+__device__ __forceinline__ void horner_either(bool odd, const float (&xh)[U], const float (&xl)[U],
+                                              float (&th)[U], float (&tl)[U])
 {
     constexpr int D = DC > DS ? DC : DS;
     constexpr double sign = (K & 1) ? -1.0 : 1.0;
     constexpr DFConst c = df_const(K <= DC ? sign * inv_factorial<2 * K>() : 0.0);
     constexpr DFConst s = df_const(K <= DS ? sign * inv_factorial<2 * K + 1>() : 0.0);
     const float ch = odd ? s.h : c.h, cl = odd ? s.l : c.l;
-    if constexpr (K == D) {
-        th = ch;
-        tl = cl;
-    } else {
-        float uh, ul;
-        horner_either<DC, DS, K + 1>(odd, xh, xl, uh, ul);
-        df_mul(xh, xl, uh, ul, th, tl);
-        df_add(th, tl, ch, cl);
+    if constexpr (K < D)
+        horner_either<DC, DS, K + 1, U>(odd, xh, xl, th, tl);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        if constexpr (K == D) {
+            th[u] = ch;
+            tl[u] = cl;
+        } else {
+            float ph, pl;
+            df_mul(xh[u], xl[u], th[u], tl[u], ph, pl);
+            df_add(ph, pl, ch, cl);
+            th[u] = ph;
+            tl[u] = pl;
+        }
     }
 }
 
-// One EXACT step on L = 2 or 4 lanes per point (step_f64_exact's operations).  Lane k
-// of a point: P is P_x (k even) or P_y (k odd); L = 2 holds a (k = 0) or b (k = 1) in
-// v[0], v[1]; L = 4 holds Re a, Im a, Re b, Im b.
-template <int DC, int DS, int L>
-__device__ __forceinline__ void step_f64_lanes(double (&v)[4 / L], double P, int k)
+// EXACT steps on L = 2 or 4 lanes per point (step_f64_exact's operations).  Lane k of a
+// point: L = 2 holds a (k = 0) or b (k = 1) in v[0], v[1]; L = 4 holds Re a, Im a, Re b,
+// Im b.  An operator's entries as the lane applies them:
+template <int L, int U>
+struct LaneOps {
+    double m[U], sr[U], si[U];  // cos - 1; -+ Re q; +- Im q (L = 2: Im q)
+};
+
+// The operators of U steps, stage by stage for all of them (a step's own chain of
+// conversions, shuffles and double-float series takes ~900 cycles).  P: the lane's P_x
+// (k even) or P_y (k odd).
+template <int DC, int DS, int L, int U>
+__device__ __forceinline__ void lane_ops(LaneOps<L, U> &o, const double (&P)[U], int k)
 {
     const bool odd = k & 1;
-    const float2 own = square_df(P);
-    const float oh = shfl_x(own.x, 1), ol = shfl_x(own.y, 1);
-    float xh = odd ? oh : own.x, xl = odd ? ol : own.y;          // P_x^2
-    df_add(xh, xl, odd ? own.x : oh, odd ? own.y : ol);          // + P_y^2
-    float th, tl, uh, ul;
-    horner_either<DC, DS, 1>(odd, xh, xl, th, tl);
-    df_mul(xh, xl, th, tl, uh, ul);
-    const double mine = df_to_f64(uh, ul), other = shfl_x(mine, 1);
-    const double m = odd ? other : mine, s1 = odd ? mine : other;
-    const double q = fma(s1, P, P), p = shfl_x(q, 1);
-    const double qr = odd ? q : p, qi = odd ? p : q;
-    if constexpr (L == 2) {
-        const double sr = odd ? qr : -qr;
-        const double tr = shfl_x(v[0], 1), ti = shfl_x(v[1], 1);
-        const double nr = fma(m, v[0], fma(sr, tr, fma(qi, ti, v[0])));
-        const double ni = fma(m, v[1], fma(sr, ti, fma(-qi, tr, v[1])));
-        v[0] = nr;
-        v[1] = ni;
-    } else {
-        const double sr = (k & 2) ? qr : -qr, si = odd ? -qi : qi;
-        const double t1 = shfl_x(v[0], 2), t2 = shfl_x(v[0], 3);
-        v[0] = fma(m, v[0], fma(sr, t1, fma(si, t2, v[0])));
+    float2 own[U];
+    float xh[U], xl[U], th[U], tl[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+        own[u] = square_df(P[u]);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        th[u] = shfl_x(own[u].x, 1);
+        tl[u] = shfl_x(own[u].y, 1);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {  // P_x^2 + P_y^2
+        xh[u] = odd ? th[u] : own[u].x;
+        xl[u] = odd ? tl[u] : own[u].y;
+        df_add(xh[u], xl[u], odd ? own[u].x : th[u], odd ? own[u].y : tl[u]);
+    }
+    horner_either<DC, DS, 1, U>(odd, xh, xl, th, tl);
+    double mine[U], q[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        float ph, pl;
+        df_mul(xh[u], xl[u], th[u], tl[u], ph, pl);
+        mine[u] = df_to_f64(ph, pl);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const double other = shfl_x(mine[u], 1);
+        o.m[u] = odd ? other : mine[u];
+        q[u] = fma(odd ? mine[u] : other, P[u], P[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const double p = shfl_x(q[u], 1);
+        const double qr = odd ? q[u] : p, qi = odd ? p : q[u];
+        if constexpr (L == 2) {
+            o.sr[u] = odd ? qr : -qr;
+            o.si[u] = qi;
+        } else {
+            o.sr[u] = (k & 2) ? qr : -qr;
+            o.si[u] = odd ? -qi : qi;
+        }
+    }
+}
+
+template <int L, int U>
+__device__ __forceinline__ void lane_apply(double (&v)[4 / L], const LaneOps<L, U> &o)
+{
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        if constexpr (L == 2) {
+            const double tr = shfl_x(v[0], 1), ti = shfl_x(v[1], 1);
+            const double nr = fma(o.m[u], v[0], fma(o.sr[u], tr, fma(o.si[u], ti, v[0])));
+            const double ni = fma(o.m[u], v[1], fma(o.sr[u], ti, fma(-o.si[u], tr, v[1])));
+            v[0] = nr;
+            v[1] = ni;
+        } else {
+            const double t1 = shfl_x(v[0], 2), t2 = shfl_x(v[0], 3);
+            v[0] = fma(o.m[u], v[0], fma(o.sr[u], t1, fma(o.si[u], t2, v[0])));
+        }
+    }
+}
+
+// A chunk's steps: the operators of the next kLaneSteps steps are formed beside the
+// current ones' updates.  A warp waits out the issue of its own FP64 instructions, so
+// this hides shuffles and FP32 latency only, and only 4 lanes per point, which run
+// where a scheduler has one warp or two, take it (64^2 x 2000: 1.29 -> 1.08 ms); on 2
+// lanes the registers push out warps that hide more (4 steps on 256^2: 4.84 -> 5.31
+// ms).  a: the lane's component of the chunk's entries (every second double).
+template <int L>
+constexpr int kLaneSteps = L == 4 ? 4 : 1;
+template <int DC, int DS, int L>
+__device__ __forceinline__ void lane_steps(double (&v)[4 / L], const double *a, double t, int len,
+                                           int k)
+{
+    constexpr int U = kLaneSteps<L>;
+    const auto block = [&](LaneOps<L, U> &o, int j) {
+        double P[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            P[u] = t + a[2 * (j + u)];
+        lane_ops<DC, DS, L, U>(o, P, k);
+    };
+    int j = 0;
+    if (len >= U) {
+        LaneOps<L, U> cur;
+        block(cur, 0);
+        for (j = U; j + U <= len; j += U) {
+            LaneOps<L, U> next;
+            block(next, j);
+            lane_apply<L, U>(v, cur);
+            cur = next;
+        }
+        lane_apply<L, U>(v, cur);
+    }
+    for (; j < len; ++j) {
+        LaneOps<L, 1> o;
+        const double P[1] = {t + a[2 * j]};
+        lane_ops<DC, DS, L, 1>(o, P, k);
+        lane_apply<L, 1>(v, o);
     }
 }
 
@@ -394,10 +486,7 @@ __device__ void body_flat(const ReqDesc &R, int tile, F64Smem &sm, int *err)
         const double t = (k & 1) ? pt.ty : pt.tx;
         const WarpStager<double2> st(R, &sm.stage[0][0], sm.bars);
         if (!st.run(err, [&](const double2 *e, int len) {
-                const double *a = reinterpret_cast<const double *>(e) + (k & 1);
-#pragma unroll 2
-                for (int j = 0; j < len; ++j)
-                    step_f64_lanes<DC, DS, L>(v, t + a[2 * j], k);
+                lane_steps<DC, DS, L>(v, reinterpret_cast<const double *>(e) + (k & 1), t, len, k);
             }))
             return;
         if (valid) {
@@ -473,7 +562,7 @@ __device__ __forceinline__ void dispatch_f64(const ReqDesc &R, int tile, F64Smem
 }
 
 template <int L>
-__global__ void __launch_bounds__(32 * kF64Warps, L == 0 ? 4 : 5)
+__global__ void __launch_bounds__(32 * kF64Warps, L == 4 ? 2 : L == 0 ? 4 : 5)
     evolve_f64_kernel(const __grid_constant__ EvolveArgs args)
 {
     __shared__ __align__(128) F64Smem smem[kF64Warps];
