@@ -131,4 +131,24 @@ __device__ __forceinline__ void granule_sums(float2 *red, int n_gran, double *pa
     }
 }
 
+// The same tree for a granule held by one warp, lane l with its points l + 32 i in
+// v[i]: slot j plus slot j + s for s = 128, 64, 32 inside the lane, s = 16 .. 1 across
+// lanes.  The sum ends in lane 0's v[0].
+constexpr int kGranulePerLane = kGranule / 32;
+__device__ __forceinline__ void granule_tree(float2 (&v)[kGranulePerLane], int lane)
+{
+#pragma unroll
+    for (int s = kGranulePerLane / 2; s > 0; s >>= 1)
+#pragma unroll
+        for (int i = 0; i < s; ++i)
+            df_add(v[i].x, v[i].y, v[i + s].x, v[i + s].y);
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) {
+        const float h = __shfl_down_sync(0xffffffffu, v[0].x, s);
+        const float l = __shfl_down_sync(0xffffffffu, v[0].y, s);
+        if (lane < s)
+            df_add(v[0].x, v[0].y, h, l);
+    }
+}
+
 }  // namespace dsp

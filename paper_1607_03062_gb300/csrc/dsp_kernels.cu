@@ -49,7 +49,7 @@ struct ProjShape {
     static constexpr int warp_bytes = bufs * 2 * plane;  // a warp's ring
     static constexpr int smem = warps * (warp_bytes + bufs * 8);
 };
-constexpr int kProjPer = kGranule / 32;  // points per lane and granule
+constexpr int kProjPer = kGranulePerLane;  // points per lane and granule
 static_assert(kTilePoints % kGranule == 0, "tiles hold whole granules");
 
 template <int PREC>
@@ -177,19 +177,7 @@ __global__ void __launch_bounds__(ProjShape<PREC>::threads, 1)
                     }
                 }
             }
-            // granule_sums' tree: s = 128, 64, 32 within the lane, s = 16 .. 1 across lanes
-#pragma unroll
-            for (int s = kProjPer / 2; s > 0; s >>= 1)
-#pragma unroll
-                for (int i = 0; i < s; ++i)
-                    df_add(v[i].x, v[i].y, v[i + s].x, v[i + s].y);
-#pragma unroll
-            for (int s = 16; s > 0; s >>= 1) {
-                const float h = __shfl_down_sync(0xffffffffu, v[0].x, s);
-                const float l = __shfl_down_sync(0xffffffffu, v[0].y, s);
-                if (lane < s)
-                    df_add(v[0].x, v[0].y, h, l);
-            }
+            granule_tree(v, lane);
             const int64_t gi = gbase / kGranule;
             if (lane == 0 && gi < (R.n_points + kGranule - 1) / kGranule)
                 R.partials[gi] = df_to_f64(v[0].x, v[0].y);
@@ -200,20 +188,34 @@ __global__ void __launch_bounds__(ProjShape<PREC>::threads, 1)
     }
 }
 
-// One CTA per density: fixed-order per-thread sums of the granule partials,
-// then a pairwise tree.
-__global__ void __launch_bounds__(1024) finalize_kernel(const __grid_constant__ FinalizeArgs args)
+// One cluster per density: 1024 fixed-order strided sums of the granule partials (sum t
+// takes partials t, t + 1024, ...), then a pairwise tree over them.  The strided sums of
+// a large map are a chain of FP64 adds per thread (64 for 4096^2), and one CTA of 1024
+// threads puts 32 warps of them on one SM's FP64 pipe: 25 us for 65536 partials.  Spread
+// over a cluster of 8 CTAs each scheduler has one warp; the sums meet in rank 0's shared
+// memory for the tree.  The order of every addition is the one-CTA kernel's.
+constexpr int kFinSums = 1024, kFinCtas = 8, kFinThreads = kFinSums / kFinCtas;
+__global__ void __cluster_dims__(kFinCtas, 1, 1) __launch_bounds__(kFinThreads)
+    finalize_kernel(const __grid_constant__ FinalizeArgs args)
 {
-    __shared__ double red[1024];
-    const FinDesc &f = args.f[blockIdx.x];
+    __shared__ double red[kFinSums];
+    const FinDesc &f = args.f[blockIdx.x / kFinCtas];
+    const int rank = blockIdx.x % kFinCtas;
+    const int slot = rank * kFinThreads + threadIdx.x;
     double acc = 0.0;
-    for (int64_t i = threadIdx.x; i < f.n_parts; i += blockDim.x)
+#pragma unroll 8
+    for (int64_t i = slot; i < f.n_parts; i += kFinSums)
         acc += f.partials[i];
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int s = 512; s > 0; s >>= 1) {
-        if (threadIdx.x < s)
-            red[threadIdx.x] += red[threadIdx.x + s];
+    uint32_t dst;  // rank 0's red[slot]
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(dst) : "r"(smem_addr(&red[slot])));
+    asm volatile("barrier.cluster.arrive;\n\tbarrier.cluster.wait;" ::: "memory");
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(dst), "d"(acc) : "memory");
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+    if (rank != 0)
+        return;
+    for (int s = kFinSums / 2; s > 0; s >>= 1) {
+        for (int i = threadIdx.x; i < s; i += kFinThreads)
+            red[i] += red[i + s];
         __syncthreads();
     }
     if (threadIdx.x == 0)
@@ -349,7 +351,7 @@ cudaError_t launch_finalize(const FinalizeArgs &args, cudaStream_t stream)
 {
     if (args.count <= 0)
         return cudaSuccess;
-    finalize_kernel<<<args.count, 1024, 0, stream>>>(args);
+    finalize_kernel<<<args.count * kFinCtas, kFinThreads, 0, stream>>>(args);
     return cudaGetLastError();
 }
 
