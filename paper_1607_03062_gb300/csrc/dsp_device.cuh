@@ -125,6 +125,42 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
 }
 
 // ---------------------------------------------------------------------------
+// Packed FP32x2 arithmetic: lane 0 and lane 1 of every float2 belong to two
+// different momenta; each lane is rounded as the scalar FP32 operation would
+// be, so one instruction issues the arithmetic of two spinors and either lane's
+// result is the one-momentum result.  Code written for V = float2 performs the
+// same roundings for one momentum as V = float (non-contracting intrinsics).
+// ---------------------------------------------------------------------------
+
+__device__ __forceinline__ float2 bc2(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 neg2(float2 v) { return make_float2(-v.x, -v.y); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, neg2(b)); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
+[[maybe_unused]] __device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
+[[maybe_unused]] __device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+[[maybe_unused]] __device__ __forceinline__ float vfma(float a, float b, float c)
+{
+    return __fmaf_rn(a, b, c);
+}
+[[maybe_unused]] __device__ __forceinline__ float vneg(float a) { return -a; }
+[[maybe_unused]] __device__ __forceinline__ float2 vadd(float2 a, float2 b) { return add2(a, b); }
+[[maybe_unused]] __device__ __forceinline__ float2 vmul(float2 a, float2 b) { return mul2(a, b); }
+[[maybe_unused]] __device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c)
+{
+    return fma2(a, b, c);
+}
+[[maybe_unused]] __device__ __forceinline__ float2 vneg(float2 a) { return neg2(a); }
+template <typename V>
+__device__ __forceinline__ V vbc(float v);
+template <>
+[[maybe_unused]] __device__ __forceinline__ float vbc<float>(float v) { return v; }
+template <>
+[[maybe_unused]] __device__ __forceinline__ float2 vbc<float2>(float v) { return bc2(v); }
+
+// ---------------------------------------------------------------------------
 // Taylor series in x = theta^2 (written from the power series of cos and sin)
 //   cos(theta) - 1    = sum_{k>=1} (-x)^k / (2k)!
 //   sin(theta)/theta  = sum_{k>=0} (-x)^k / (2k+1)!
@@ -225,76 +261,89 @@ __device__ __forceinline__ double project_point(double Px, double Py, double sgn
 // form: their squares would lose bits near the bottom of the float range.
 constexpr float kProjTinyE2 = 0x1p-90f;
 
+// V = float: one point; float2: two, each lane with the same operations.
+template <typename V>
+__device__ __forceinline__ void vtwo_sum(V a, V b, V &s, V &e)
+{
+    s = vadd(a, b);
+    const V bb = vadd(s, vneg(a));
+    e = vadd(vadd(a, vneg(vadd(s, vneg(bb)))), vadd(b, vneg(bb)));
+}
+__device__ __forceinline__ float vrsqrt(float x) { return rsqrtf(x); }
+__device__ __forceinline__ float2 vrsqrt(float2 x) { return make_float2(rsqrtf(x.x), rsqrtf(x.y)); }
+__device__ __forceinline__ bool at_least(float x, float lim) { return x >= lim; }
+__device__ __forceinline__ bool at_least(float2 x, float lim) { return x.x >= lim && x.y >= lim; }
+
 // |c+|^2 = oh + ol for the node s P_out = (xh + xl, yh + yl) (s = valley) and
 // the spinor a = (ar, ai), b = (br, bi), each component hi + lo:
 //   c+ = (a + conj(w) b)/sqrt(2),  w = s (P_x + i P_y)/|P|,
 //   cr = ar + wr br + wi bi,  ci = ai + wr bi - wi br.
-// Returns false (and leaves oh, ol unset) when E^2 < kProjTinyE2.
-__device__ __forceinline__ bool project_df(float xh, float xl, float yh, float yl, float arh,
-                                           float arl, float aih, float ail, float brh, float brl,
-                                           float bih, float bil, float &oh, float &ol)
+// Returns false (oh, ol then mean nothing) when E^2 < kProjTinyE2 (V = float2: of
+// either point).
+template <typename V>
+__device__ __forceinline__ bool project_df(V xh, V xl, V yh, V yl, V arh, V arl, V aih, V ail,
+                                           V brh, V brl, V bih, V bil, V &oh, V &ol)
 {
     // E^2 = Px^2 + Py^2 to ~2^-46
-    const float x2 = __fmul_rn(xh, xh);
-    const float x2e = __fmaf_rn(__fadd_rn(xh, xh), xl, __fmaf_rn(xh, xh, -x2));
-    const float y2 = __fmul_rn(yh, yh);
-    const float y2e = __fmaf_rn(__fadd_rn(yh, yh), yl, __fmaf_rn(yh, yh, -y2));
-    float sh, se;
-    two_sum(x2, y2, sh, se);
-    se = __fadd_rn(se, __fadd_rn(x2e, y2e));
-    if (!(sh >= kProjTinyE2))
-        return false;
+    const V x2 = vmul(xh, xh);
+    const V x2e = vfma(vadd(xh, xh), xl, vfma(xh, xh, vneg(x2)));
+    const V y2 = vmul(yh, yh);
+    const V y2e = vfma(vadd(yh, yh), yl, vfma(yh, yh, vneg(y2)));
+    V sh, se;
+    vtwo_sum(x2, y2, sh, se);
+    se = vadd(se, vadd(x2e, y2e));
     // r = 1/E = r0 + rc: one Newton step r0 (1 - t/2) from the FP32 estimate r0,
     // with t = E^2 r0^2 - 1 evaluated to ~2^-46 (p - 1 is exact: p is near 1)
-    const float r0 = rsqrtf(sh);
-    const float q = __fmul_rn(r0, r0), qe = __fmaf_rn(r0, r0, -q);
-    const float p = __fmul_rn(sh, q), pe = __fmaf_rn(sh, q, -p);
-    const float t = __fadd_rn(__fadd_rn(p, -1.0f), __fmaf_rn(sh, qe, __fmaf_rn(se, q, pe)));
-    const float rc = __fmul_rn(__fmul_rn(-0.5f, r0), t);
+    const V r0 = vrsqrt(sh);
+    const V q = vmul(r0, r0), qe = vfma(r0, r0, vneg(q));
+    const V p = vmul(sh, q), pe = vfma(sh, q, vneg(p));
+    const V t = vadd(vadd(p, vbc<V>(-1.0f)), vfma(sh, qe, vfma(se, q, pe)));
+    const V rc = vmul(vmul(vbc<V>(-0.5f), r0), t);
     // w = (wr + wre) + i (wi + wie) = s P / E
-    const float wr = __fmul_rn(xh, r0);
-    const float wre = __fmaf_rn(xh, rc, __fmaf_rn(xl, r0, __fmaf_rn(xh, r0, -wr)));
-    const float wi = __fmul_rn(yh, r0);
-    const float wie = __fmaf_rn(yh, rc, __fmaf_rn(yl, r0, __fmaf_rn(yh, r0, -wi)));
+    const V wr = vmul(xh, r0);
+    const V wre = vfma(xh, rc, vfma(xl, r0, vfma(xh, r0, vneg(wr))));
+    const V wi = vmul(yh, r0);
+    const V wie = vfma(yh, rc, vfma(yl, r0, vfma(yh, r0, vneg(wi))));
     // cr: the three large terms ar, wr br, wi bi exactly (split products, TwoSum),
     // then the small ones (lo parts, product errors, cross terms) in FP32
-    float crh, crl;
+    V crh, crl;
     {
-        const float p1 = __fmul_rn(wr, brh), e1 = __fmaf_rn(wr, brh, -p1);
-        const float p2 = __fmul_rn(wi, bih), e2 = __fmaf_rn(wi, bih, -p2);
-        float t1, te, ce;
-        two_sum(p1, p2, t1, te);
-        two_sum(arh, t1, crh, ce);
-        float l = __fadd_rn(__fadd_rn(ce, te), __fadd_rn(arl, __fadd_rn(e1, e2)));
-        l = __fmaf_rn(wre, brh, __fmaf_rn(wr, brl, l));
-        crl = __fmaf_rn(wie, bih, __fmaf_rn(wi, bil, l));
+        const V p1 = vmul(wr, brh), e1 = vfma(wr, brh, vneg(p1));
+        const V p2 = vmul(wi, bih), e2 = vfma(wi, bih, vneg(p2));
+        V t1, te, ce;
+        vtwo_sum(p1, p2, t1, te);
+        vtwo_sum(arh, t1, crh, ce);
+        V l = vadd(vadd(ce, te), vadd(arl, vadd(e1, e2)));
+        l = vfma(wre, brh, vfma(wr, brl, l));
+        crl = vfma(wie, bih, vfma(wi, bil, l));
     }
-    float cih, cil;
+    V cih, cil;
     {
-        const float p3 = __fmul_rn(wr, bih), e3 = __fmaf_rn(wr, bih, -p3);
-        const float p4 = __fmul_rn(-wi, brh), e4 = __fmaf_rn(-wi, brh, -p4);
-        float t2, te, ce;
-        two_sum(p3, p4, t2, te);
-        two_sum(aih, t2, cih, ce);
-        float l = __fadd_rn(__fadd_rn(ce, te), __fadd_rn(ail, __fadd_rn(e3, e4)));
-        l = __fmaf_rn(wre, bih, __fmaf_rn(wr, bil, l));
-        cil = __fmaf_rn(-wie, brh, __fmaf_rn(-wi, brl, l));
+        const V nwi = vneg(wi);
+        const V p3 = vmul(wr, bih), e3 = vfma(wr, bih, vneg(p3));
+        const V p4 = vmul(nwi, brh), e4 = vfma(nwi, brh, vneg(p4));
+        V t2, te, ce;
+        vtwo_sum(p3, p4, t2, te);
+        vtwo_sum(aih, t2, cih, ce);
+        V l = vadd(vadd(ce, te), vadd(ail, vadd(e3, e4)));
+        l = vfma(wre, bih, vfma(wr, bil, l));
+        cil = vfma(vneg(wie), brh, vfma(nwi, brl, l));
     }
     // |c|^2 = cr^2 + ci^2 after renormalising each pair (cancellation can leave
     // the lo part as large as the hi part)
-    float ch, cl, dh, dl;
-    two_sum(crh, crl, ch, cl);
-    two_sum(cih, cil, dh, dl);
-    const float c2 = __fmul_rn(ch, ch);
-    const float c2e = __fmaf_rn(__fadd_rn(ch, ch), cl, __fmaf_rn(ch, ch, -c2));
-    const float d2 = __fmul_rn(dh, dh);
-    const float d2e = __fmaf_rn(__fadd_rn(dh, dh), dl, __fmaf_rn(dh, dh, -d2));
-    float nh, ne;
-    two_sum(c2, d2, nh, ne);
-    ne = __fadd_rn(ne, __fadd_rn(c2e, d2e));
-    oh = __fmul_rn(0.5f, nh);  // exact scalings
-    ol = __fmul_rn(0.5f, ne);
-    return true;
+    V ch, cl, dh, dl;
+    vtwo_sum(crh, crl, ch, cl);
+    vtwo_sum(cih, cil, dh, dl);
+    const V c2 = vmul(ch, ch);
+    const V c2e = vfma(vadd(ch, ch), cl, vfma(ch, ch, vneg(c2)));
+    const V d2 = vmul(dh, dh);
+    const V d2e = vfma(vadd(dh, dh), dl, vfma(dh, dh, vneg(d2)));
+    V nh, ne;
+    vtwo_sum(c2, d2, nh, ne);
+    ne = vadd(ne, vadd(c2e, d2e));
+    oh = vmul(vbc<V>(0.5f), nh);  // exact scalings
+    ol = vmul(vbc<V>(0.5f), ne);
+    return at_least(sh, kProjTinyE2);
 }
 
 // |c+|^2 in FP32 (FP32_MIXED, whose map is a float): from the hi parts of the
@@ -657,18 +706,8 @@ struct MixedPoint {
 };
 
 // ---------------------------------------------------------------------------
-// Packed FP32x2 steps: lane 0 and lane 1 of every float2 belong to two
-// different momenta; each lane is rounded as the scalar FP32 operation would
-// be, so one instruction issues the arithmetic of two spinors and either lane's
-// result is the one-momentum result.
+// Packed FP32x2 steps
 // ---------------------------------------------------------------------------
-
-__device__ __forceinline__ float2 bc2(float v) { return make_float2(v, v); }
-__device__ __forceinline__ float2 neg2(float2 v) { return make_float2(-v.x, -v.y); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, neg2(b)); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
 template <int D, int K, int ODD>
 __device__ __forceinline__ float2 horner2(float2 x)
@@ -773,31 +812,8 @@ __device__ __forceinline__ void step_magnus2(MixedPack &p, const float4 &e)
 }
 
 // ---------------------------------------------------------------------------
-// Step groups, written for V = float2 (two momenta per instruction; a V = float
-// instantiation performs the same roundings for one) with non-contracting
-// intrinsics.
+// Step groups
 // ---------------------------------------------------------------------------
-
-[[maybe_unused]] __device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
-[[maybe_unused]] __device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
-[[maybe_unused]] __device__ __forceinline__ float vfma(float a, float b, float c)
-{
-    return __fmaf_rn(a, b, c);
-}
-[[maybe_unused]] __device__ __forceinline__ float vneg(float a) { return -a; }
-[[maybe_unused]] __device__ __forceinline__ float2 vadd(float2 a, float2 b) { return add2(a, b); }
-[[maybe_unused]] __device__ __forceinline__ float2 vmul(float2 a, float2 b) { return mul2(a, b); }
-[[maybe_unused]] __device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c)
-{
-    return fma2(a, b, c);
-}
-[[maybe_unused]] __device__ __forceinline__ float2 vneg(float2 a) { return neg2(a); }
-template <typename V>
-__device__ __forceinline__ V vbc(float v);
-template <>
-[[maybe_unused]] __device__ __forceinline__ float vbc<float>(float v) { return v; }
-template <>
-[[maybe_unused]] __device__ __forceinline__ float2 vbc<float2>(float v) { return bc2(v); }
 
 template <typename V, int D, int K, int ODD>
 __device__ __forceinline__ V vhorner(V x)

@@ -65,6 +65,42 @@ __device__ __forceinline__ double f32_to_f64(float f)
     return __longlong_as_double(static_cast<long long>(d));
 }
 
+// split_f64 for 2^-74 <= |x| < 2^128 (in_split_range): the same hi and lo in half the
+// instructions, with no case to select.
+__device__ __forceinline__ bool in_split_range(double x)
+{
+    const unsigned int e =
+        static_cast<unsigned int>(static_cast<unsigned long long>(__double_as_longlong(x)) >> 32)
+        << 1;
+    return e - (949u << 21) < ((1151u - 949u) << 21);
+}
+__device__ __forceinline__ void split_f64_normal(double x, float &hi, float &lo)
+{
+    const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x));
+    const unsigned int top = static_cast<unsigned int>(b >> 32);
+    const unsigned int low = static_cast<unsigned int>(b);
+    // exponent e - 896 and the fraction's first 23 bits, then the sign
+    const unsigned int m = __funnelshift_l(low, top, 3) - (896u << 23);
+    const unsigned int h = (m & 0x7FFFFFFFu) | (top & 0x80000000u);
+    hi = __uint_as_float(h);
+    lo = __fmul_rn(__uint2float_rn(low & 0x1FFFFFFFu),
+                   __uint_as_float((h & 0xFF800000u) - (52u << 23)));  // +-2^(e - 1075)
+}
+
+// f32_to_f64 for a normal float (in_float_range).
+__device__ __forceinline__ bool in_float_range(float f)
+{
+    const unsigned int e = __float_as_uint(f) << 1;
+    return e - (1u << 24) < (254u << 24);
+}
+__device__ __forceinline__ double normal_to_f64(float f)
+{
+    const unsigned int u = __float_as_uint(f);
+    return __hiloint2double(
+        static_cast<int>((((u & 0x7FFFFFFFu) >> 3) + (896u << 20)) | (u & 0x80000000u)),
+        static_cast<int>(u << 29));
+}
+
 // hi + lo rounded to a double (one FP64 add).
 __device__ __forceinline__ double df_to_f64(float hi, float lo)
 {

@@ -52,6 +52,79 @@ struct ProjShape {
 constexpr int kProjPer = kGranulePerLane;  // points per lane and granule
 static_assert(kTilePoints % kGranule == 0, "tiles hold whole granules");
 
+// The state of a staged granule's point l, as hi/lo pairs.
+template <int PREC>
+__device__ __forceinline__ SpinorDF granule_spinor(const unsigned char *src, int l)
+{
+    constexpr int kPlane = ProjShape<PREC>::plane;
+    SpinorDF d;
+    if constexpr (PREC == 1) {  // hi plane, lo plane
+        const float4 u = reinterpret_cast<const float4 *>(src)[l];
+        const float4 q = reinterpret_cast<const float4 *>(src + kPlane)[l];
+        d = SpinorDF{u.x, q.x, u.y, q.y, u.z, q.z, u.w, q.w};
+    } else {  // a plane, b plane
+        const double2 u = reinterpret_cast<const double2 *>(src)[l];
+        const double2 q = reinterpret_cast<const double2 *>(src + kPlane)[l];
+        split_f64(u.x, d.arh, d.arl);
+        split_f64(u.y, d.aih, d.ail);
+        split_f64(q.x, d.brh, d.brl);
+        split_f64(q.y, d.bih, d.bil);
+    }
+    return d;
+}
+
+// FP64: the points l and l + 32 of a granule inside one row together, in packed FP32x2
+// (project_df on float2: the same operations per point).  Where every lane's values
+// are in the ordinary range the conversions take their short forms too; one vote per
+// pair keeps the warp together (a branch per lane was slower than the long forms).
+// Issue-bound before: 351 instructions a point, a third of them conversions; 4096^2
+// state 206 -> 153 us, the same bits.
+__device__ __forceinline__ void project_pair(const ReqDesc &R, const unsigned char *src,
+                                             int64_t gbase, int64_t col0, int64_t row, int l,
+                                             float2 cx0, float2 cx1, float2 cy, float2 &v0,
+                                             float2 &v1)
+{
+    constexpr unsigned int kAll = 0xffffffffu;
+    const double2 *a = reinterpret_cast<const double2 *>(src);
+    const double2 *b = reinterpret_cast<const double2 *>(src + ProjShape<0>::plane);
+    const double2 a0 = a[l], a1 = a[l + 32], b0 = b[l], b1 = b[l + 32];
+    bool ok = in_split_range(a0.x) && in_split_range(a0.y) && in_split_range(b0.x) &&
+              in_split_range(b0.y) && in_split_range(a1.x) && in_split_range(a1.y) &&
+              in_split_range(b1.x) && in_split_range(b1.y);
+    if (__all_sync(kAll, ok)) {
+        float2 arh, arl, aih, ail, brh, brl, bih, bil, oh, ol;
+        split_f64_normal(a0.x, arh.x, arl.x);
+        split_f64_normal(a1.x, arh.y, arl.y);
+        split_f64_normal(a0.y, aih.x, ail.x);
+        split_f64_normal(a1.y, aih.y, ail.y);
+        split_f64_normal(b0.x, brh.x, brl.x);
+        split_f64_normal(b1.x, brh.y, brl.y);
+        split_f64_normal(b0.y, bih.x, bil.x);
+        split_f64_normal(b1.y, bih.y, bil.y);
+        ok = project_df(make_float2(cx0.x, cx1.x), make_float2(cx0.y, cx1.y), bc2(cy.x), bc2(cy.y),
+                        arh, arl, aih, ail, brh, brl, bih, bil, oh, ol);
+        ok = ok && in_float_range(oh.x) && in_float_range(oh.y) && in_float_range(ol.x) &&
+             in_float_range(ol.y);
+        const double d0 = __dadd_rn(normal_to_f64(oh.x), normal_to_f64(ol.x));
+        const double d1 = __dadd_rn(normal_to_f64(oh.y), normal_to_f64(ol.y));
+        ok = ok && in_split_range(d0) && in_split_range(d1);
+        if (__all_sync(kAll, ok)) {
+            if (R.map) {
+                static_cast<double *>(R.map)[gbase + l] = d0;
+                static_cast<double *>(R.map)[gbase + l + 32] = d1;
+            }
+            split_f64_normal(d0, v0.x, v0.y);
+            split_f64_normal(d1, v1.x, v1.y);
+            return;
+        }
+    }
+    v0 = store_point<0>(R.map, gbase + l,
+                        project_node_at<0>(R, cx0, cy, col0 + l, row, granule_spinor<0>(src, l)));
+    v1 = store_point<0>(
+        R.map, gbase + l + 32,
+        project_node_at<0>(R, cx1, cy, col0 + l + 32, row, granule_spinor<0>(src, l + 32)));
+}
+
 template <int PREC>
 __global__ void __launch_bounds__(ProjShape<PREC>::threads, 1)
     project_kernel(const __grid_constant__ EvolveArgs args)
@@ -65,7 +138,8 @@ __global__ void __launch_bounds__(ProjShape<PREC>::threads, 1)
     uint64_t *bars = reinterpret_cast<uint64_t *>(proj_dyn + Sh::warps * Sh::warp_bytes) + NB * w;
     constexpr int kGranPerTile = kTilePoints / kGranule;
     const int total = args.total_tiles * kGranPerTile;  // granules of the launch
-    const int wid = blockIdx.x * Sh::warps + w, nw = gridDim.x * Sh::warps;
+    // granules go to the CTAs in turn, so that a small grid's spread over the SMs
+    const int wid = w * gridDim.x + blockIdx.x, nw = gridDim.x * Sh::warps;
     if (lane == 0) {
         for (int b = 0; b < NB; ++b)
             mbar_init(&bars[b], 1);
@@ -123,23 +197,7 @@ __global__ void __launch_bounds__(ProjShape<PREC>::threads, 1)
             col0 = __shfl_sync(0xffffffffu, col0, 0);
             row0 = __shfl_sync(0xffffffffu, row0, 0);
             const unsigned char *src = buf + b * 2 * kProjPlane;
-            // the state of the lane's point l = lane + 32 i, as hi/lo pairs
-            const auto spinor = [&](int l) {
-                SpinorDF d;
-                if constexpr (PREC == 1) {  // hi plane, lo plane
-                    const float4 u = reinterpret_cast<const float4 *>(src)[l];
-                    const float4 q = reinterpret_cast<const float4 *>(src + kProjPlane)[l];
-                    d = SpinorDF{u.x, q.x, u.y, q.y, u.z, q.z, u.w, q.w};
-                } else {  // a plane, b plane
-                    const double2 u = reinterpret_cast<const double2 *>(src)[l];
-                    const double2 q = reinterpret_cast<const double2 *>(src + kProjPlane)[l];
-                    split_f64(u.x, d.arh, d.arl);
-                    split_f64(u.y, d.aih, d.ail);
-                    split_f64(q.x, d.brh, d.brl);
-                    split_f64(q.y, d.bih, d.bil);
-                }
-                return d;
-            };
+            const auto spinor = [&](int l) { return granule_spinor<PREC>(src, l); };
             float2 v[kProjPer];
             if (gbase + kGranule <= R.n_points && col0 + kGranule <= R.nx) {
                 // a whole granule inside one row (every grid whose nx is a multiple of 256):
@@ -149,12 +207,19 @@ __global__ void __launch_bounds__(ProjShape<PREC>::threads, 1)
 #pragma unroll
                 for (int i = 0; i < kProjPer; ++i)
                     cx[i] = R.nodes_out[col0 + lane + 32 * i];
+                if constexpr (PREC == 0) {
 #pragma unroll
-                for (int i = 0; i < kProjPer; ++i) {
-                    const int l = lane + 32 * i;
-                    v[i] = store_point<PREC>(
-                        R.map, gbase + l,
-                        project_node_at<PREC>(R, cx[i], cy, col0 + l, row0, spinor(l)));
+                    for (int i = 0; i < kProjPer; i += 2)
+                        project_pair(R, src, gbase, col0, row0, lane + 32 * i, cx[i], cx[i + 1],
+                                     cy, v[i], v[i + 1]);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < kProjPer; ++i) {
+                        const int l = lane + 32 * i;
+                        v[i] = store_point<PREC>(
+                            R.map, gbase + l,
+                            project_node_at<PREC>(R, cx[i], cy, col0 + l, row0, spinor(l)));
+                    }
                 }
             } else {
                 int64_t col = col0 + lane, row = row0;
@@ -335,11 +400,9 @@ cudaError_t launch_project(const EvolveArgs &args, int precision, cudaStream_t s
                                  ProjShape<0>::smem);
     if (e != cudaSuccess)
         return e;
-    // one CTA per SM, no more warps than granules
+    // one CTA per SM, no more CTAs than granules
     const int granules = args.total_tiles * (kTilePoints / kGranule);
-    const int warps = precision == 1 ? ProjShape<1>::warps : ProjShape<0>::warps;
-    const int need = (granules + warps - 1) / warps;
-    const int grid = need < sms ? need : sms;
+    const int grid = granules < sms ? granules : sms;
     if (precision == 1)
         project_kernel<1><<<grid, ProjShape<1>::threads, ProjShape<1>::smem, stream>>>(args);
     else
