@@ -1230,14 +1230,17 @@ dsp_status dsp_solve_segmented(dsp_grid *g, int32_t segments, void *map_dev, dou
         return dsp_solve(g, map_dev, n_host);
     int64_t S = segments;
     if (S == 0) {
-        // FP64 evolution is bound by the FP64 pipe: one segment-tile per SM.  FP32_MIXED
-        // segments are short and latency bound, and the FP64 combine grows with S: one
-        // segment-tile per two SMs.  At least 16 steps a segment.  (Measured on the 64^2
-        // x 2000-step case, 4 tiles: S = 38 / 19 beat S = 76 by 8% / 40%.)
-        const int sms = sm_count();
-        const int64_t ctas = g->precision == DSP_FP64 ? sms : (sms + 1) / 2;
-        S = (ctas + g->n_tiles - 1) / g->n_tiles;
-        S = std::min<int64_t>(S, g->n_steps / 16);
+        // A segment has one warp per 32 points.  FP32_MIXED: one warp per scheduler, each
+        // with a short run left and few columns to combine (64^2 x 2000 steps: 62 us with
+        // 2 to 5 segments, 74 with 1, 77 with 16, launches included).  FP64: 16, so that the
+        // fullest scheduler is close to the average, in segments of 48 steps and more
+        // (64^2 x 2000: 343 us with 38, 401 with 6, 464 with 5; 128^2 x 20000: 9.0 ms with 19,
+        // 12.4 with 5).
+        const int64_t warps = (g->n_points + 31) / 32;
+        const bool f64 = g->precision == DSP_FP64;
+        const int64_t want = (f64 ? 64 : 4) * static_cast<int64_t>(sm_count());
+        S = (want + warps - 1) / warps;
+        S = std::min<int64_t>(S, g->n_steps / (f64 ? 48 : 16));
     }
     S = std::max<int64_t>(1, std::min<int64_t>(S, g->n_steps));
     const size_t slab = 32 * static_cast<size_t>(g->n_points);
@@ -1272,8 +1275,12 @@ dsp_status dsp_solve_segmented(dsp_grid *g, int32_t segments, void *map_dev, dou
     std::vector<ReqDesc> descs;
     descs.reserve(static_cast<size_t>(S));
     for (int64_t k = 0; k < S; ++k) {
-        const int64_t b = k * g->n_steps / S, e_ = (k + 1) * g->n_steps / S;
-        ReqDesc d = make_desc(g, b, e_, false, nullptr);
+        // long segments start on whole step groups
+        const auto start = [&](int64_t i) {
+            const int64_t n = i * g->n_steps / S;
+            return i < S && g->n_steps / S >= 2 * dsp::kGroupMax ? n - n % dsp::kGroupMax : n;
+        };
+        ReqDesc d = make_desc(g, start(k), start(k + 1), false, nullptr);
         d.state = static_cast<unsigned char *>(g->seg_buf) + static_cast<size_t>(k) * slab;
         d.fresh = 1;
         d.init_identity = 1;

@@ -73,24 +73,36 @@ __device__ __forceinline__ SpinorDF granule_spinor(const unsigned char *src, int
     return d;
 }
 
-// FP64: the points l and l + 32 of a granule inside one row together, in packed FP32x2
-// (project_df on float2: the same operations per point).  Where every lane's values
-// are in the ordinary range the conversions take their short forms too; one vote per
-// pair keeps the warp together (a branch per lane was slower than the long forms).
-// Issue-bound before: 351 instructions a point, a third of them conversions; 4096^2
-// state 206 -> 153 us, the same bits.
-__device__ __forceinline__ void project_pair(const ReqDesc &R, const unsigned char *src,
-                                             int64_t gbase, int64_t col0, int64_t row, int l,
-                                             float2 cx0, float2 cx1, float2 cy, float2 &v0,
+// A point of the grid that a lane projects, and its nodes.
+struct ProjPoint {
+    int64_t idx;      // -1: none (past the grid's end)
+    int64_t col, row;
+    float2 cx, cy;
+};
+
+// FP64: the points l and l + 32 of a granule together, in packed FP32x2 (project_df on
+// float2: the same operations per point).  Where every lane's values are in the
+// ordinary range the conversions take their short forms too; one vote per pair keeps
+// the warp together (a branch per lane was slower than the long forms).  Issue-bound
+// before: 351 instructions a point, a third of them conversions; 4096^2 state 206 ->
+// 153 us, the same bits.
+// ALL: both points exist.
+template <bool ALL>
+__device__ __forceinline__ void project_pair(const ReqDesc &R, const unsigned char *src, int l,
+                                             const ProjPoint &p0, const ProjPoint &p1, float2 &v0,
                                              float2 &v1)
 {
+    const bool in0 = ALL || p0.idx >= 0, in1 = ALL || p1.idx >= 0;
     constexpr unsigned int kAll = 0xffffffffu;
     const double2 *a = reinterpret_cast<const double2 *>(src);
     const double2 *b = reinterpret_cast<const double2 *>(src + ProjShape<0>::plane);
-    const double2 a0 = a[l], a1 = a[l + 32], b0 = b[l], b1 = b[l + 32];
+    const double2 one = make_double2(1.0, 1.0);
+    const double2 a0 = in0 ? a[l] : one, b0 = in0 ? b[l] : one;
+    const double2 a1 = in1 ? a[l + 32] : one, b1 = in1 ? b[l + 32] : one;
     bool ok = in_split_range(a0.x) && in_split_range(a0.y) && in_split_range(b0.x) &&
               in_split_range(b0.y) && in_split_range(a1.x) && in_split_range(a1.y) &&
               in_split_range(b1.x) && in_split_range(b1.y);
+    v0 = v1 = make_float2(0.0f, 0.0f);
     if (__all_sync(kAll, ok)) {
         float2 arh, arl, aih, ail, brh, brl, bih, bil, oh, ol;
         split_f64_normal(a0.x, arh.x, arl.x);
@@ -101,28 +113,37 @@ __device__ __forceinline__ void project_pair(const ReqDesc &R, const unsigned ch
         split_f64_normal(b1.x, brh.y, brl.y);
         split_f64_normal(b0.y, bih.x, bil.x);
         split_f64_normal(b1.y, bih.y, bil.y);
-        ok = project_df(make_float2(cx0.x, cx1.x), make_float2(cx0.y, cx1.y), bc2(cy.x), bc2(cy.y),
-                        arh, arl, aih, ail, brh, brl, bih, bil, oh, ol);
+        ok = project_df(make_float2(p0.cx.x, p1.cx.x), make_float2(p0.cx.y, p1.cx.y),
+                        make_float2(p0.cy.x, p1.cy.x), make_float2(p0.cy.y, p1.cy.y), arh, arl,
+                        aih, ail, brh, brl, bih, bil, oh, ol);
         ok = ok && in_float_range(oh.x) && in_float_range(oh.y) && in_float_range(ol.x) &&
              in_float_range(ol.y);
         const double d0 = __dadd_rn(normal_to_f64(oh.x), normal_to_f64(ol.x));
         const double d1 = __dadd_rn(normal_to_f64(oh.y), normal_to_f64(ol.y));
         ok = ok && in_split_range(d0) && in_split_range(d1);
         if (__all_sync(kAll, ok)) {
-            if (R.map) {
-                static_cast<double *>(R.map)[gbase + l] = d0;
-                static_cast<double *>(R.map)[gbase + l + 32] = d1;
+            double *map = static_cast<double *>(R.map);
+            if (in0) {
+                if (map)
+                    map[p0.idx] = d0;
+                split_f64_normal(d0, v0.x, v0.y);
             }
-            split_f64_normal(d0, v0.x, v0.y);
-            split_f64_normal(d1, v1.x, v1.y);
+            if (in1) {
+                if (map)
+                    map[p1.idx] = d1;
+                split_f64_normal(d1, v1.x, v1.y);
+            }
             return;
         }
     }
-    v0 = store_point<0>(R.map, gbase + l,
-                        project_node_at<0>(R, cx0, cy, col0 + l, row, granule_spinor<0>(src, l)));
-    v1 = store_point<0>(
-        R.map, gbase + l + 32,
-        project_node_at<0>(R, cx1, cy, col0 + l + 32, row, granule_spinor<0>(src, l + 32)));
+    if (in0)
+        v0 = store_point<0>(R.map, p0.idx,
+                            project_node_at<0>(R, p0.cx, p0.cy, p0.col, p0.row,
+                                               granule_spinor<0>(src, l)));
+    if (in1)
+        v1 = store_point<0>(R.map, p1.idx,
+                            project_node_at<0>(R, p1.cx, p1.cy, p1.col, p1.row,
+                                               granule_spinor<0>(src, l + 32)));
 }
 
 template <int PREC>
@@ -207,38 +228,54 @@ __global__ void __launch_bounds__(ProjShape<PREC>::threads, 1)
 #pragma unroll
                 for (int i = 0; i < kProjPer; ++i)
                     cx[i] = R.nodes_out[col0 + lane + 32 * i];
-                if constexpr (PREC == 0) {
 #pragma unroll
-                    for (int i = 0; i < kProjPer; i += 2)
-                        project_pair(R, src, gbase, col0, row0, lane + 32 * i, cx[i], cx[i + 1],
-                                     cy, v[i], v[i + 1]);
-                } else {
-#pragma unroll
-                    for (int i = 0; i < kProjPer; ++i) {
-                        const int l = lane + 32 * i;
+                for (int i = 0; i < kProjPer; i += PREC == 0 ? 2 : 1) {
+                    const int l = lane + 32 * i;
+                    if constexpr (PREC == 0)
+                        project_pair<true>(R, src, l, ProjPoint{gbase + l, col0 + l, row0, cx[i], cy},
+                                           ProjPoint{gbase + l + 32, col0 + l + 32, row0,
+                                                     cx[i + 1], cy},
+                                           v[i], v[i + 1]);
+                    else
                         v[i] = store_point<PREC>(
                             R.map, gbase + l,
                             project_node_at<PREC>(R, cx[i], cy, col0 + l, row0, spinor(l)));
-                    }
                 }
             } else {
                 int64_t col = col0 + lane, row = row0;
-                while (col >= R.nx) {
-                    col -= R.nx;
-                    ++row;
-                }
-#pragma unroll
-                for (int i = 0; i < kProjPer; ++i) {
-                    const int l = lane + 32 * i;
-                    const int64_t idx = gbase + l;
-                    v[i] = make_float2(0.0f, 0.0f);
-                    if (idx < R.n_points)
-                        v[i] = store_point<PREC>(R.map, idx,
-                                                 project_node<PREC>(R, col, row, spinor(l)));
-                    col += 32;
+                const auto wrap = [&] {
                     while (col >= R.nx) {
                         col -= R.nx;
                         ++row;
+                    }
+                };
+                wrap();
+                // point i of the lane; called in order
+                const auto next_point = [&](int i) {
+                    const int64_t idx = gbase + lane + 32 * i;
+                    ProjPoint p{-1, col, row, make_float2(1.0f, 0.0f), make_float2(1.0f, 0.0f)};
+                    if (idx < R.n_points) {
+                        p.idx = idx;
+                        p.cx = R.nodes_out[col];
+                        p.cy = R.nodes_out[R.nx + row];
+                    }
+                    col += 32;
+                    wrap();
+                    return p;
+                };
+#pragma unroll
+                for (int i = 0; i < kProjPer; i += PREC == 0 ? 2 : 1) {
+                    const int l = lane + 32 * i;
+                    const ProjPoint p = next_point(i);
+                    if constexpr (PREC == 0) {
+                        const ProjPoint q = next_point(i + 1);
+                        project_pair<false>(R, src, l, p, q, v[i], v[i + 1]);
+                    } else {
+                        v[i] = make_float2(0.0f, 0.0f);
+                        if (p.idx >= 0)
+                            v[i] = store_point<PREC>(R.map, p.idx,
+                                                     project_node_at<PREC>(R, p.cx, p.cy, p.col,
+                                                                           p.row, spinor(l)));
                     }
                 }
             }
@@ -288,7 +325,10 @@ __global__ void __cluster_dims__(kFinCtas, 1, 1) __launch_bounds__(kFinThreads)
 }
 
 // Time-parallel combination, one thread per momentum: psi <- M_s psi for s =
-// 0 .. S-1 in time order, starting from v(p + A_in), all in FP64.
+// 0 .. S-1 in time order, starting from v(p + A_in), all in FP64.  Bound by FP64 latency
+// on a small grid: 16 FP64 operations per segment, 4 more to bring an FP32_MIXED column
+// to double (the conversions themselves are integer operations: a cvt issues on the
+// FP64 pipe), the columns of 4 segments loaded ahead.
 template <int PREC>
 __global__ void __launch_bounds__(128) combine_kernel(const __grid_constant__ CombineArgs a)
 {
@@ -301,16 +341,17 @@ __global__ void __launch_bounds__(128) combine_kernel(const __grid_constant__ Co
     double ar, ai, br, bi;
     initial_spinor(px + a.a_in[0], py + a.a_in[1], vs, ar, ai, br, bi);
     const size_t slab = static_cast<size_t>(a.n_points) * 32;
+#pragma unroll 4
     for (int s = 0; s < a.n_segments; ++s) {
         const unsigned char *seg = static_cast<const unsigned char *>(a.segs) + s * slab;
         double alr, ali, ber, bei;  // (alpha, beta): first column of M_s
         if constexpr (PREC == 1) {
             const float4 h = reinterpret_cast<const float4 *>(seg)[idx];
             const float4 l = reinterpret_cast<const float4 *>(seg)[a.n_points + idx];
-            alr = static_cast<double>(h.x) + l.x;
-            ali = static_cast<double>(h.y) + l.y;
-            ber = static_cast<double>(h.z) + l.z;
-            bei = static_cast<double>(h.w) + l.w;
+            alr = df_to_f64(h.x, l.x);
+            ali = df_to_f64(h.y, l.y);
+            ber = df_to_f64(h.z, l.z);
+            bei = df_to_f64(h.w, l.w);
         } else {
             const double2 c0 = reinterpret_cast<const double2 *>(seg)[idx];
             const double2 c1 = reinterpret_cast<const double2 *>(seg)[a.n_points + idx];
