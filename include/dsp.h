@@ -263,7 +263,7 @@ dsp_status dsp_get_cursor(const dsp_grid *g, int64_t *cursor, int64_t *n_steps);
  * diagonal (EXACT and STRANG_XY: the real diagonal cos(theta), so a step of
  * the product costs 8 multiply-adds instead of 12; MAGNUS4: cos|n|) and divide
  * the product by the square root of its determinant, so the applied operator
- * is unitary to FP32 rounding.  Where G > 1, EXACT and MAGNUS4 evaluate the
+ * is unitary to FP32 rounding.  Where G > 1, the library may evaluate the
  * operator of 16, 8 or 4 aligned steps at once, from the expansion of their
  * product in what A changes inside the group (its coefficients are formed once
  * per pulse), as long as the terms it drops, summed over the run, stay below

@@ -947,8 +947,7 @@ dsp_status prepare_pulse(dsp_grid *g, const double *a_mid, int64_t n_steps, doub
     g->group = choose_group(g->precision, g->scheme, g->tdeg, tmax);
     // groups that the grid's piece rule allows may be evaluated expanded: then the
     // device makes the per-step table too, from the caller's
-    g->by_groups = g->expand && g->group > 1 && g->scheme != DSP_SCHEME_STRANG_XY &&
-                   first_group_size(tmax) < dsp::kNumGroupSizes;
+    g->by_groups = g->expand && g->group > 1 && first_group_size(tmax) < dsp::kNumGroupSizes;
     if (g->by_groups) {
         host.resize(GroupMemory(g).raw_bytes);
         std::memcpy(host.data(), a_mid, host.size());

@@ -1,5 +1,4 @@
-// dsp_group.cu -- the FP32_MIXED evolve kernel on expanded step groups (EXACT and
-// MAGNUS4), and the kernel that expands a pulse's groups.  Shared device code is in
+// dsp_group.cu -- the FP32_MIXED evolve kernel on expanded step groups, and the kernel that expands a pulse's groups.  Shared device code is in
 // dsp_device.cuh.
 
 #include "dsp_device.cuh"
@@ -18,7 +17,9 @@ namespace {
 // instead of per step,
 //   w_z  = C + S x m1 + x (S x n3 + x S x n5)           x = S.S, u x v = u_x v_y - u_y v_x
 //   w_xy = S + (S_y, -S_x) (S x u2 + x S x u4) + K S
-// (GroupEntry).  What the expansion drops is summed over the run (GroupSums); the
+// (GroupEntry).  A STRANG_XY step is exp(-i sigma.P') with P' = P + cubic(P) in closed
+// series, so its groups are those of P': the same w with the cubic and fifth-order terms
+// of P' added to w_xy and their part of S x m1 to w_z (group_step).  What the expansion drops is summed over the run (GroupSums); the
 // kernels pick G and the level from the sums (pick_plan), and where no G passes the
 // step-by-step chains (dsp_strip.cu, dsp_mixed.cu), queued behind, take the run.
 //
@@ -47,8 +48,8 @@ namespace {
 // 209.2 -> 35.5 ms (lite, G = 16); 1024^2 x 3e4 Gaussian pulse 22.6 -> 5.1 ms (wide,
 // 16); 1000 x 750 x 2e4 two colours 10.36 -> 2.48 ms (wide, 16; contiguous tiles
 // before); 512^2 x 12000 MAGNUS4 3.14 -> 0.70 ms; 256^2 x 2e4 paper pulse 1.42 ->
-// 0.40 ms.  2-norm error of |c+|^2 against 64 bits on the last three: 3.7e-7 -> 2.3e-7,
-// 2.1e-7 -> 1.2e-7, 5.0e-7 -> 2.3e-7.
+// 0.40 ms; 512 x 384 x 12000 STRANG_XY 1.79 -> 0.63 ms.  2-norm error of |c+|^2 against 64 bits on the last four: 3.7e-7 -> 2.3e-7,
+// 2.1e-7 -> 1.2e-7, 5.0e-7 -> 2.3e-7, 2.9e-7 -> 1.1e-7.
 // ---------------------------------------------------------------------------
 
 constexpr int kGrpChunk = 32;  // group entries per staged chunk: one per lane
@@ -79,6 +80,7 @@ struct GroupCol {
     float Sx, Tx;  // hi of S_x; lite: S_x hi + lo
     float m1y, n3y, n5y, u2y, u4y;
     float kx, Kyx;  // wide: lo of S_x plus Kxx S_x; Kyx
+    float C;
 };
 
 // The row part of a group (V = float2: the two rows of a pack).
@@ -107,7 +109,9 @@ __device__ __forceinline__ GroupCol group_col(const float4 *e, float gxh, float 
         c.u2y = e1.y;
         c.u4y = e1.z;
         c.kx = __fmaf_rn(c.Sx, e1.w, lo);
-        c.Kyx = e[2].x;
+        const float4 e2 = e[2];
+        c.Kyx = e2.x;
+        c.C = e2.w;
     }
     return c;
 }
@@ -211,8 +215,12 @@ __device__ __forceinline__ void get_row(const float4 (*rows)[kGrpChunk], int, in
 
 // psi <- exp(-i sigma.w) psi for one group.  The operator's M - I is
 // [[m - i q_z, -(q_y + i q_x)], [q_y - i q_x, m + i q_z]], m = cos|w| - 1, q = sinc|w| w.
-template <bool WIDE, typename V>
-__device__ __forceinline__ void group_step(GroupPoint<V> &p, const GroupCol &c, const GroupRow<V> &r)
+// STRANG (wide only): the steps' P' = P + (-P_x P_y^2 (1/3 + (2 P_x^2 + P_y^2)/45),
+// P_y P_x^2 (1/6 + 7 P_x^2/360 - 2 P_y^2/45)) at P = S/G, and through its derivative
+// S x m1 gains (P_x^2/6 + P_y^2/3)(S_x m1_y + S_y m1_x); g2 = 1/G^2, C the entry's.
+template <bool WIDE, bool STRANG, typename V>
+__device__ __forceinline__ void group_step(GroupPoint<V> &p, const GroupCol &c,
+                                           const GroupRow<V> &r, float g2)
 {
     if constexpr (!WIDE) {
         const V Tx = vbc<V>(c.Tx);
@@ -224,14 +232,30 @@ __device__ __forceinline__ void group_step(GroupPoint<V> &p, const GroupCol &c, 
         apply_group(p, m, vneg(vfma(s, wz, wz)), vfma(s, r.Sy, r.Sy), vfma(s, Tx, Tx));
     } else {
         const V Sx = vbc<V>(c.Sx), Sy = r.Sy;
-        const V x0 = vfma(Sx, Sx, vmul(Sy, Sy));
+        const V v2 = vmul(Sy, Sy);
+        const V x0 = vfma(Sx, Sx, v2);
         const V A1 = vfma(Sx, vbc<V>(c.m1y), r.r1), A3 = vfma(Sx, vbc<V>(c.n3y), r.r3);
         const V A5 = vfma(Sx, vbc<V>(c.n5y), r.r5);
-        const V wz = vfma(x0, vfma(x0, A5, A3), A1);
+        V wz = vfma(x0, vfma(x0, A5, A3), A1);
         const V e = vfma(x0, vfma(Sx, vbc<V>(c.u4y), r.e4), vfma(Sx, vbc<V>(c.u2y), r.e2));
         // w_xy = S + v, v small
-        const V vx = vfma(Sy, e, vadd(vbc<V>(c.kx), r.kx));
-        const V vy = vfma(vneg(Sx), e, vfma(Sx, vbc<V>(c.Kyx), r.ky));
+        V vx = vfma(Sy, e, vadd(vbc<V>(c.kx), r.kx));
+        V vy = vfma(vneg(Sx), e, vfma(Sx, vbc<V>(c.Kyx), r.ky));
+        if constexpr (STRANG) {
+            // X = P_x^2, Y = P_y^2
+            const float Xs = __fmul_rn(g2, __fmul_rn(c.Sx, c.Sx));
+            const V X = vbc<V>(Xs), Y = vmul(vbc<V>(g2), v2);
+            const V hx = vfma(Y, vbc<V>(1.0f / 45.0f),
+                              vbc<V>(__fmaf_rn(Xs, 2.0f / 45.0f, 1.0f / 3.0f)));
+            const V hy = vfma(Y, vbc<V>(-2.0f / 45.0f),
+                              vbc<V>(__fmaf_rn(Xs, 7.0f / 360.0f, 1.0f / 6.0f)));
+            vx = vfma(vmul(vneg(Y), hx), Sx, vx);
+            vy = vfma(vmul(X, hy), Sy, vy);
+            // S_x m1_y + S_y m1_x = 2 S_x m1_y - (A1 - C)
+            const V sym = vfma(vbc<V>(__fadd_rn(c.Sx, c.Sx)), vbc<V>(c.m1y),
+                               vadd(vbc<V>(c.C), vneg(A1)));
+            wz = vfma(vfma(Y, vbc<V>(1.0f / 3.0f), vbc<V>(__fmul_rn(Xs, 1.0f / 6.0f))), sym, wz);
+        }
         const V x = vfma(vadd(Sx, Sx), vx, vfma(vadd(Sy, Sy), vy, vfma(wz, wz, x0)));
         const V s = vmul(vhorner<V, kWideDS, 1, 1>(x), x);
         // q = S + (s S + v), the sum left unrounded for the update
@@ -270,6 +294,17 @@ __device__ __forceinline__ void single_step(GroupPoint<V> &p, V Px, V Py, float 
     apply_group(p, m, vneg(vfma(s, nz, nz)), vfma(s, Py, Py), vfma(s, Px, Px));
 }
 
+template <typename V>
+__device__ __forceinline__ void single_step_strang(GroupPoint<V> &p, V Px, V Py)
+{  // coeffs_strang's operations
+    const V xx = vmul(Px, Px), xy = vmul(Py, Py);
+    const V cx = vmul(vhorner<V, kSingleDC, 1, 0>(xx), xx);
+    const V cy = vmul(vhorner<V, kSingleDC, 1, 0>(xy), xy);
+    const V sx = vfma(vmul(vhorner<V, kSingleDS, 1, 1>(xx), xx), Px, Px);
+    const V sy = vfma(vmul(vhorner<V, kSingleDS, 1, 1>(xy), xy), Py, Py);
+    apply_group(p, vfma(cx, cy, vadd(cx, cy)), vbc<V>(0.0f), sy, vfma(cy, sx, sx));
+}
+
 // A warp's spinors: H rows of one column per lane, as packs of two rows (H = 4, 2)
 // or one row alone (H = 1).
 template <int H>
@@ -284,7 +319,7 @@ __device__ __forceinline__ float &lane_of(float2 &v, int k) { return (k & 1) ? v
 __device__ __forceinline__ float2 pair_of(float a, float b, float2 *) { return make_float2(a, b); }
 __device__ __forceinline__ float pair_of(float a, float, float *) { return a; }
 
-template <int H, bool WIDE>
+template <int H, bool WIDE, bool STRANG>
 __device__ void body_group(const ReqDesc &R, int size, int tile, WarpSmem &sm, int *err)
 {
     using RowsT = Rows<H>;
@@ -355,7 +390,11 @@ __device__ void body_group(const ReqDesc &R, int size, int tile, WarpSmem &sm, i
             const float4 p0 = sm.prow[2 * q], p1 = sm.prow[H == 1 ? 0 : 2 * q + 1];
             const float y0 = __fadd_rn(p0.x * inv_g, __fadd_rn(a.y, p0.y * inv_g));
             const float y1 = __fadd_rn(p1.x * inv_g, __fadd_rn(a.y, p1.y * inv_g));
-            single_step(s.p[q], vbc<V>(Px), pair_of(y0, y1, static_cast<V *>(nullptr)), a.z, a.w);
+            const V Py = pair_of(y0, y1, static_cast<V *>(nullptr));
+            if constexpr (STRANG)
+                single_step_strang(s.p[q], vbc<V>(Px), Py);
+            else
+                single_step(s.p[q], vbc<V>(Px), Py, a.z, a.w);
         }
     };
 
@@ -433,7 +472,7 @@ __device__ void body_group(const ReqDesc &R, int size, int tile, WarpSmem &sm, i
             for (int q = 0; q < N; ++q) {
                 GroupRow<V> r;
                 get_row<WIDE>(sm.rows, q, j, r);
-                group_step<WIDE>(s.p[q], cc, r);
+                group_step<WIDE, STRANG>(s.p[q], cc, r, inv_g * inv_g);
             }
         }
         __syncwarp();  // the warp is done with the stage and the row parts
@@ -483,10 +522,12 @@ __global__ void __launch_bounds__(32 * kGroupWarps, 4)
     const GroupPick pick = pick_plan(R.groups);
     if (pick.size == kNumGroupSizes)
         return;  // step by step
-    if (pick.wide)
-        body_group<H, true>(R, pick.size, tile, sm, R.err);
+    if (R.scheme == 1)
+        body_group<H, true, true>(R, pick.size, tile, sm, R.err);
+    else if (pick.wide)
+        body_group<H, true, false>(R, pick.size, tile, sm, R.err);
     else
-        body_group<H, false>(R, pick.size, tile, sm, R.err);
+        body_group<H, false, false>(R, pick.size, tile, sm, R.err);
 }
 
 template <int H>
@@ -518,6 +559,8 @@ static_assert(kGroupWarps * sizeof(WarpSmem) <= 48 * 1024, "dynamic shared memor
 // (Magnus series; Blanes, Casas, Oteo and Ros, Phys. Rep. 470 (2009) 151.)  MAGNUS4
 // steps exp(-i (sigma.P_n + sigma_z P_n x D_n)) add the sigma_z parts of their
 // commutators to the disturbance: the same polynomials with other coefficients.
+// STRANG_XY's P' adds the second derivative of its cubic terms, sum d d, to K (the rest
+// of P' depends on S alone and is the evolve kernel's).
 // The next power of x = |S|^2 is folded into the kept ones (its Chebyshev
 // economisation on [0, eps^2], eps = G theta_max the largest |S| of the box).
 //
@@ -654,13 +697,33 @@ __device__ __forceinline__ void expand_group(const PrepArgs &args, int64_t g, fl
         u2 = u2 - static_cast<float>(k * i) * D1;
         wide += static_cast<float>(i) * sD * (s * eps + 0.03f * e7);
     }
+    // (the next power of K S, fitted to smooth pulses, at half the box's x)
+    const float kk = static_cast<float>(k) * (1.0f + 0.08f * X);
+    float Kxx = kk * Lyy, Kxy = -kk * Lxy, Kyx = -kk * Lyx, Kyy = kk * Lxx;
+    const float Kn = static_cast<float>(k) * (fabsf(Lxx) + fabsf(Lxy) + fabsf(Lyx) + fabsf(Lyy));
+    if (args.scheme == 1) {
+        float dxx = 0.0f, dxy = 0.0f, dyy = 0.0f;
+#pragma unroll
+        for (int n = 0; n < G; ++n) {
+            dxx += d[n].x * d[n].x;
+            dxy += d[n].x * d[n].y;
+            dyy += d[n].y * d[n].y;
+        }
+        constexpr float third = static_cast<float>(1.0 / (3.0 * G));
+        Kxx -= third * dyy;
+        Kxy -= 2.0f * third * dxy;
+        Kyx += third * dxy;
+        Kyy += 0.5f * third * dxx;
+        // the derivative of P' at the other terms, the next orders of P'
+        const float t2 = X * static_cast<float>(1.0 / G2);
+        wide += 0.1f * size1(n1) * eps * t2 * t2 +
+                0.7f * t2 * (size1(n3) * e3 + size1(u2) * X + Kn * eps) +
+                0.02f * eps * t2 * t2 * t2;
+    }
     // x^3 on [0, X] as 3/2 X x^2 - 9/16 X^2 x + X^3/32, off by X^3/32
     n5 = n5 + (1.5f * X) * n7;
     n3 = n3 - (0.5625f * X * X) * n7;
     n1 = n1 + (X * X * X * 0.03125f) * n7;
-    // the next power of K S, fitted to smooth pulses, at half the box's x
-    const float kk = static_cast<float>(k) * (1.0f + 0.08f * X);
-    const float Kn = kk * (fabsf(Lxx) + fabsf(Lxy) + fabsf(Lyx) + fabsf(Lyy));
     wide += size1(n7) * e7 * (0.05f + 0.1f * X) + 0.1f * size1(u4) * e3 * e3 + 0.07f * Kn * e3 +
             0.25f * X * s_odd * s_even + s * s * s * (1.0f / 24.0f);
     const float wz = fabsf(C) + size1(n1) * eps + size1(n3) * e3;
@@ -670,10 +733,10 @@ __device__ __forceinline__ void expand_group(const PrepArgs &args, int64_t g, fl
     float4 *e = reinterpret_cast<float4 *>(
         args.entries + group_entries_before(args.n_steps, I) + g);
     e[0] = make_float4(xh, static_cast<float>(sx - static_cast<double>(xh)), n1.y, n3.y);
-    e[1] = make_float4(n5.y, u2.y, u4.y, kk * Lyy);
-    e[2] = make_float4(-kk * Lyx, yh, static_cast<float>(sy - static_cast<double>(yh)), C);
+    e[1] = make_float4(n5.y, u2.y, u4.y, Kxx);
+    e[2] = make_float4(Kyx, yh, static_cast<float>(sy - static_cast<double>(yh)), C);
     e[3] = make_float4(n1.x, n3.x, n5.x, u2.x);
-    e[4] = make_float4(u4.x, -kk * Lxy, kk * Lxx, 0.0f);
+    e[4] = make_float4(u4.x, Kxy, Kyy, 0.0f);
 }
 
 // Adds the threads' estimates to a sum, in fixed point (clamped above the budget).

@@ -1,4 +1,4 @@
-"""FP32-mixed step groups evaluated from their expansion (EXACT and MAGNUS4): against the FP64
+"""FP32-mixed step groups evaluated from their expansion: against the FP64
 oracle, against the same steps taken one by one, and bitwise across the kernel's warp tiles, at
 grid sizes around its 32-column, 4-row tiles.
 
@@ -45,7 +45,9 @@ def solve(size, table, scheme="exact", valley=1, expand=True, tiling=1, pieces=N
 # steps); a count that is no multiple of 16 leaves steps alone at the end
 @pytest.mark.parametrize("size", SIZES)
 @pytest.mark.parametrize("scheme,steps", [("exact", 24005), ("exact", 5000), ("exact", 2403),
-                                          ("exact", 1501), ("magnus4", 6007), ("magnus4", 2600)])
+                                          ("exact", 1501), ("magnus4", 6007), ("magnus4", 2600),
+                                          ("strang_xy", 24005), ("strang_xy", 5000),
+                                          ("strang_xy", 2403), ("strang_xy", 1501)])
 def test_expansion_against_oracle_and_single_steps(orc, size, scheme, steps):
     pulse = W.sin2_pulse(2.0, 1.2, 4.0, eps=0.6)
     sample, oracle_table = ((B.sample_pulse_gauss, orc.pulse_table_gauss) if scheme == "magnus4"
