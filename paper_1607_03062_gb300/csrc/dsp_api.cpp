@@ -170,30 +170,69 @@ int32_t choose_group(int32_t precision, int32_t scheme, int32_t tdeg, double the
     return 1;
 }
 
-// dt * max over steps and box corners of |p + A_n| (|P| is convex in p, so the
-// maximum over the box is at a corner).  The squared magnitude of a corner is
-// (c_x + A_x)^2 + (c_y + A_y)^2, and a rounded sum grows with either term, so
-// the largest corner of a step is the larger x square plus the larger y square:
-// two squares per coordinate and one square root for the whole table.  If the
-// squares overflow (|p + A| above ~1e154), the maximum is taken with hypot.
-double theta_max(const dsp_grid *g, const double *a_mid, int64_t n, double dt)
+// Two doubles side by side, so that the scan below works on x and y (and on two
+// steps' sums) at once.
+typedef double Pair __attribute__((vector_size(16)));
+typedef long long PairMask __attribute__((vector_size(16)));
+inline Pair load_pair(const double *p)
 {
-    const double cx0 = g->px_min, cx1 = g->px_max, cy0 = g->py_min, cy1 = g->py_max;
-    double m2 = 0.0;
-    for (int64_t k = 0; k < n; ++k) {
-        const double x0 = cx0 + a_mid[2 * k], x1 = cx1 + a_mid[2 * k];
-        const double y0 = cy0 + a_mid[2 * k + 1], y1 = cy1 + a_mid[2 * k + 1];
-        m2 = std::max(m2, std::max(x0 * x0, x1 * x1) + std::max(y0 * y0, y1 * y1));
+    Pair v;
+    std::memcpy(&v, p, sizeof(v));
+    return v;
+}
+inline Pair larger(Pair a, Pair b) { return a < b ? b : a; }
+
+// Scans a table's n samples (A_x, A_y): false if one is not finite; else *tmax = dt *
+// max over samples and box corners of |p + A_n| (|P| is convex in p, so the maximum
+// over the box is at a corner).  The squared magnitude of a corner is (c_x + A_x)^2 +
+// (c_y + A_y)^2, and a rounded sum grows with either term, so the largest corner of a
+// step is the larger x square plus the larger y square: two squares per coordinate and
+// one square root for the whole table.  If the squares overflow (|p + A| above ~1e154),
+// the maximum is taken with hypot.  (Four steps per turn on independent accumulators;
+// the scan is most of what dsp_set_pulse does on the host.)
+bool scan_table(const dsp_grid *g, const double *a_mid, int64_t n, double dt, double *tmax)
+{
+    const Pair lo = {g->px_min, g->py_min}, hi = {g->px_max, g->py_max};
+    Pair m[2] = {{0.0, 0.0}, {0.0, 0.0}}, bad[2] = {{0.0, 0.0}, {0.0, 0.0}};
+    const auto corner = [&](Pair a) {
+        const Pair p = lo + a, q = hi + a;
+        return larger(p * p, q * q);
+    };
+    const auto two = [&](const double *p, int i) {
+        const Pair a0 = load_pair(p), a1 = load_pair(p + 2);
+        bad[i] += (a0 - a0) + (a1 - a1);  // 0, or NaN from an infinity or a NaN
+        const Pair f0 = corner(a0), f1 = corner(a1);
+        const Pair s = __builtin_shuffle(f0, f1, PairMask{0, 2}) +
+                       __builtin_shuffle(f0, f1, PairMask{1, 3});
+        m[i] = larger(m[i], s);
+    };
+    int64_t k = 0;
+    for (; k + 4 <= n; k += 4) {
+        two(a_mid + 2 * k, 0);
+        two(a_mid + 2 * k + 4, 1);
     }
-    if (std::isfinite(m2))
-        return dt * std::sqrt(m2);
-    double m = 0.0;
-    const double cx[2] = {cx0, cx1}, cy[2] = {cy0, cy1};
-    for (int64_t k = 0; k < n; ++k)
+    double m2 = std::max(std::max(m[0][0], m[0][1]), std::max(m[1][0], m[1][1]));
+    const Pair b = bad[0] + bad[1];
+    double rest = b[0] + b[1];
+    for (; k < n; ++k) {
+        const Pair a = load_pair(a_mid + 2 * k), f = corner(a);
+        rest += (a[0] - a[0]) + (a[1] - a[1]);
+        m2 = std::max(m2, f[0] + f[1]);
+    }
+    if (!(rest == 0.0))
+        return false;
+    if (std::isfinite(m2)) {
+        *tmax = dt * std::sqrt(m2);
+        return true;
+    }
+    double h = 0.0;
+    const double cx[2] = {g->px_min, g->px_max}, cy[2] = {g->py_min, g->py_max};
+    for (k = 0; k < n; ++k)
         for (int i = 0; i < 2; ++i)
             for (int j = 0; j < 2; ++j)
-                m = std::max(m, std::hypot(cx[i] + a_mid[2 * k], cy[j] + a_mid[2 * k + 1]));
-    return dt * m;
+                h = std::max(h, std::hypot(cx[i] + a_mid[2 * k], cy[j] + a_mid[2 * k + 1]));
+    *tmax = dt * h;
+    return true;
 }
 
 // SMs of the device, looked up once for the process (152 where there is none to ask).
@@ -246,22 +285,27 @@ int32_t first_group_size(double theta_max)
     return i;
 }
 
-// Layout of a grid's expanded-group memory: the caller's table in FP64, the sums, the
-// entries of every group size.
+// Layout of a grid's expanded-group memory: what one copy uploads (the caller's table
+// in FP64, the sums as zeros, the projection nodes), then the entries of every group
+// size.
 struct GroupMemory {
-    size_t raw_bytes, entry_bytes;
-    explicit GroupMemory(const dsp_grid *g) : GroupMemory(g->scheme, g->n_steps) {}
-    GroupMemory(int32_t scheme, int64_t n)
-        : raw_bytes((scheme == DSP_SCHEME_MAGNUS4 ? 32 : 16) * static_cast<size_t>(n)),
+    size_t raw_bytes, node_bytes, entry_bytes;
+    explicit GroupMemory(const dsp_grid *g)
+        : raw_bytes((g->scheme == DSP_SCHEME_MAGNUS4 ? 32 : 16) * static_cast<size_t>(g->n_steps)),
+          node_bytes((sizeof(float2) * (static_cast<size_t>(g->nx) + static_cast<size_t>(g->ny)) +
+                      15) & ~static_cast<size_t>(15)),
           entry_bytes(0)
     {
         for (int i = 0; i < dsp::kNumGroupSizes; ++i)
-            entry_bytes += sizeof(dsp::GroupEntry) * static_cast<size_t>(n / dsp::group_size(i));
+            entry_bytes +=
+                sizeof(dsp::GroupEntry) * static_cast<size_t>(g->n_steps / dsp::group_size(i));
     }
     static constexpr size_t kSums = 64;
-    size_t total() const { return raw_bytes + kSums + entry_bytes; }
-    unsigned char *sums(void *base) const { return static_cast<unsigned char *>(base) + raw_bytes; }
-    unsigned char *entries(void *base) const { return sums(base) + kSums; }
+    size_t upload() const { return raw_bytes + kSums + node_bytes; }
+    size_t total() const { return upload() + entry_bytes; }
+    size_t sums() const { return raw_bytes; }
+    size_t nodes() const { return raw_bytes + kSums; }
+    size_t entries() const { return upload(); }
 };
 static_assert(sizeof(dsp::GroupSums) <= GroupMemory::kSums, "the sums' slot");
 
@@ -274,7 +318,10 @@ ReqDesc make_desc(const dsp_grid *g, int64_t begin, int64_t end, bool project, v
     r.map = map;
     r.partials = g->partials;
     r.err = g->scal ? &g->scal->err : nullptr;
-    r.nodes_out = g->nodes;
+    r.nodes_out = g->by_groups ? reinterpret_cast<const float2 *>(
+                                     static_cast<const unsigned char *>(g->groups) +
+                                     GroupMemory(g).nodes())
+                               : g->nodes;
     r.px_min = g->px_min;
     r.py_min = g->py_min;
     r.hx = g->hx;
@@ -315,8 +362,9 @@ ReqDesc make_desc(const dsp_grid *g, int64_t begin, int64_t end, bool project, v
     if (g->by_groups && end > begin) {
         const GroupMemory m(g);
         r.by_groups = 1;
-        r.groups.entries = reinterpret_cast<const dsp::GroupEntry *>(m.entries(g->groups));
-        r.groups.sums = reinterpret_cast<const dsp::GroupSums *>(m.sums(g->groups));
+        const unsigned char *base = static_cast<const unsigned char *>(g->groups);
+        r.groups.entries = reinterpret_cast<const dsp::GroupEntry *>(base + m.entries());
+        r.groups.sums = reinterpret_cast<const dsp::GroupSums *>(base + m.sums());
         r.groups.n_steps = g->n_steps;
         r.groups.eps = static_cast<float>(dsp::group_size(0) * g->theta_max);
         r.groups.first = first_group_size(g->theta_max);
@@ -698,10 +746,9 @@ dsp_status validate_pulse_args(const dsp_grid *g, const double *a_mid, int64_t n
         return DSP_E_INVALID;
     if (!finite(a_in[0]) || !finite(a_in[1]) || !finite(a_out[0]) || !finite(a_out[1]))
         return DSP_E_INVALID;
-    for (int64_t k = 0; k < 2 * n_steps; ++k)
-        if (!finite(a_mid[k]))
-            return DSP_E_INVALID;
-    const double tmax = n_steps > 0 ? theta_max(g, a_mid, n_steps, dt) : 0.0;
+    double tmax = 0.0;
+    if (n_steps > 0 && !scan_table(g, a_mid, n_steps, dt, &tmax))
+        return DSP_E_INVALID;
     if (tmax > kPi)
         return DSP_E_CFL;
     if (tmax_out)
@@ -727,11 +774,22 @@ size_t table_bytes(int32_t precision, int32_t scheme, int64_t n)
     return (entry_bytes(precision, scheme) * static_cast<size_t>(n) + 15) & ~static_cast<size_t>(15);
 }
 
+// Host memory to be filled before it is read (a vector would zero it first).
+struct HostBytes {
+    std::unique_ptr<unsigned char[]> p;
+    size_t n = 0;
+    void alloc(size_t bytes)
+    {
+        p.reset(new unsigned char[bytes]);
+        n = bytes;
+    }
+    unsigned char *data() const { return p.get(); }
+    size_t size() const { return n; }
+};
+
 // Fills the table layout the kernels read (see ReqDesc::table).
-void build_table(const dsp_grid *g, const double *a_mid, int64_t n, double dt,
-                 std::vector<unsigned char> &out)
+void build_table(const dsp_grid *g, const double *a_mid, int64_t n, double dt, unsigned char *out)
 {
-    out.resize(static_cast<size_t>(n) * entry_bytes(g->precision, g->scheme));
     // valley K- is stepped as K+ on -P, so its table holds -dt*A
     const double vs = g->valley > 0 ? 1.0 : -1.0;
     if (g->scheme == DSP_SCHEME_MAGNUS4) {
@@ -745,14 +803,14 @@ void build_table(const dsp_grid *g, const double *a_mid, int64_t n, double dt,
             const double dx = kappa * (vs * (dt * (a[2] - a[0])));
             const double dy = kappa * (vs * (dt * (a[3] - a[1])));
             if (g->precision == DSP_FP64) {
-                double *t = reinterpret_cast<double *>(out.data()) + 4 * k;
+                double *t = reinterpret_cast<double *>(out) + 4 * k;
                 t[0] = bx;
                 t[1] = by;
                 t[2] = dx;
                 t[3] = dy;
             } else {
                 // Abar rounded with error feedback, as for the midpoint table below
-                float *t = reinterpret_cast<float *>(out.data()) + 4 * k;
+                float *t = reinterpret_cast<float *>(out) + 4 * k;
                 const double vx = bx + mresid[0], vy = by + mresid[1];
                 t[0] = static_cast<float>(vx);
                 t[1] = static_cast<float>(vy);
@@ -765,7 +823,7 @@ void build_table(const dsp_grid *g, const double *a_mid, int64_t n, double dt,
         return;
     }
     if (g->precision == DSP_FP64) {
-        double *t = reinterpret_cast<double *>(out.data());
+        double *t = reinterpret_cast<double *>(out);
         for (int64_t k = 0; k < n; ++k) {
             t[2 * k] = vs * (dt * a_mid[2 * k]);
             t[2 * k + 1] = vs * (dt * a_mid[2 * k + 1]);
@@ -775,7 +833,7 @@ void build_table(const dsp_grid *g, const double *a_mid, int64_t n, double dt,
         // rounding residual, so the running sum of the stored dt*A stays within half
         // a float ulp of the exact running sum.  The phase integrates A over time; the
         // per-step roundings then cannot random-walk in it, however long the run.
-        float *t = reinterpret_cast<float *>(out.data());
+        float *t = reinterpret_cast<float *>(out);
         double resid[2] = {0.0, 0.0};
         for (int64_t k = 0; k < n; ++k)
             for (int c = 0; c < 2; ++c) {
@@ -791,9 +849,8 @@ void build_table(const dsp_grid *g, const double *a_mid, int64_t n, double dt,
 // valley, formed in FP64 as the kernels form the grid nodes (p = lo + (i + 1/2) h),
 // each split into an FP32 hi + lo pair for the double-float projection: nx
 // columns, then the grid's ny rows (global rows row0 ...).
-void build_nodes(const dsp_grid *g, std::vector<float2> &out)
+void build_nodes(const dsp_grid *g, float2 *out)
 {
-    out.resize(static_cast<size_t>(g->nx) + static_cast<size_t>(g->ny));
     const double vs = g->valley > 0 ? 1.0 : -1.0;
     const auto put = [&](size_t k, double v) {
         const float h = static_cast<float>(v);
@@ -920,12 +977,12 @@ dsp_status create_grid_impl(int32_t nx, int32_t ny, double px_min, double px_max
     return DSP_OK;
 }
 
-// Host part of setting a pulse: validates, fills the grid's pulse fields, lays
-// out the device table in `host` and the projection nodes in `nodes`.  Nothing
-// is queued.
+// Host part of setting a pulse: validates, fills the grid's pulse fields, and lays out
+// in `host` what is uploaded: for expanded groups GroupMemory's upload (the device makes
+// the per-step table from it), else the per-step table, padded to 16 bytes, and the
+// projection nodes.  Nothing is queued.
 dsp_status prepare_pulse(dsp_grid *g, const double *a_mid, int64_t n_steps, double dt,
-                         const double a_in[2], const double a_out[2],
-                         std::vector<unsigned char> &host, std::vector<float2> &nodes)
+                         const double a_in[2], const double a_out[2], HostBytes &host)
 {
     // every (A_x, A_y) sample of the table, whatever the samples per step
     const int64_t n_samples = n_steps * samples_per_step(g->scheme);
@@ -945,19 +1002,23 @@ dsp_status prepare_pulse(dsp_grid *g, const double *a_mid, int64_t n_steps, doub
     g->level = choose_level(g->precision, tmax, n_steps);
     g->tdeg = g->precision == DSP_FP32_MIXED ? choose_tan_degree(g->scheme, tmax, n_steps) : 0;
     g->group = choose_group(g->precision, g->scheme, g->tdeg, tmax);
-    // groups that the grid's piece rule allows may be evaluated expanded: then the
-    // device makes the per-step table too, from the caller's
-    g->by_groups = g->expand && g->group > 1 && first_group_size(tmax) < dsp::kNumGroupSizes;
-    if (g->by_groups) {
-        host.resize(GroupMemory(g).raw_bytes);
-        std::memcpy(host.data(), a_mid, host.size());
-    } else {
-        build_table(g, a_mid, n_steps, dt, host);
-    }
     g->fresh = true;
     g->projected = false;
     g->state_stale = false;
-    build_nodes(g, nodes);
+    // groups that the grid's piece rule allows may be evaluated expanded
+    g->by_groups = g->expand && g->group > 1 && first_group_size(tmax) < dsp::kNumGroupSizes;
+    if (g->by_groups) {
+        const GroupMemory m(g);
+        host.alloc(m.upload());
+        std::memcpy(host.data(), a_mid, m.raw_bytes);
+        std::memset(host.data() + m.sums(), 0, m.kSums);
+        build_nodes(g, reinterpret_cast<float2 *>(host.data() + m.nodes()));
+    } else {
+        const size_t tb = table_bytes(g->precision, g->scheme, n_steps);
+        host.alloc(tb + node_bytes(g));
+        build_table(g, a_mid, n_steps, dt, host.data());
+        build_nodes(g, reinterpret_cast<float2 *>(host.data() + tb));
+    }
     return DSP_OK;
 }
 
@@ -975,19 +1036,18 @@ cudaError_t prep_groups(const dsp_grid *g, cudaStream_t stream)
     a.first = first_group_size(g->theta_max);
     a.eps = static_cast<float>(dsp::group_size(0) * g->theta_max);
     a.table = g->table;
-    a.entries = reinterpret_cast<dsp::GroupEntry *>(m.entries(g->groups));
-    a.sums = reinterpret_cast<dsp::GroupSums *>(m.sums(g->groups));
-    const cudaError_t e = cudaMemsetAsync(a.sums, 0, sizeof(dsp::GroupSums), stream);
-    return e == cudaSuccess ? dsp::launch_prep_groups(a, stream) : e;
+    unsigned char *base = static_cast<unsigned char *>(g->groups);
+    a.entries = reinterpret_cast<dsp::GroupEntry *>(base + m.entries());
+    a.sums = reinterpret_cast<dsp::GroupSums *>(base + m.sums());
+    return dsp::launch_prep_groups(a, stream);
 }
 
 dsp_status set_pulse_impl(dsp_grid *g, const double *a_mid, int64_t n_steps, double dt,
                           const double a_in[2], const double a_out[2])
 {
     dsp_grid staged = *g;
-    std::vector<unsigned char> host;
-    std::vector<float2> nodes;
-    dsp_status s = prepare_pulse(&staged, a_mid, n_steps, dt, a_in, a_out, host, nodes);
+    HostBytes host;
+    dsp_status s = prepare_pulse(&staged, a_mid, n_steps, dt, a_in, a_out, host);
     if (s != DSP_OK)
         return s;
     cudaError_t e = cudaSuccess;
@@ -999,7 +1059,7 @@ dsp_status set_pulse_impl(dsp_grid *g, const double *a_mid, int64_t n_steps, dou
                 e = cudaFree(g->groups);
             g->groups = nullptr;
             g->groups_cap = 0;
-            g->by_groups = false;  // the pulse before goes on step by step
+            g->has_pulse = false;  // the pulse before is gone
         }
         if (e == cudaSuccess)
             e = cudaMalloc(&g->groups, gbytes);
@@ -1017,6 +1077,7 @@ dsp_status set_pulse_impl(dsp_grid *g, const double *a_mid, int64_t n_steps, dou
                 e = cudaFree(g->table);
             g->table = nullptr;
             g->table_cap = 0;
+            g->has_pulse = false;  // the pulse before is gone
         }
         if (e == cudaSuccess)
             e = cudaMalloc(&g->table, table_bytes(g->precision, g->scheme, n_steps));
@@ -1026,18 +1087,21 @@ dsp_status set_pulse_impl(dsp_grid *g, const double *a_mid, int64_t n_steps, dou
         }
         g->table_cap = n_steps;
     }
-    if (n_steps > 0) {
-        e = cudaMemcpyAsync(staged.by_groups ? g->groups : g->table, host.data(), host.size(),
-                            cudaMemcpyHostToDevice, g->stream);
-        if (e == cudaSuccess && staged.by_groups) {
+    if (staged.by_groups) {
+        e = cudaMemcpyAsync(g->groups, host.data(), host.size(), cudaMemcpyHostToDevice, g->stream);
+        if (e == cudaSuccess) {
             staged.table = g->table;
             staged.groups = g->groups;
             e = prep_groups(&staged, g->stream);
         }
-        if (e != cudaSuccess)
-            return latch_cuda(g, e);
+    } else {
+        const size_t tb = host.size() - node_bytes(g);
+        if (n_steps > 0)
+            e = cudaMemcpyAsync(g->table, host.data(), tb, cudaMemcpyHostToDevice, g->stream);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(g->nodes, host.data() + tb, node_bytes(g), cudaMemcpyHostToDevice,
+                                g->stream);
     }
-    e = cudaMemcpyAsync(g->nodes, nodes.data(), node_bytes(g), cudaMemcpyHostToDevice, g->stream);
     if (e != cudaSuccess)
         return latch_cuda(g, e);
     staged.table = g->table;
@@ -1795,28 +1859,17 @@ dsp_status server_admit(dsp_server *s, ServerReq *r)
     const dsp_request &p = r->p;
     fill_grid(&r->g, p.nx, p.ny, p.px_min, p.px_max, p.py_min, p.py_max, p.precision, p.scheme,
               p.valley, s->stream);
-    std::vector<unsigned char> host;
-    std::vector<float2> nodes;
-    dsp_status st =
-        prepare_pulse(&r->g, r->a_mid.data(), p.n_steps, p.dt, p.a_in, p.a_out, host, nodes);
+    HostBytes host;
+    dsp_status st = prepare_pulse(&r->g, r->a_mid.data(), p.n_steps, p.dt, p.a_in, p.a_out, host);
     if (st != DSP_OK)
         return st;
     r->g.keep_final_state = false;  // a finished request's state is never read again
-    // One copy uploads the table (padded to 16 bytes) and the projection nodes; for
-    // expanded groups the nodes and the caller's table, from which the device makes
-    // the rest: block holds table | nodes | group memory, the last two from o_nodes.
+    // One copy uploads the table and the projection nodes, or what the expanded groups
+    // start from, which then lies behind the table that the device fills.
     const size_t tb = table_bytes(p.precision, p.scheme, p.n_steps);
-    const size_t nb = (node_bytes(&r->g) + 15) & ~static_cast<size_t>(15);
     const bool by_groups = r->g.by_groups;
-    std::vector<unsigned char> up((by_groups ? 0 : tb) + nb, 0);
-    std::memcpy(up.data() + (by_groups ? 0 : tb), nodes.data(), node_bytes(&r->g));
-    if (by_groups)
-        up.insert(up.end(), host.begin(), host.end());
-    else if (!host.empty())
-        std::memcpy(up.data(), host.data(), host.size());
-    host.swap(up);
     const size_t o_up = by_groups ? tb : 0;  // where the upload lands after o_table
-    const size_t region = tb + nb + (by_groups ? GroupMemory(&r->g).total() : 0);
+    const size_t region = by_groups ? tb + GroupMemory(&r->g).total() : host.size();
     const size_t pts = static_cast<size_t>(r->g.n_points);
     const size_t o_table = align256(32 * pts);
     const size_t o_part = o_table + align256(region);
@@ -1836,8 +1889,8 @@ dsp_status server_admit(dsp_server *s, ServerReq *r)
     r->g.state = b;
     r->g.table = b + o_table;
     r->g.table_cap = p.n_steps;
-    r->g.nodes = reinterpret_cast<float2 *>(b + o_table + tb);
-    r->g.groups = by_groups ? b + o_table + tb + nb : nullptr;
+    r->g.nodes = by_groups ? nullptr : reinterpret_cast<float2 *>(b + o_table + tb);
+    r->g.groups = by_groups ? b + o_table + tb : nullptr;
     r->g.partials = reinterpret_cast<double *>(b + o_part);
     r->g.scal = reinterpret_cast<DeviceScalars *>(b + o_scal);
     r->map_dev = b + o_map;
@@ -1852,7 +1905,7 @@ dsp_status server_admit(dsp_server *s, ServerReq *r)
     }
     // table: host -> pinned staging -> device on the copy stream; the compute
     // stream waits for it before the first launch
-    if (!host.empty()) {
+    {
         if (cudaEventSynchronize(s->upload_done) != cudaSuccess)  // staging free again
             return server_fail(s, DSP_E_CUDA);
         if (host.size() > s->staging_cap) {
@@ -1872,9 +1925,6 @@ dsp_status server_admit(dsp_server *s, ServerReq *r)
             cudaStreamWaitEvent(s->stream, s->upload_done, 0) != cudaSuccess)
             return server_fail(s, DSP_E_CUDA);
     }
-    if (host.empty() && (cudaEventRecord(s->upload_done, s->copy_stream) != cudaSuccess ||
-                         cudaStreamWaitEvent(s->stream, s->upload_done, 0) != cudaSuccess))
-        return server_fail(s, DSP_E_CUDA);
     r->footprint = footprint_of(p);
     s->used += r->footprint;
     r->state = DSP_REQ_ACTIVE;
