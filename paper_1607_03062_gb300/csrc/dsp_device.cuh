@@ -513,10 +513,10 @@ __host__ __device__ __forceinline__ int64_t group_entries_before(int64_t n_steps
 }
 
 // The group size a run takes (an index of group_size, kNumGroupSizes: step by
-// step) and whether its groups are evaluated at the wide level.
+// step) and the level its groups are evaluated at.
 struct GroupPick {
     int size;
-    bool wide;
+    int level;
 };
 __device__ __forceinline__ GroupPick pick_plan(const GroupTable &t)
 {
@@ -525,10 +525,12 @@ __device__ __forceinline__ GroupPick pick_plan(const GroupTable &t)
     for (int i = t.first; i < kNumGroupSizes; ++i)
         if (t.n_steps >= group_size(i) && __ldg(&t.sums->wide[i]) <= budget) {
             const float eps = t.eps / static_cast<float>(1 << i);
-            return {i, !(eps <= static_cast<float>(kGroupAngleLite) &&
-                         __ldg(&t.sums->lite[i]) <= budget)};
+            const bool lite =
+                eps <= static_cast<float>(kGroupAngleLite) && __ldg(&t.sums->lite[i]) <= budget;
+            return {i, lite ? kGroupLite
+                       : eps <= static_cast<float>(kGroupAngleFull) ? kGroupFull : kGroupWide};
         }
-    return {kNumGroupSizes, true};
+    return {kNumGroupSizes, kGroupWide};
 }
 // A step-by-step kernel leaves a request of a pair to the expanded groups where the
 // plan picked them.

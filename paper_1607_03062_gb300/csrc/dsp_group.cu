@@ -24,16 +24,16 @@ namespace {
 // step-by-step chains (dsp_strip.cu, dsp_mixed.cu), queued behind, take the run.
 //
 // S comes as hi + lo (each from an exact sum of the hi/lo halves of G dt p and of
-// the group's sum of dt A), so no step's momentum is rounded on the way.  Two levels:
-//   lite  drops n5, u2, u4 and K (their sums passed the bound too) and
-//               adds the lo part of S to its hi part;
-//   wide  keeps everything, applies S and the small rest of w apart (the
-//               rounding of their sum is not paid), and takes cos|w| - 1 from the
-//               rounded vector part of the operator, so that the operator is unitary
-//               to the rounding of its entries however large the group's angle.
+// the group's sum of dt A), so no step's momentum is rounded on the way.  Three levels:
+//   lite  drops n5, u2, u4 and K (their sums passed the bound too) and adds the lo
+//         part of S to its hi part;
+//   full  keeps everything, and takes cos|w| - 1 from the rounded vector part of the
+//         operator, so that the operator is unitary to the rounding of its entries;
+//   wide  also applies S and the small rest of w apart, because at large group angles
+//         the rounding of their sum would show.
 //
-// What bounds it: FP32 issue.  Per spinor and group 42 (lite) or 72 (wide) lane
-// operations plus a column part shared by the warp's rows, against 9 and more per
+// What bounds it: FP32 issue.  Per spinor and group 42 (lite), 64 (full) or 76 (wide)
+// lane operations plus a column part shared by the warp's rows, against 9 and more per
 // spinor and STEP of the chains.
 //
 // Tiles: one warp owns 32 columns x H rows (H = 4, 2: packed FP32x2 row pairs; H =
@@ -56,10 +56,11 @@ constexpr int kGrpChunk = 32;  // group entries per staged chunk: one per lane
 constexpr int kGrpStage = kGrpChunk * static_cast<int>(sizeof(GroupEntry));
 static_assert(sizeof(GroupEntry) % 16 == 0, "bulk copies of whole entries");
 
-// cos - 1 and sinc - 1 series degrees in |w|^2: at the level's largest angle the
-// first omitted terms turn a group by 1e-11 (lite, 0.25) and 3e-12 (wide, 0.72; its
-// cos, off by 4e-11, is corrected from the sinc), 1e-7 over 1e4 groups.
-constexpr int kLiteDC = 4, kLiteDS = 3, kWideDC = 5, kWideDS = 5;
+// cos - 1 and sinc - 1 series degrees in |w|^2: at a level's largest angle the
+// first omitted terms turn a group by 1e-11 (lite, 0.25), 1e-13 (full, 0.32) and 3e-12
+// (wide, 0.72), 1e-7 over 1e4 groups; the cos of full and wide, off by 3e-9 and 4e-11,
+// is corrected from the sinc.
+constexpr int kLiteDC = 4, kLiteDS = 3, kFullDC = 3, kFullDS = 4, kWideDC = 5, kWideDS = 5;
 // Steps outside whole groups, one at a time: theta <= kGroupAngleTan / 2.
 constexpr int kSingleDC = 4, kSingleDS = 4;
 
@@ -215,14 +216,14 @@ __device__ __forceinline__ void get_row(const float4 (*rows)[kGrpChunk], int, in
 
 // psi <- exp(-i sigma.w) psi for one group.  The operator's M - I is
 // [[m - i q_z, -(q_y + i q_x)], [q_y - i q_x, m + i q_z]], m = cos|w| - 1, q = sinc|w| w.
-// STRANG (wide only): the steps' P' = P + (-P_x P_y^2 (1/3 + (2 P_x^2 + P_y^2)/45),
+// STRANG (full and wide): the steps' P' = P + (-P_x P_y^2 (1/3 + (2 P_x^2 + P_y^2)/45),
 // P_y P_x^2 (1/6 + 7 P_x^2/360 - 2 P_y^2/45)) at P = S/G, and through its derivative
 // S x m1 gains (P_x^2/6 + P_y^2/3)(S_x m1_y + S_y m1_x); g2 = 1/G^2, C the entry's.
-template <bool WIDE, bool STRANG, typename V>
+template <int LEVEL, bool STRANG, typename V>
 __device__ __forceinline__ void group_step(GroupPoint<V> &p, const GroupCol &c,
                                            const GroupRow<V> &r, float g2)
 {
-    if constexpr (!WIDE) {
+    if constexpr (LEVEL == kGroupLite) {
         const V Tx = vbc<V>(c.Tx);
         const V x = vfma(Tx, Tx, r.y2);
         const V A1 = vfma(Tx, vbc<V>(c.m1y), r.r1), A3 = vfma(Tx, vbc<V>(c.n3y), r.r3);
@@ -256,15 +257,27 @@ __device__ __forceinline__ void group_step(GroupPoint<V> &p, const GroupCol &c,
                                vadd(vbc<V>(c.C), vneg(A1)));
             wz = vfma(vfma(Y, vbc<V>(1.0f / 3.0f), vbc<V>(__fmul_rn(Xs, 1.0f / 6.0f))), sym, wz);
         }
+        // m = cos - 1 with one Newton step on (1 + m)^2 + q.q = 1, y = q.q
+        const auto cos1 = [](V m, V y) {
+            return vfma(vbc<V>(-0.5f), vfma(vbc<V>(2.0f), m, vfma(m, m, y)), m);
+        };
+        if constexpr (LEVEL == kGroupFull) {
+            const V Tx = vadd(Sx, vx), Ty = vadd(Sy, vy);
+            const V x = vfma(Tx, Tx, vfma(Ty, Ty, vmul(wz, wz)));
+            const V s = vmul(vhorner<V, kFullDS, 1, 1>(x), x);
+            const V qx = vfma(s, Tx, Tx), qy = vfma(s, Ty, Ty), qz = vfma(s, wz, wz);
+            const V m = cos1(vmul(vhorner<V, kFullDC, 1, 0>(x), x),
+                             vfma(qx, qx, vfma(qy, qy, vmul(qz, qz))));
+            apply_group(p, m, vneg(qz), qy, qx);
+            return;
+        }
         const V x = vfma(vadd(Sx, Sx), vx, vfma(vadd(Sy, Sy), vy, vfma(wz, wz, x0)));
         const V s = vmul(vhorner<V, kWideDS, 1, 1>(x), x);
         // q = S + (s S + v), the sum left unrounded for the update
         const V qx = vfma(s, Sx, vx), qy = vfma(s, Sy, vy), qz = vfma(s, wz, wz);
         const V fx = vadd(Sx, qx), fy = vadd(Sy, qy);
-        // m = cos - 1 with one Newton step on (1 + m)^2 + q.q = 1
-        V m = vmul(vhorner<V, kWideDC, 1, 0>(x), x);
-        const V y = vfma(fx, fx, vfma(fy, fy, vmul(qz, qz)));
-        m = vfma(vbc<V>(-0.5f), vfma(vbc<V>(2.0f), m, vfma(m, m, y)), m);
+        const V m = cos1(vmul(vhorner<V, kWideDC, 1, 0>(x), x),
+                         vfma(fx, fx, vfma(fy, fy, vmul(qz, qz))));
         const V nqx = vneg(qx), nqy = vneg(qy), nqz = vneg(qz), nSx = vneg(Sx), nSy = vneg(Sy);
         V dar = vfma(m, p.ar, vfma(qz, p.ai, vfma(nqy, p.br, vfma(qx, p.bi, p.lar))));
         V dai = vfma(m, p.ai, vfma(nqz, p.ar, vfma(nqy, p.bi, vfma(nqx, p.br, p.lai))));
@@ -319,9 +332,10 @@ __device__ __forceinline__ float &lane_of(float2 &v, int k) { return (k & 1) ? v
 __device__ __forceinline__ float2 pair_of(float a, float b, float2 *) { return make_float2(a, b); }
 __device__ __forceinline__ float pair_of(float a, float, float *) { return a; }
 
-template <int H, bool WIDE, bool STRANG>
+template <int H, int LEVEL, bool STRANG>
 __device__ void body_group(const ReqDesc &R, int size, int tile, WarpSmem &sm, int *err)
 {
+    constexpr bool WIDE = LEVEL != kGroupLite;  // the entries' parts that full and wide read
     using RowsT = Rows<H>;
     using V = typename RowsT::V;
     constexpr int N = RowsT::N;
@@ -472,7 +486,7 @@ __device__ void body_group(const ReqDesc &R, int size, int tile, WarpSmem &sm, i
             for (int q = 0; q < N; ++q) {
                 GroupRow<V> r;
                 get_row<WIDE>(sm.rows, q, j, r);
-                group_step<WIDE, STRANG>(s.p[q], cc, r, inv_g * inv_g);
+                group_step<LEVEL, STRANG>(s.p[q], cc, r, inv_g * inv_g);
             }
         }
         __syncwarp();  // the warp is done with the stage and the row parts
@@ -523,11 +537,14 @@ __global__ void __launch_bounds__(32 * kGroupWarps, 4)
     if (pick.size == kNumGroupSizes)
         return;  // step by step
     if (R.scheme == 1)
-        body_group<H, true, true>(R, pick.size, tile, sm, R.err);
-    else if (pick.wide)
-        body_group<H, true, false>(R, pick.size, tile, sm, R.err);
+        pick.level == kGroupWide ? body_group<H, kGroupWide, true>(R, pick.size, tile, sm, R.err)
+                                 : body_group<H, kGroupFull, true>(R, pick.size, tile, sm, R.err);
+    else if (pick.level == kGroupWide)
+        body_group<H, kGroupWide, false>(R, pick.size, tile, sm, R.err);
+    else if (pick.level == kGroupFull)
+        body_group<H, kGroupFull, false>(R, pick.size, tile, sm, R.err);
     else
-        body_group<H, false, false>(R, pick.size, tile, sm, R.err);
+        body_group<H, kGroupLite, false>(R, pick.size, tile, sm, R.err);
 }
 
 template <int H>

@@ -78,10 +78,12 @@ struct GroupEntry {
 };
 // Largest group angle G theta_max of each level of the expansion.  In an exact CPU
 // emulation of the kernel's FP32 arithmetic against FP64 steps (2-norm error of
-// |c+|^2 over 600 points; step-by-step chains, then lite or wide): 2048^2 sin^2
-// pulse, angle 0.16: 4.2e-7, 2.8e-7; paper pulse, 0.55: 5.7e-7, 2.1e-7; Gaussian
+// |c+|^2 over 600 points; step-by-step chains, then lite, full or wide): 2048^2 sin^2
+// pulse, angle 0.16: 4.2e-7, 2.8e-7 (lite); Gaussian pulse, 0.31: 2.5e-7, 2.3e-7 (full;
+// at 0.63 it would be 3.0e-7); wide: paper pulse, 0.55: 5.7e-7, 2.1e-7; Gaussian
 // pulse, 0.63: 2.5e-7, 1.7e-7; 64^2 sin^2 pulse, 0.49: 9.4e-8, 5.8e-8.
-constexpr double kGroupAngleLite = 0.25, kGroupAngleWide = 0.72;
+constexpr int kGroupLite = 0, kGroupFull = 1, kGroupWide = 2;
+constexpr double kGroupAngleLite = 0.25, kGroupAngleFull = 0.32, kGroupAngleWide = 0.72;
 constexpr int kGroupWarps = 4;  // most warps per CTA of the expanded-group kernel
 constexpr int kF64Warps = 4;    // most warps per CTA of the FP64 kernels
 constexpr int kNumGroupSizes = 3;
@@ -89,7 +91,7 @@ constexpr int kNumGroupSizes = 3;
 __host__ __device__ constexpr int group_size(int i) { return 16 >> i; }
 
 // What a run's groups come to, on the device: per group size the sums of what the
-// wide and the lite level drop (kPlanUnit fixed point, so the sum does not depend
+// full and wide (one sum) and the lite level drop (kPlanUnit fixed point, so the sum does not depend
 // on its order).
 struct GroupSums {
     unsigned long long wide[kNumGroupSizes], lite[kNumGroupSizes];
