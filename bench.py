@@ -139,17 +139,16 @@ class ClockSampler:
 # SHA-256 of the kernel source the counters were taken on; a different source
 # means the counters are stale and the traffic is reported as null.
 KERNEL_TRAFFIC = {
-    "evolve_strip_kernel": {"bytes": 95.11e6,
-                            "source_sha256": "74889d15ce1ba2e7c4751818ff356b4b99ed59e4886b167b6c79eeb474c6e413"},
+    "evolve_group_kernel": {"bytes": None, "source_sha256": ""},
 }
 
 
 def kernel_source_sha256():
-    """SHA-256 over the strip kernel's translation unit (dsp_strip.cu and the headers
-    it includes)."""
+    """SHA-256 over the expanded-group kernel's translation unit (dsp_group.cu and the
+    headers it includes)."""
     import hashlib
     h = hashlib.sha256()
-    for name in ("dsp_strip.cu", "dsp_device.cuh", "dsp_internal.h", "dsp_df.cuh"):
+    for name in ("dsp_group.cu", "dsp_device.cuh", "dsp_internal.h", "dsp_df.cuh"):
         with open(os.path.join(ROOT, "paper_1607_03062_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()
@@ -243,6 +242,14 @@ def ops_strang(dc, ds, group=1, strips=False, tdeg=0):
     return coef + tan_chain_ops(group)
 
 
+def ops_groups(steps, level, strang=False):
+    """FP32 lane instructions per spinor-step of expanded groups of `steps` steps: per
+    group 42 (level 0), 64 (1) or 76 (2) for the operator and the compensated update, 11
+    more for STRANG_XY's momentum, and the column part (9 scalar ops per lane) shared by
+    its 4 rows."""
+    return ((42, 64, 76)[level] + (11 if strang else 0) + 9 / 4.0) / steps
+
+
 def ops_fp64(dc, ds, strips=False):
     """FP64 instructions per spinor-step of the FP64 EXACT step: dt P (2) + the small parts
     m = cos(theta) - 1 and s1 = sin(theta)/theta - 1 (evaluated in double-float FP32
@@ -315,7 +322,7 @@ def run_gpu(args):
     kept = {}  # (precision, sample) -> host |c+|^2 map, for the accuracy check
     dens_by = {}  # (precision, sample) -> density
 
-    strips_seen = []
+    strips_seen, groups_seen = [], []
 
     def timed_solves(prec, warm, steps, sample_offset, keep_sample=None):
         h, state, mp = make(prec)
@@ -345,9 +352,12 @@ def run_gpu(args):
                 dens.append(B.reduce_density(h))
                 info = B.get_info(h)
                 strips_seen.append(bool(info["row_strips"]))
+                groups_seen.append(B.get_groups(h))
                 if prec == "fp64":
                     ops.append(ops_fp64(info["cos_degree"], info["sinc_degree"],
                                         bool(info["row_strips"])))
+                elif groups_seen[-1][0]:
+                    ops.append(ops_groups(*groups_seen[-1]))
                 else:
                     ops.append(ops_mixed(info["cos_degree"], info["sinc_degree"],
                                          info["group_steps"], bool(info["row_strips"]),
@@ -370,6 +380,10 @@ def run_gpu(args):
     work_per_solve = float(n) * n * nsteps
     value = work_per_solve * args.steps * world / tot
     strips_used = bool(strips_seen) and all(strips_seen)
+    # a pulse that may be expanded: the expanded-group launch and the projection come on
+    # top of the step-by-step launches, which return at once
+    expanded = bool(groups_seen) and all(g[0] > 0 for g in groups_seen)
+    groups_mixed = list(groups_seen)
 
     # ---- FP64 ----
     fp64 = None
@@ -415,9 +429,10 @@ def run_gpu(args):
         dist.all_reduce(t, op=dist.ReduceOp.MAX)
         e2e_tot = float(t.item())
     e2e = {"value": work_per_solve * args.steps * world / e2e_tot, "unit": METRIC,
-           # the FP32 pulse table the host builds and the projection nodes (hi/lo
-           # float pairs of every column and row)
-           "h2d_bytes_per_step": 8 * nsteps + 8 * (n + n),
+           # the caller's FP64 table, from which the device makes the rest, 64 bytes of
+           # zeroed sums and the projection nodes (hi/lo float pairs of every column
+           # and row); step by step the FP32 table that the host builds instead
+           "h2d_bytes_per_step": ((16 * nsteps + 64) if expanded else 8 * nsteps) + 8 * (n + n),
            "d2h_bytes_per_step": 4 * n * n + 16,
            "note": "dsp_solve_host: host midpoint table in, host |c+|^2 map (pinned) and density out"}
 
@@ -454,12 +469,13 @@ def run_gpu(args):
     peaks = load_peaks()
     # achieved = algorithmic FP32 instructions of each timed launch / its event time
     achieved = statistics.mean(o * work_per_solve / t for o, t in zip(o_mixed, t_mixed)) / 1e12
-    kernel_name = "evolve_strip_kernel" if strips_used else "evolve_mixed_kernel"
+    kernel_name = ("evolve_group_kernel" if expanded else
+                   "evolve_strip_kernel" if strips_used else "evolve_mixed_kernel")
     peak = SMS * FP32_LANES_PER_SM * SM_MAX_MHZ_NOMINAL * 1e6 / 1e12
     roof = {"bound": "alu", "achieved": achieved, "peak": peak,
             "unit": "Tinst/s (FP32 lane instructions)", "frac": achieved / peak,
             "traffic": kernel_traffic(kernel_name), "kernel": kernel_name,
-            "ops_per_spinor_step": o_mixed,
+            "ops_per_spinor_step": o_mixed, "groups": groups_mixed,
             "peak_basis": "152 SMs x 128 FP32 lanes x 2070 MHz (unit counts x max SM clock)"}
     roof["ceiling_spinor_steps_per_s"] = peak * 1e12 / statistics.mean(o_mixed)
     if clocks.get("sm_mhz"):
@@ -494,14 +510,14 @@ def run_gpu(args):
                    "samples_rotated": N_SAMPLES, "scheme": "exact midpoint exponential",
                    "l2": "flushed between steps (256 MB write)",
                    "parallelism": f"replicas x{world} (independent samples per rank)"},
-        "gpu_launches": args.steps * launches_per_solve(
-            n, strips_used, torch.cuda.get_device_properties(local).multi_processor_count),
+        "gpu_launches": args.steps * ((2 if expanded else 0) + launches_per_solve(
+            n, strips_used, torch.cuda.get_device_properties(local).multi_processor_count)),
         "e2e": e2e,
         "roofline": roof, "cpu_baseline": cpu, "clocks": clocks,
         "peaks_file": {k: peaks.get(k) for k in ("hbm_gbs", "bf16_tflops", "sm_max_mhz")},
-        "arithmetic": "FP32 spinor stored compensated (hi + lo); momentum p + A from an FP32 "
-                      "hi/lo p and one error-fed FP32 A per step; FP64 initial state; "
-                      "double-float projection; FP64 density",
+        "arithmetic": "FP32 spinor stored compensated (hi + lo); momentum p + A from FP32 "
+                      "hi/lo halves of p and of each group's sum of A; FP64 initial state; "
+                      "FP32 projection; FP64 density",
         "density_first_step": d_mixed[0] if d_mixed else None,
         "serving": serving, "small_grid": small, "magnus4": magnus, "strang_xy": strang,
         "projection": projection, "accuracy_vs_oracle": accuracy, "fp64": fp64,
@@ -526,7 +542,7 @@ def scheme_leg(args, cfgs, stream, world, rank, scheme, warm=1, reps=2):
     """The same 2048^2 x 1e5-step solves with another step scheme, FP32-mixed, in
     step groups like EXACT: the fourth-order Magnus step (two Gauss-point samples
     per step) or the sigma_x / sigma_y split.  Instructions per spinor-step from
-    ops_magnus4 / ops_strang."""
+    ops_groups, or step by step ops_magnus4 / ops_strang."""
     import torch
 
     from paper_1607_03062_gb300 import binding as B
@@ -555,7 +571,9 @@ def scheme_leg(args, cfgs, stream, world, rank, scheme, warm=1, reps=2):
         if k >= warm:
             times.append(e0.elapsed_time(e1) / 1e3)
             info = B.get_info(h)
-            ops.append(ops_fn(info["cos_degree"], info["sinc_degree"], info["group_steps"],
+            groups = B.get_groups(h)
+            ops.append(ops_groups(*groups, strang=scheme == "strang_xy") if groups[0] else
+                       ops_fn(info["cos_degree"], info["sinc_degree"], info["group_steps"],
                               bool(info["row_strips"]), info["tan_degree"]))
     B.destroy_grid(h)
     work = float(n) * n * args.time_steps

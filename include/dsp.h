@@ -290,6 +290,13 @@ typedef struct {
  * the paper has no counterpart). */
 dsp_status dsp_get_info(const dsp_grid *g, dsp_grid_info *info);
 
+/* How the current pulse's steps are taken (bookkeeping, the paper has no
+ * counterpart): *steps = 16, 8 or 4 when launches evaluate that many aligned steps
+ * at once from their expansion (see group_steps above), 0 when they go step by
+ * step; *level = 0 (the smallest pulses: fewest terms), 1 or 2 (every term, at
+ * group angles up to 0.32 and up to 0.72).  Synchronises the grid's stream. */
+dsp_status dsp_get_groups(dsp_grid *g, int32_t *steps, int32_t *level);
+
 /* Test hook for the failure path (not in the paper).  The next launch on this
  * grid announces its first A(t) chunk to the CTA's mbarrier but never copies
  * it, so every CTA's bounded wait for it runs out (after about 2 s).  The CTA

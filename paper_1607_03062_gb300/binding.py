@@ -41,7 +41,7 @@ EXPORTS = (
     "dsp_server_query", "dsp_server_cancel", "dsp_server_destroy", "dsp_density_noalloc",
     "dsp_get_info", "dsp_solve_segmented", "dsp_sample_pulse_gauss",
     "dsp_test_withhold_next_copy", "dsp_create_band", "dsp_set_keep_final_state",
-    "dsp_test_tiling", "dsp_test_expansion",
+    "dsp_test_tiling", "dsp_test_expansion", "dsp_get_groups",
 )
 
 
@@ -129,6 +129,7 @@ def lib() -> ctypes.CDLL:
                 "dsp_test_withhold_next_copy": (i32, [p]),
                 "dsp_test_tiling": (i32, [p, i32]),
                 "dsp_test_expansion": (i32, [p, i32]),
+                "dsp_get_groups": (i32, [p, pi32, pi32]),
             }
             for name, (res, args) in sig.items():
                 fn = getattr(L, name)
@@ -272,6 +273,15 @@ def get_info(h: int) -> dict:
     info = GridInfo()
     _check(lib().dsp_get_info(ctypes.c_void_p(h), ctypes.byref(info)), "get_info")
     return {n: getattr(info, n) for n, _ in GridInfo._fields_}
+
+
+def get_groups(h: int):
+    """(steps, level): the steps that the current pulse's launches evaluate at once from
+    their expansion (0: they go step by step) and the expansion's level."""
+    n, lv = ctypes.c_int32(), ctypes.c_int32()
+    _check(lib().dsp_get_groups(ctypes.c_void_p(h), ctypes.byref(n), ctypes.byref(lv)),
+           "get_groups")
+    return n.value, lv.value
 
 
 def save_state(h: int, buf: np.ndarray) -> int:

@@ -1504,6 +1504,42 @@ dsp_status dsp_test_expansion(dsp_grid *g, int32_t on)
     return DSP_OK;
 }
 
+dsp_status dsp_get_groups(dsp_grid *g, int32_t *steps, int32_t *level)
+{
+    dsp_status s = check_usable(g);
+    if (s != DSP_OK)
+        return s;
+    if (!steps || !level)
+        return DSP_E_INVALID;
+    if (!g->has_pulse)
+        return DSP_E_STATE;
+    *steps = *level = 0;
+    if (!g->by_groups)
+        return DSP_OK;
+    dsp::GroupSums sums;
+    cudaError_t e = cudaMemcpyAsync(
+        &sums, static_cast<unsigned char *>(g->groups) + GroupMemory(g).sums(), sizeof(sums),
+        cudaMemcpyDeviceToHost, g->stream);
+    if (e == cudaSuccess)
+        e = cudaStreamSynchronize(g->stream);
+    if (e != cudaSuccess)
+        return latch_cuda(g, e);
+    // the kernels' pick_plan
+    const unsigned long long budget =
+        static_cast<unsigned long long>(dsp::kPlanBudget / dsp::kPlanUnit);
+    for (int i = first_group_size(g->theta_max); i < dsp::kNumGroupSizes; ++i)
+        if (g->n_steps >= dsp::group_size(i) && sums.wide[i] <= budget) {
+            const double eps = dsp::group_size(i) * g->theta_max;
+            *steps = dsp::group_size(i);
+            *level = g->scheme != DSP_SCHEME_STRANG_XY && eps <= dsp::kGroupAngleLite &&
+                             sums.lite[i] <= budget
+                         ? dsp::kGroupLite
+                         : eps <= dsp::kGroupAngleFull ? dsp::kGroupFull : dsp::kGroupWide;
+            break;
+        }
+    return DSP_OK;
+}
+
 dsp_status dsp_get_info(const dsp_grid *g, dsp_grid_info *info)
 {
     if (!g || !info)
