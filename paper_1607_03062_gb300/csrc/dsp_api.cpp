@@ -2,9 +2,10 @@
 // handles, pulse tables, launches, the density reduction, the pulse sampler and
 // the continuous-batching server.
 //
-// The hot path runs entirely in the kernels of dsp_kernels.cu; this file only
-// validates, lays out the per-step table in the layout the kernels read, and
-// queues work on the caller's CUDA stream.
+// The hot path runs entirely in the kernels (dsp_group.cu, dsp_f64.cu, dsp_strip.cu,
+// dsp_mixed.cu, dsp_kernels.cu); this file only validates, lays out the pulse's table
+// in the layout the kernels read, picks the launches' shapes, and queues work on the
+// caller's CUDA stream.
 
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
@@ -287,7 +288,7 @@ int32_t first_group_size(double theta_max)
 
 // Layout of a grid's expanded-group memory: what one copy uploads (the caller's table
 // in FP64, the sums as zeros, the projection nodes), then the entries of every group
-// size.
+// size it may use.
 struct GroupMemory {
     size_t raw_bytes, node_bytes, entry_bytes;
     explicit GroupMemory(const dsp_grid *g)
@@ -296,7 +297,7 @@ struct GroupMemory {
                       15) & ~static_cast<size_t>(15)),
           entry_bytes(0)
     {
-        for (int i = 0; i < dsp::kNumGroupSizes; ++i)
+        for (int i = first_group_size(g->theta_max); i < dsp::kNumGroupSizes; ++i)
             entry_bytes +=
                 sizeof(dsp::GroupEntry) * static_cast<size_t>(g->n_steps / dsp::group_size(i));
     }
@@ -359,7 +360,9 @@ ReqDesc make_desc(const dsp_grid *g, int64_t begin, int64_t end, bool project, v
     r.tdeg = g->tdeg;
     r.withhold_first_copy = g->withhold_next ? 1 : 0;
     r.table_steps = g->table_cap;
-    if (g->by_groups && end > begin) {
+    // (a launch without one whole group of the smallest size has no use for them)
+    constexpr int64_t least = dsp::group_size(dsp::kNumGroupSizes - 1);
+    if (g->by_groups && (begin + least - 1) / least < end / least) {
         const GroupMemory m(g);
         r.by_groups = 1;
         const unsigned char *base = static_cast<const unsigned char *>(g->groups);
@@ -977,6 +980,18 @@ dsp_status create_grid_impl(int32_t nx, int32_t ny, double px_min, double px_max
     return DSP_OK;
 }
 
+// Whether the grid's pulse may be evaluated on expanded groups: its step groups (the
+// piece rule of dsp_evolve) allow it, a group size is within the expansion's angle, the
+// rows fill a good part of the kernel's 32 columns (below 8 columns the step-by-step
+// kernels' contiguous tiles do less work than a quarter-filled warp), and the memory
+// (67 bytes a step and less) stays small.
+bool may_expand(const dsp_grid *g)
+{
+    return g->group > 1 && g->nx >= 8 &&
+           first_group_size(g->theta_max) < dsp::kNumGroupSizes &&
+           GroupMemory(g).total() <= (static_cast<size_t>(4) << 30);
+}
+
 // Host part of setting a pulse: validates, fills the grid's pulse fields, and lays out
 // in `host` what is uploaded: for expanded groups GroupMemory's upload (the device makes
 // the per-step table from it), else the per-step table, padded to 16 bytes, and the
@@ -1006,7 +1021,7 @@ dsp_status prepare_pulse(dsp_grid *g, const double *a_mid, int64_t n_steps, doub
     g->projected = false;
     g->state_stale = false;
     // groups that the grid's piece rule allows may be evaluated expanded
-    g->by_groups = g->expand && g->group > 1 && first_group_size(tmax) < dsp::kNumGroupSizes;
+    g->by_groups = g->expand && may_expand(g);
     if (g->by_groups) {
         const GroupMemory m(g);
         host.alloc(m.upload());
@@ -1051,7 +1066,7 @@ dsp_status set_pulse_impl(dsp_grid *g, const double *a_mid, int64_t n_steps, dou
     if (s != DSP_OK)
         return s;
     cudaError_t e = cudaSuccess;
-    const size_t gbytes = staged.by_groups ? GroupMemory(&staged).total() : 0;
+    size_t gbytes = staged.by_groups ? GroupMemory(&staged).total() : 0;
     if (gbytes > g->groups_cap) {
         if (g->groups) {
             e = cudaStreamSynchronize(g->stream);  // the old groups may still be read
@@ -1063,12 +1078,23 @@ dsp_status set_pulse_impl(dsp_grid *g, const double *a_mid, int64_t n_steps, dou
         }
         if (e == cudaSuccess)
             e = cudaMalloc(&g->groups, gbytes);
-        if (e != cudaSuccess) {
+        if (e == cudaErrorMemoryAllocation) {  // no room: step by step
             cudaGetLastError();
             g->groups = nullptr;
-            return e == cudaErrorMemoryAllocation ? DSP_E_NOMEM : latch_cuda(g, e);
+            gbytes = 0;
+            staged.expand = false;
+            s = prepare_pulse(&staged, a_mid, n_steps, dt, a_in, a_out, host);
+            staged.expand = g->expand;
+            e = cudaSuccess;
+            if (s != DSP_OK)
+                return s;
+        } else if (e != cudaSuccess) {
+            cudaGetLastError();
+            g->groups = nullptr;
+            return latch_cuda(g, e);
+        } else {
+            g->groups_cap = gbytes;
         }
-        g->groups_cap = gbytes;
     }
     if (n_steps > g->table_cap) {
         if (g->table) {
@@ -1890,9 +1916,10 @@ void server_release(dsp_server *s, ServerReq *r)
 }
 
 // Allocates from the pool and queues the table upload of one request.
-dsp_status server_admit(dsp_server *s, ServerReq *r)
+dsp_status server_admit(dsp_server *s, ServerReq *r, bool expand = true)
 {
     const dsp_request &p = r->p;
+    r->g.expand = expand;
     fill_grid(&r->g, p.nx, p.ny, p.px_min, p.px_max, p.py_min, p.py_max, p.precision, p.scheme,
               p.valley, s->stream);
     HostBytes host;
@@ -1918,7 +1945,7 @@ dsp_status server_admit(dsp_server *s, ServerReq *r)
     void *block = nullptr;
     if (cudaMallocAsync(&block, total, s->copy_stream) != cudaSuccess) {
         cudaGetLastError();
-        return DSP_E_NOMEM;
+        return by_groups ? server_admit(s, r, false) : DSP_E_NOMEM;
     }
     unsigned char *b = static_cast<unsigned char *>(block);
     r->block = block;

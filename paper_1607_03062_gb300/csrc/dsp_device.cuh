@@ -1,8 +1,9 @@
 // dsp_device.cuh -- device code shared by the kernels of the split-operator
 // massless-Dirac solver (sm_103a; not installed).  The kernels themselves are in
-// dsp_mixed.cu (FP32_MIXED, contiguous tiles), dsp_strip.cu (FP32_MIXED, row
-// strips) and dsp_kernels.cu (FP64, projection, density, time segments), compiled
-// as separate translation units.
+// dsp_group.cu (FP32_MIXED, expanded step groups), dsp_mixed.cu and dsp_strip.cu
+// (FP32_MIXED step by step, contiguous tiles and row strips), dsp_f64.cu (FP64) and
+// dsp_kernels.cu (projection, density, time segments), compiled as separate
+// translation units.
 //
 // Method (arXiv 1607.03062):
 //   Sec. II Eq. (free_spin1..4)  initial state v(p + A_in), normalised;
@@ -12,31 +13,29 @@
 //                                theta = dt |P_n|;
 //   Sec. II Eq. (pair_prod_homo) |c+|^2 = |u(p + A_out)^dag psi|^2, summed to n.
 //
-// GB300 design (one CTA = one tile of 1024 momenta; FP32-mixed: 256 threads x 4
-// spinors, FP64: 512 threads x 2 spinors):
+// GB300 design:
 //   * the spinors stay in registers across all steps of a launch: one 16-byte
 //     read and one write per spinor plane per launch;
-//   * A(t) is staged in shared memory in 16 KB chunks (2048 FP32_MIXED steps,
-//     1024 FP64 ones) by 1-D bulk copies (cp.async.bulk) completing on an
-//     mbarrier, double buffered, so the step loop reads each entry with one
-//     broadcast shared-memory load;
+//   * tiles are as small as one warp (32 columns x 1 to 4 rows; FP64 also 8 to 32
+//     points) where the kernel shares nothing across warps, so that a launch is
+//     shaped by the load of the chip's schedulers;
+//   * the pulse's table or group coefficients are staged in shared memory by 1-D bulk
+//     copies (cp.async.bulk) completing on an mbarrier, double buffered, so the step
+//     loop reads each entry with a broadcast shared-memory load;
 //   * cos(theta) - 1 and sin(theta)/theta are evaluated as their Taylor series
 //     in x = theta^2 = |dt P|^2 (no square root, no sin/cos call): the degree is
 //     chosen per request on the host from theta_max so truncation stays below
 //     the working precision;
-//   * FP32_MIXED: dt*p is split into hi + lo (two floats, the momentum of every
-//     point to ~1e-16 relative), dt*A(t_n) is one float per step, and
-//     P_n = p_hi + (A_n + p_lo): the FP32 roundings of P then change from step
-//     to step with A instead of shifting every step's momentum by the same
-//     amount, and the first one is at A's scale, not P's;
+//   * FP32_MIXED: momenta and potentials enter as hi + lo pairs of floats (step by
+//     step: dt*A(t_n) as one float per step and P_n = p_hi + (A_n + p_lo), whose FP32
+//     roundings change from step to step with A);
 //   * FP32_MIXED: the spinor is stored as hi + lo and each update adds the
 //     increment (U - I) psi with a Fast2Sum, so the FP32 rounding of psi does not
-//     random-walk over 1e5 steps; every scheme multiplies 2 to 16 steps into one
-//     SU(2) matrix first, so the compensated update is paid once per group, and
-//     two momenta share each packed FP32x2 instruction;
-//   * the projection and the per-tile partial sums of |c+|^2 are fused into the
-//     last launch; partial sums use a fixed pairwise tree, so the density is
-//     bitwise reproducible and independent of the batch a request ran in.
+//     random-walk over 1e5 steps; up to 16 steps are one SU(2) matrix, from the
+//     expansion of their product or multiplied out, so the compensated update is
+//     paid once per group, and two momenta share each packed FP32x2 instruction;
+//   * partial sums of |c+|^2 use a fixed pairwise tree, so the density is bitwise
+//     reproducible and independent of the tiling and of the batch a request ran in.
 // No tensor cores: the work is 2x2 complex arithmetic per momentum.
 
 #pragma once
@@ -503,11 +502,11 @@ __device__ __forceinline__ bool table_range_ok(const ReqDesc &R, int64_t first, 
 #endif
 }
 
-// Entries of all group sizes before size i (kNumGroupSizes: all of them).
-__host__ __device__ __forceinline__ int64_t group_entries_before(int64_t n_steps, int i)
+// Entries of the group sizes first ... i - 1, which lie before size i's.
+__device__ __forceinline__ int64_t group_entries_before(int64_t n_steps, int first, int i)
 {
     int64_t n = 0;
-    for (int k = 0; k < i; ++k)
+    for (int k = first; k < i; ++k)
         n += n_steps / group_size(k);
     return n;
 }

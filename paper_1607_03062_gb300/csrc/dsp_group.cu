@@ -1,5 +1,5 @@
-// dsp_group.cu -- the FP32_MIXED evolve kernel on expanded step groups, and the kernel that expands a pulse's groups.  Shared device code is in
-// dsp_device.cuh.
+// dsp_group.cu -- the FP32_MIXED evolve kernel on expanded step groups, and the kernel
+// that expands a pulse's groups.  Shared device code is in dsp_device.cuh.
 
 #include "dsp_device.cuh"
 
@@ -19,9 +19,9 @@ namespace {
 //   w_xy = S + (S_y, -S_x) (S x u2 + x S x u4) + K S
 // (GroupEntry).  A STRANG_XY step is exp(-i sigma.P') with P' = P + cubic(P) in closed
 // series, so its groups are those of P': the same w with the cubic and fifth-order terms
-// of P' added to w_xy and their part of S x m1 to w_z (group_step).  What the expansion drops is summed over the run (GroupSums); the
-// kernels pick G and the level from the sums (pick_plan), and where no G passes the
-// step-by-step chains (dsp_strip.cu, dsp_mixed.cu), queued behind, take the run.
+// of P' added to w_xy and their part of S x m1 to w_z (group_step).  What the
+// expansion drops is summed over the run (GroupSums); the kernels pick G and the level
+// from the sums (pick_plan), and where no G passes the step-by-step chains (dsp_strip.cu, dsp_mixed.cu), queued behind, take the run.
 //
 // S comes as hi + lo (each from an exact sum of the hi/lo halves of G dt p and of
 // the group's sum of dt A), so no step's momentum is rounded on the way.  Three levels:
@@ -34,7 +34,8 @@ namespace {
 //
 // What bounds it: FP32 issue.  Per spinor and group 42 (lite), 64 (full) or 76 (wide)
 // lane operations plus a column part shared by the warp's rows, against 9 and more per
-// spinor and STEP of the chains.
+// spinor and STEP of the chains.  FMA pipe 88% busy (lite; packed instructions hold it
+// two cycles), issue 50%, DRAM idle.
 //
 // Tiles: one warp owns 32 columns x H rows (H = 4, 2: packed FP32x2 row pairs; H =
 // 1: scalar), any nx (columns past the row's end idle), and works alone: its own
@@ -45,11 +46,12 @@ namespace {
 // The projection is the projection kernel's, on the state this kernel leaves.
 //
 // Measured (GB300, whole solves, step by step -> expanded): 2048^2 x 1e5 sin^2 pulse
-// 209.2 -> 35.5 ms (lite, G = 16); 1024^2 x 3e4 Gaussian pulse 22.6 -> 5.1 ms (wide,
-// 16); 1000 x 750 x 2e4 two colours 10.36 -> 2.48 ms (wide, 16; contiguous tiles
-// before); 512^2 x 12000 MAGNUS4 3.14 -> 0.70 ms; 256^2 x 2e4 paper pulse 1.42 ->
-// 0.40 ms; 512 x 384 x 12000 STRANG_XY 1.79 -> 0.63 ms.  2-norm error of |c+|^2 against 64 bits on the last four: 3.7e-7 -> 2.3e-7,
-// 2.1e-7 -> 1.2e-7, 5.0e-7 -> 2.3e-7, 2.9e-7 -> 1.1e-7.
+// 209.2 -> 35.2 ms (lite, G = 16); 1024^2 x 3e4 Gaussian pulse 22.6 -> 5.03 ms (wide,
+// 16); 1000 x 750 x 2e4 two colours 10.36 -> 2.46 ms (wide, 16; contiguous tiles
+// before); 512^2 x 12000 MAGNUS4 3.14 -> 0.575 ms (full); 256^2 x 2e4 paper pulse 1.42
+// -> 0.375 ms; 512 x 384 x 12000 STRANG_XY 1.79 -> 0.55 ms (full).  2-norm error of
+// |c+|^2 against 64 bits on the last four: 3.7e-7 -> 2.3e-7, 2.0e-7 -> 1.3e-7, 5.0e-7
+// -> 2.3e-7, 2.8e-7 -> 1.2e-7.
 // ---------------------------------------------------------------------------
 
 constexpr int kGrpChunk = 32;  // group entries per staged chunk: one per lane
@@ -427,7 +429,7 @@ __device__ void body_group(const ReqDesc &R, int size, int tile, WarpSmem &sm, i
     const int64_t head_end = g1 > g0 ? g0 * G : R.step_end;
     const int nchunks = static_cast<int>((g1 - g0 + kGrpChunk - 1) / kGrpChunk);
     const GroupEntry *entries =
-        R.groups.entries + group_entries_before(R.groups.n_steps, size) + g0;
+        R.groups.entries + group_entries_before(R.groups.n_steps, R.groups.first, size) + g0;
     const auto chunk_len = [&](int c) {
         const int64_t rem = g1 - g0 - static_cast<int64_t>(c) * kGrpChunk;
         return rem < kGrpChunk ? static_cast<int>(rem) : kGrpChunk;
@@ -748,7 +750,7 @@ __device__ __forceinline__ void expand_group(const PrepArgs &args, int64_t g, fl
            0.5f * wz * wz;
     const float xh = static_cast<float>(sx), yh = static_cast<float>(sy);
     float4 *e = reinterpret_cast<float4 *>(
-        args.entries + group_entries_before(args.n_steps, I) + g);
+        args.entries + group_entries_before(args.n_steps, args.first, I) + g);
     e[0] = make_float4(xh, static_cast<float>(sx - static_cast<double>(xh)), n1.y, n3.y);
     e[1] = make_float4(n5.y, u2.y, u4.y, Kxx);
     e[2] = make_float4(Kyx, yh, static_cast<float>(sy - static_cast<double>(yh)), C);

@@ -17,8 +17,8 @@ constexpr int kStripHeight = 4;
 // Points per density partial sum (a granule: point index / kGranule); every CTA
 // shape covers whole granules.
 constexpr int kGranule = 256;
-// Requests one evolve launch can carry in its parameter block (96 x 280 bytes:
-// within the 32 KB kernel-parameter limit).
+// Requests one evolve launch can carry in its parameter block (within the 32 KB
+// kernel-parameter limit, asserted below).
 constexpr int kMaxReqPerLaunch = 96;
 // Device-side error bits (the launch's error word).
 constexpr int kErrTimeout = 1;
@@ -91,8 +91,8 @@ constexpr int kNumGroupSizes = 3;
 __host__ __device__ constexpr int group_size(int i) { return 16 >> i; }
 
 // What a run's groups come to, on the device: per group size the sums of what the
-// full and wide (one sum) and the lite level drop (kPlanUnit fixed point, so the sum does not depend
-// on its order).
+// full and wide (one sum) and the lite level drop (kPlanUnit fixed point, so the sum
+// does not depend on its order).
 struct GroupSums {
     unsigned long long wide[kNumGroupSizes], lite[kNumGroupSizes];
 };
@@ -101,8 +101,8 @@ constexpr double kPlanUnit = 0x1p-50;
 // FP32_MIXED's target is 1e-5 per point.
 constexpr double kPlanBudget = 4e-6;
 
-// The groups of a pulse: entries of each size, one size after the other, and the
-// sums.  The kernels pick the largest size whose sum is in the budget (pick_plan),
+// The groups of a pulse: entries of each size from `first` on, one after the other, and
+// the sums.  The kernels pick the largest size whose sum is in the budget (pick_plan),
 // or none: then the run goes step by step.
 struct GroupTable {
     const GroupEntry *entries;
@@ -145,10 +145,12 @@ struct ReqDesc {
     int64_t step_begin, step_end;  // table entries [step_begin, step_end) this launch
     int32_t nx, ny;
     int32_t row0;     // global row index of the grid's first row (row bands; 0 otherwise)
-    int32_t store_state;  // 1: write the spinor state back at the end of the launch
+    int32_t store_state;  // 1: write the spinor state back at the end of the launch (always
+                          // by the FP64 and expanded-group kernels)
     int32_t scheme, valley, level;
     int32_t fresh;    // 1: start from v(p + A_in) instead of reading the state
-    int32_t project;  // 1: project at the end (map + partials)
+    int32_t project;  // 1: project at the end (map + partials; in the evolve launch itself
+                      // only step by step in FP32_MIXED)
     int32_t tile_begin;  // first CTA of this request in the launch
     int32_t n_tiles;
     int32_t init_identity;  // with fresh: start from the column (1, 0) of the identity
