@@ -54,10 +54,11 @@ typedef int32_t dsp_status;
                               built with -DDSP_BOUNDS_CHECK (accesses are skipped) */
 
 /* Arithmetic of the evolution. */
-#define DSP_FP64 0       /* the spinor and its update in FP64; in the EXACT scheme the
-                            small parts cos(theta) - 1 and sin(theta)/theta - 1 are
-                            evaluated in double-float FP32 arithmetic (~1e-19
-                            absolute, below an FP64 ulp of the state)               */
+#define DSP_FP64 0       /* the spinor and its update in FP64; the small parts
+                            cos(theta) - 1 and sin(theta)/theta - 1 are evaluated in
+                            double-float FP32 arithmetic (~1e-19 absolute, below an
+                            FP64 ulp of the state; STRANG_XY and MAGNUS4 at theta
+                            above ~0.2 in FP64)                                     */
 #define DSP_FP32_MIXED 1 /* spinor in compensated FP32 (hi + lo); dt P_n formed as
                             dt p_hi + (dt A_n + dt p_lo) with dt p an FP32 hi/lo
                             pair and dt A_n one FP32 per step, rounded on the host
@@ -117,10 +118,11 @@ dsp_status dsp_create_band(int32_t nx, int32_t ny, int32_t row_begin, int32_t ro
                            void *state_dev, int64_t state_dev_bytes, dsp_grid **out);
 
 /* keep = 1 (the default): every launch leaves the spinor state in device
- * memory.  keep = 0: the launch that takes the last step and projects in the
- * same kernel (dsp_solve, dsp_solve_host) does not write the final state back,
- * saving 32 bytes of HBM writes per point when only the map and the density
- * are wanted.  The final state is then gone: dsp_project, dsp_solve and
+ * memory.  keep = 0: a step-by-step FP32_MIXED launch that takes the last step and
+ * projects in the same kernel (dsp_solve, dsp_solve_host) does not write the final
+ * state back, saving 32 bytes of HBM writes per point when only the map and the
+ * density are wanted (FP64 and expanded groups project from the state and need it).
+ * The final state is then gone, whatever the kernel: dsp_project, dsp_solve and
  * dsp_save_state return DSP_E_STATE until the next dsp_set_pulse or
  * dsp_load_state.  The map and the density are bitwise the same either way.
  * Not in the paper (a memory-traffic option). */
@@ -159,8 +161,8 @@ dsp_status dsp_evolve(dsp_grid *g, int64_t steps);
  * DSP_FP64 evaluates |c+|^2 in double-float arithmetic (pairs of FP32, about
  * 48 bits, ~1e-14 absolute); DSP_FP32_MIXED in FP32 from the hi parts of the
  * state (error below ~4e-7 |c+|, the size of the float map's own rounding).
- * Either way it is the same code as the projection fused into the last evolve
- * launch, so the two give the same bits.  A projection of
+ * Either way it is the same code as the projection of dsp_solve, so the two give
+ * the same bits.  A projection of
  * a state already on the device reads it (32 bytes per point) without writing
  * it back and writes the map (4 or 8 bytes per point).  Asynchronous. */
 dsp_status dsp_project(dsp_grid *g, void *map_dev);
@@ -205,7 +207,7 @@ dsp_status dsp_density_noalloc(const void *map_dev, int32_t precision, int32_t n
                                void *cuda_stream, double *n_host);
 
 /* The whole hot path in one call: evolves the remaining steps (Sec. III, Eq.
- * (ev_op_dt)) with the projection fused into the same kernel, writes map_dev
+ * (ev_op_dt)), projects behind the last step, writes map_dev
  * (may be NULL: then an internal map is used) and the density (Sec. II, Eq.
  * (pair_prod_homo)) to *n_host (may be NULL).  Synchronises when n_host is
  * not NULL. */
@@ -377,7 +379,7 @@ dsp_status dsp_sample_pulse_gauss(const dsp_pulse_spec *spec, int64_t n_steps, d
  * (each a whole solve) are queued on submit and admitted FIFO while the device
  * footprint fits the budget and a slot is free; every dsp_server_step advances
  * all admitted requests by up to chunk_steps in ONE batched launch, retires
- * the ones that finished (projection fused, density reduced, map copied to
+ * the ones that finished (projected, density reduced, map copied to
  * the server's host buffer) and admits more.  A request's result is bitwise
  * the same alone or in any mix.                                              */
 /* ------------------------------------------------------------------------- */

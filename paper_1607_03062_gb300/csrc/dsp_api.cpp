@@ -552,8 +552,8 @@ cudaError_t launch_groups(const std::vector<ReqDesc> &reqs, cudaStream_t stream)
 
 // Shape of an FP64 launch (launch_evolve_f64's lanes) by the FP64 instructions of its
 // fullest scheduler (dsp_f64.cu): per warp and step 65 for 4 rows x 32 columns, 18, 9
-// or 6 flat on 1, 2 or 4 lanes per point (EXACT); STRANG_XY ~70 and 36, whose series
-// are FP64 and shared along rows and columns.
+// or 6 flat on 1, 2 or 4 lanes per point (EXACT); STRANG_XY 62 and 24, whose small parts
+// belong to one coordinate each and are shared along rows and columns.
 int f64_lanes(const std::vector<ReqDesc> &reqs, int scheme)
 {
     if (scheme == DSP_SCHEME_MAGNUS4)
@@ -562,7 +562,7 @@ int f64_lanes(const std::vector<ReqDesc> &reqs, int scheme)
         int lanes;
         double exact, strang;
     };
-    constexpr Shape shapes[4] = {{0, 65.0, 70.0}, {1, 18.0, 36.0}, {2, 9.0, 0.0}, {4, 6.0, 0.0}};
+    constexpr Shape shapes[4] = {{0, 65.0, 62.0}, {1, 18.0, 24.0}, {2, 9.0, 0.0}, {4, 6.0, 0.0}};
     int best = 0;
     double best_t = 0.0;
     for (const Shape &sh : shapes) {

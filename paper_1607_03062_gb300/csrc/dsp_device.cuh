@@ -174,29 +174,6 @@ __host__ __device__ constexpr double inv_factorial()
         return inv_factorial<N - 1>() / static_cast<double>(N);
 }
 
-// Horner tail sum_{k=K..D} c_k x^(k-K) with c_k = (-1)^k / (2k + ODD)!; every
-// coefficient is a compile-time constant rounded once to T.
-template <typename T, int D, int K, int ODD>
-__device__ __forceinline__ T horner(T x)
-{
-    constexpr T c = static_cast<T>(((K & 1) ? -1.0 : 1.0) * inv_factorial<2 * K + ODD>());
-    if constexpr (K == D)
-        return c;
-    else
-        return fma(horner<T, D, K + 1, ODD>(x), x, c);
-}
-
-template <int D>
-__device__ __forceinline__ double cos_f64(double x)
-{
-    return horner<double, D, 0, 0>(x);
-}
-template <int D>
-__device__ __forceinline__ double sinc_f64(double x)
-{
-    return horner<double, D, 0, 1>(x);
-}
-
 // ---------------------------------------------------------------------------
 // Per-point set-up shared by both precisions (all FP64, once per launch)
 // ---------------------------------------------------------------------------

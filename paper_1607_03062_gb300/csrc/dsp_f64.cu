@@ -79,6 +79,63 @@ __device__ __forceinline__ void step_f64_exact(F64Point &s, double Px, double Py
     s.ar = nar; s.ai = nai; s.br = nbr; s.bi = nbi;
 }
 
+// sum_{k=K..D} c_k x^(k-K), c_k = (-1)^k / (2k + ODD)!, in FP64.
+template <int D, int K, int ODD>
+__device__ __forceinline__ double horner_f64(double x)
+{
+    constexpr double c = ((K & 1) ? -1.0 : 1.0) * inv_factorial<2 * K + ODD>();
+    if constexpr (K == D)
+        return c;
+    else
+        return fma(horner_f64<D, K + 1, ODD>(x), x, c);
+}
+
+// STRANG_XY and MAGNUS4 form their small parts in double-float up to this cosine
+// degree (theta below ~0.2, where their ~2^-46 relative error is below an FP64 ulp of
+// the state), in FP64 above.
+constexpr int kDfDegree = 5;
+
+// The FP64 MAGNUS4 step in the same way: n = (dt Pbar, n_z), n_z = Pbar x D, |n|^2 and
+// the small parts in double-float (kDfDegree), the update and q in FP64.  26 FP64
+// operations where the FP64 series took 26 + dc + ds.
+template <int DC, int DS>
+__device__ __forceinline__ void step_f64_magnus(F64Point &s, double Px, double Py, double2 d)
+{
+    const double nz = fma(Px, d.y, -(Py * d.x));
+    double c, qr, qi, qz;
+    if constexpr (DC <= kDfDegree) {
+        const float2 px2 = square_df(Px), py2 = square_df(Py), nz2 = square_df(nz);
+        float xh = px2.x, xl = px2.y;
+        df_add(xh, xl, py2.x, py2.y);
+        df_add(xh, xl, nz2.x, nz2.y);  // |n|^2
+        float th, tl, uh, ul;
+        horner_df<DC, 1, 0>(xh, xl, th, tl);
+        df_mul(xh, xl, th, tl, uh, ul);
+        c = 1.0 + df_to_f64(uh, ul);
+        horner_df<DS, 1, 1>(xh, xl, th, tl);
+        df_mul(xh, xl, th, tl, uh, ul);
+        const double s1 = df_to_f64(uh, ul);
+        qr = fma(s1, Py, Py);
+        qi = fma(s1, Px, Px);
+        qz = fma(s1, nz, nz);
+    } else {
+        const double x = fma(Px, Px, fma(Py, Py, nz * nz));
+        c = horner_f64<DC, 0, 0>(x);
+        const double sn = horner_f64<DS, 0, 1>(x);
+        qr = sn * Py;
+        qi = sn * Px;
+        qz = sn * nz;
+    }
+    // a' = (c - i qz) a - q b ; b' = conj(q) a + (c + i qz) b, q = qr + i qi: the small
+    // terms first, one rounding at the state's size (from psi + m psi each term would
+    // round there: 1.2 to 1.6 times the error over 12000 and 50000 steps)
+    const double nar = fma(c, s.ar, fma(qz, s.ai, fma(-qr, s.br, qi * s.bi)));
+    const double nai = fma(c, s.ai, fma(-qz, s.ar, fma(-qr, s.bi, -(qi * s.br))));
+    const double nbr = fma(c, s.br, fma(-qz, s.bi, fma(qr, s.ar, qi * s.ai)));
+    const double nbi = fma(c, s.bi, fma(qz, s.br, fma(qr, s.ai, -(qi * s.ar))));
+    s.ar = nar; s.ai = nai; s.br = nbr; s.bi = nbi;
+}
+
 // psi <- U psi for U = [[c, -q], [conj(q), c]] (STRANG_XY), in FP64.
 __device__ __forceinline__ void apply_f64(F64Point &s, double c, double qr, double qi)
 {
@@ -89,45 +146,48 @@ __device__ __forceinline__ void apply_f64(F64Point &s, double c, double qr, doub
     s.ar = nar; s.ai = nai; s.br = nbr; s.bi = nbi;
 }
 
+// STRANG_XY's parts of one coordinate: {cos P, sin P} (the small parts by kDfDegree);
+// and its step from those of x and y, c = cos y cos x, q = sin y + i cos y sin x.  24
+// FP64 operations where the FP64 series took 20 + 2 dc + 2 ds; on row tiles the parts
+// of a row and of a column are formed once.
+template <int DC, int DS>
+__device__ __forceinline__ double2 strang_part(double P)
+{
+    if constexpr (DC <= kDfDegree) {
+        const float2 x = square_df(P);
+        float th, tl, uh, ul;
+        horner_df<DC, 1, 0>(x.x, x.y, th, tl);
+        df_mul(x.x, x.y, th, tl, uh, ul);
+        const double c1 = df_to_f64(uh, ul);
+        horner_df<DS, 1, 1>(x.x, x.y, th, tl);
+        df_mul(x.x, x.y, th, tl, uh, ul);
+        return make_double2(1.0 + c1, fma(df_to_f64(uh, ul), P, P));
+    } else {
+        const double x = P * P;
+        return make_double2(horner_f64<DC, 0, 0>(x), P * horner_f64<DS, 0, 1>(x));
+    }
+}
+__device__ __forceinline__ void step_f64_strang(F64Point &s, double2 x, double2 y)
+{
+    apply_f64(s, y.x * x.x, y.y, y.x * x.y);
+}
+
 template <int SCHEME, int DC, int DS>
 __device__ __forceinline__ void step_f64(F64Point &s, double2 a, double2 d)
 {
     const double Px = s.tx + a.x, Py = s.ty + a.y;  // dt * P (times the valley sign)
     if constexpr (SCHEME == 0) {
         step_f64_exact<DC, DS>(s, Px, Py, square_df(Px), square_df(Py));
-        return;
-    }
-    double c, qr, qi, qz = 0.0;
-    if constexpr (SCHEME == 1) {
-        const double xx = Px * Px, xy = Py * Py;
-        const double cy = cos_f64<DC>(xy);
-        c = cy * cos_f64<DC>(xx);
-        qr = Py * sinc_f64<DS>(xy);
-        qi = cy * (Px * sinc_f64<DS>(xx));
+    } else if constexpr (SCHEME == 2) {
+        step_f64_magnus<DC, DS>(s, Px, Py, d);
     } else {
-        const double nz = fma(Px, d.y, -(Py * d.x));  // see step_coeffs_f32
-        const double x = fma(Px, Px, fma(Py, Py, nz * nz));
-        c = cos_f64<DC>(x);
-        const double sn = sinc_f64<DS>(x);
-        qr = sn * Py;
-        qi = sn * Px;
-        qz = sn * nz;
-    }
-    // a' = (c - i qz) a - q b ; b' = conj(q) a + (c + i qz) b, q = qr + i qi
-    if constexpr (SCHEME == 2) {
-        const double nar = fma(c, s.ar, fma(qz, s.ai, fma(-qr, s.br, qi * s.bi)));
-        const double nai = fma(c, s.ai, fma(-qz, s.ar, fma(-qr, s.bi, -(qi * s.br))));
-        const double nbr = fma(c, s.br, fma(-qz, s.bi, fma(qr, s.ar, qi * s.ai)));
-        const double nbi = fma(c, s.bi, fma(qz, s.br, fma(qr, s.ai, -(qi * s.ar))));
-        s.ar = nar; s.ai = nai; s.br = nbr; s.bi = nbi;
-    } else {
-        apply_f64(s, c, qr, qi);
+        step_f64_strang(s, strang_part<DC, DS>(Px), strang_part<DC, DS>(Py));
     }
 }
 
 // The row part of a step from dt P_y, as step_f64 forms it:
 //   EXACT {P_y, (P_y^2 as a float pair, in the second double's bits)};
-//   STRANG_XY {cos(P_y), P_y * sinc(P_y)} (b = dt P_y).
+//   STRANG_XY strang_part.
 template <int SCHEME, int DC, int DS>
 __device__ __forceinline__ double2 strip64_row(double Py)
 {
@@ -137,8 +197,7 @@ __device__ __forceinline__ double2 strip64_row(double Py)
             (static_cast<unsigned long long>(__float_as_uint(p2.y)) << 32) | __float_as_uint(p2.x);
         return make_double2(Py, __longlong_as_double(static_cast<long long>(bits)));
     } else {
-        const double xy = Py * Py;
-        return make_double2(cos_f64<DC>(xy), Py * sinc_f64<DS>(xy));
+        return strang_part<DC, DS>(Py);
     }
 }
 
@@ -161,15 +220,10 @@ __device__ __forceinline__ void strip64_step(F64Point (&pt)[H], double tx, doubl
         }
         return;
     }
-    // STRANG_XY: the column's cos(dt P_x) and dt P_x sinc(dt P_x), then per row
-    const double xx = Px * Px;
-    const double cxx = cos_f64<DC>(xx);
-    const double sxx = Px * sinc_f64<DS>(xx);
+    const double2 x = strang_part<DC, DS>(Px);
 #pragma unroll
-    for (int k = 0; k < H; ++k) {
-        const double2 r = rows[k];
-        apply_f64(pt[k], r.x * cxx, r.y, r.x * sxx);
-    }
+    for (int k = 0; k < H; ++k)
+        step_f64_strang(pt[k], x, rows[k]);
 }
 
 // ---------------------------------------------------------------------------
@@ -189,13 +243,14 @@ __device__ __forceinline__ void strip64_step(F64Point (&pt)[H], double tx, doubl
 //          each forms one of P_x and P_y, of the two series, and of the two parts of
 //          q, and they trade by shuffles                                  9 for 16
 //   flat 4 8 points, a lane per real component                            6 for 8
-// Every FP64 operation of a point is the same in every shape (same operands, same
+// (STRANG_XY: rows 62, flat 24; MAGNUS4: flat 26.)  Every FP64 operation of a point is the same in every shape (same operands, same
 // rounding), so its result is bitwise the same.  STRANG_XY takes rows or flat 1,
 // MAGNUS4 flat 1.  The projection is the projection kernel's, on the state these
 // leave.
 //
 // Measured: 64^2 x 2000 steps 9.48 -> 1.08 ms (1024-point CTAs held 4 of 152 SMs;
-// flat 4 holds 512 warps), 300 x 257 x 1700 steps 8.10 -> 4.20 ms.
+// flat 4 holds 512 warps), 300 x 257 x 1700 steps 8.10 -> 4.20 ms; 1000 steps of 512^2:
+// MAGNUS4 19.8 -> 12.4 ms, STRANG_XY 9.48 -> 8.50 ms.
 // ---------------------------------------------------------------------------
 
 constexpr int kF64Stage = 1024;  // bytes per staged table chunk and warp

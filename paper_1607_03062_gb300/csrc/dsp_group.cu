@@ -34,7 +34,7 @@ namespace {
 //
 // What bounds it: FP32 issue.  Per spinor and group 42 (lite), 64 (full) or 76 (wide)
 // lane operations plus a column part shared by the warp's rows, against 9 and more per
-// spinor and STEP of the chains.  FMA pipe 88% busy (lite; packed instructions hold it
+// spinor and STEP of the chains.  FMA pipe 83% busy (lite; packed instructions hold it
 // two cycles), issue 50%, DRAM idle.
 //
 // Tiles: one warp owns 32 columns x H rows (H = 4, 2: packed FP32x2 row pairs; H =
