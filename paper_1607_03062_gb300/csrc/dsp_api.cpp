@@ -550,38 +550,45 @@ cudaError_t launch_groups(const std::vector<ReqDesc> &reqs, cudaStream_t stream)
     return cudaSuccess;
 }
 
-// Shape of an FP64 launch (launch_evolve_f64's lanes) by the FP64 instructions of its
-// fullest scheduler (dsp_f64.cu): per warp and step 65 for 4 rows x 32 columns, 18, 9
-// or 6 flat on 1, 2 or 4 lanes per point (EXACT); STRANG_XY 62 and 24, whose small parts
-// belong to one coordinate each and are shared along rows and columns.
+// Tiles of an FP64 request (launch_evolve_f64's lanes).
+int64_t f64_tiles(const ReqDesc &r, int lanes)
+{
+    return lanes == 0 ? row_tiles(r, 4) : (r.n_points + 32 / lanes - 1) / (32 / lanes);
+}
+
+// Shape of an FP64 launch (launch_evolve_f64's lanes) by the FP64 work of its fullest
+// scheduler (dsp_f64.cu), in units of 33 ns per step: 32 points flat, 4 rows x 32 columns
+// (EXACT, STRANG_XY), or 8 points on a warp pair.  `cost` is a tile's share of a busy
+// scheduler, its FP64 instructions and, for pairs, the waits between the two warps;
+// `alone` what a step takes when a scheduler has one tile, whose operators then wait for
+// its own updates.  Both measured, on grids of 16^2 to 512^2: EXACT flat at 0.8 and 2.5
+// tiles a scheduler 27.6 and 18.1, rows 93 and 64.7, pairs 6.1 and 4.8.
 int f64_lanes(const std::vector<ReqDesc> &reqs, int scheme)
 {
-    if (scheme == DSP_SCHEME_MAGNUS4)
-        return 1;
     struct Shape {
         int lanes;
-        double exact, strang;
+        double cost[3], alone[3];  // EXACT, STRANG_XY, MAGNUS4 (0: no such kernel)
     };
-    constexpr Shape shapes[4] = {{0, 65.0, 62.0}, {1, 18.0, 24.0}, {2, 9.0, 0.0}, {4, 6.0, 0.0}};
-    int best = 0;
+    constexpr Shape shapes[3] = {{1, {18.2, 24.2, 26.2}, {27.5, 39.0, 38.5}},
+                                 {0, {65.0, 62.0, 0.0}, {93.0, 72.0, 0.0}},
+                                 {4, {4.8, 7.0, 6.9}, {6.0, 10.0, 9.0}}};
+    int best = 1;
     double best_t = 0.0;
     for (const Shape &sh : shapes) {
-        const double cost = scheme == DSP_SCHEME_EXACT ? sh.exact : sh.strang;
-        if (cost == 0.0)
+        if (sh.cost[scheme] == 0.0)
             continue;
-        int64_t warps = 0;
+        int64_t tiles = 0;
         for (const ReqDesc &r : reqs)
-            warps += sh.lanes == 0 ? row_tiles(r, 4)
-                                   : (r.n_points + 32 / sh.lanes - 1) / (32 / sh.lanes);
-        const double t = launch_time(warps, cost);
-        if (sh.lanes == 0 || t < 0.98 * best_t) {
+            tiles += f64_tiles(r, sh.lanes);
+        const double t = std::max(sh.alone[scheme], launch_time(tiles, sh.cost[scheme]));
+        if (sh.lanes == 1 || t < 0.99 * best_t) {
             best = sh.lanes;
             best_t = t;
         }
     }
     for (const ReqDesc &r : reqs)
         if (r.rows > 0)
-            best = r.rows == 4 ? 0 : 1;
+            best = r.rows == 4 && scheme != DSP_SCHEME_MAGNUS4 ? 0 : 1;
     return best;
 }
 
@@ -596,9 +603,7 @@ cudaError_t launch_f64(const std::vector<ReqDesc> &reqs, cudaStream_t stream)
                 sel.push_back(r);
         const int lanes = f64_lanes(sel, scheme);
         for (size_t i = 0; i < sel.size();) {
-            i = fill_launch(sel, i, *a, [&](const ReqDesc &r) {
-                return lanes == 0 ? row_tiles(r, 4) : (r.n_points + 32 / lanes - 1) / (32 / lanes);
-            });
+            i = fill_launch(sel, i, *a, [&](const ReqDesc &r) { return f64_tiles(r, lanes); });
             const cudaError_t e = dsp::launch_evolve_f64(
                 *a, lanes, warps_per_cta(a->total_tiles, dsp::kF64Warps), stream);
             if (e != cudaSuccess)

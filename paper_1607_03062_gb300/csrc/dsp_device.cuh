@@ -16,8 +16,8 @@
 // GB300 design:
 //   * the spinors stay in registers across all steps of a launch: one 16-byte
 //     read and one write per spinor plane per launch;
-//   * tiles are as small as one warp (32 columns x 1 to 4 rows; FP64 also 8 to 32
-//     points) where the kernel shares nothing across warps, so that a launch is
+//   * tiles are as small as one warp (32 columns x 1 to 4 rows; FP64 also 32
+//     points, or 8 on a pair of warps) where the kernel shares nothing across warps, so that a launch is
 //     shaped by the load of the chip's schedulers;
 //   * the pulse's table or group coefficients are staged in shared memory by 1-D bulk
 //     copies (cp.async.bulk) completing on an mbarrier, double buffered, so the step
@@ -76,6 +76,11 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t by
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)),
                  "r"(bytes)
                  : "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
 
 // Global -> shared bulk copy; dst, src 16-byte aligned, bytes a multiple of 16.

@@ -57,10 +57,11 @@ __device__ __forceinline__ void horner_df(float xh, float xl, float &th, float &
     }
 }
 
-// The FP64 EXACT step: dt P = (Px, Py), their squares as float pairs.
+// The FP64 EXACT step's operator from dt P = (Px, Py) and their squares as float
+// pairs: m = cos(theta) - 1 and q = qr + i qi.
 template <int DC, int DS>
-__device__ __forceinline__ void step_f64_exact(F64Point &s, double Px, double Py, float2 px2,
-                                               float2 py2)
+__device__ __forceinline__ void operator_f64_exact(double Px, double Py, float2 px2, float2 py2,
+                                                   double &m, double &qr, double &qi)
 {
     float xh = px2.x, xl = px2.y;
     df_add(xh, xl, py2.x, py2.y);  // theta^2
@@ -69,9 +70,20 @@ __device__ __forceinline__ void step_f64_exact(F64Point &s, double Px, double Py
     df_mul(xh, xl, th, tl, mh, ml);
     horner_df<DS, 1, 1>(xh, xl, th, tl);  // (sin(theta)/theta - 1) / theta^2
     df_mul(xh, xl, th, tl, sh, sl);
-    const double m = df_to_f64(mh, ml), s1 = df_to_f64(sh, sl);
-    const double qr = fma(s1, Py, Py), qi = fma(s1, Px, Px);
-    // a' = a + m a - q b ; b' = b + m b + conj(q) a, q = qr + i qi
+    m = df_to_f64(mh, ml);
+    const double s1 = df_to_f64(sh, sl);
+    qr = fma(s1, Py, Py);
+    qi = fma(s1, Px, Px);
+}
+
+// The FP64 EXACT step.
+template <int DC, int DS>
+__device__ __forceinline__ void step_f64_exact(F64Point &s, double Px, double Py, float2 px2,
+                                               float2 py2)
+{
+    double m, qr, qi;
+    operator_f64_exact<DC, DS>(Px, Py, px2, py2, m, qr, qi);
+    // a' = a + m a - q b ; b' = b + m b + conj(q) a
     const double nar = fma(m, s.ar, fma(-qr, s.br, fma(qi, s.bi, s.ar)));
     const double nai = fma(m, s.ai, fma(-qr, s.bi, fma(-qi, s.br, s.ai)));
     const double nbr = fma(m, s.br, fma(qr, s.ar, fma(qi, s.ai, s.br)));
@@ -99,10 +111,10 @@ constexpr int kDfDegree = 5;
 // the small parts in double-float (kDfDegree), the update and q in FP64.  26 FP64
 // operations where the FP64 series took 26 + dc + ds.
 template <int DC, int DS>
-__device__ __forceinline__ void step_f64_magnus(F64Point &s, double Px, double Py, double2 d)
+__device__ __forceinline__ void operator_f64_magnus(double Px, double Py, double2 d, double &c,
+                                                    double &qr, double &qi, double &qz)
 {
     const double nz = fma(Px, d.y, -(Py * d.x));
-    double c, qr, qi, qz;
     if constexpr (DC <= kDfDegree) {
         const float2 px2 = square_df(Px), py2 = square_df(Py), nz2 = square_df(nz);
         float xh = px2.x, xl = px2.y;
@@ -126,6 +138,12 @@ __device__ __forceinline__ void step_f64_magnus(F64Point &s, double Px, double P
         qi = sn * Px;
         qz = sn * nz;
     }
+}
+template <int DC, int DS>
+__device__ __forceinline__ void step_f64_magnus(F64Point &s, double Px, double Py, double2 d)
+{
+    double c, qr, qi, qz;
+    operator_f64_magnus<DC, DS>(Px, Py, d, c, qr, qi, qz);
     // a' = (c - i qz) a - q b ; b' = conj(q) a + (c + i qz) b, q = qr + i qi: the small
     // terms first, one rounding at the state's size (from psi + m psi each term would
     // round there: 1.2 to 1.6 times the error over 12000 and 50000 steps)
@@ -232,25 +250,26 @@ __device__ __forceinline__ void strip64_step(F64Point (&pt)[H], double tx, doubl
 // What bounds every FP64 launch is the FP64 pipe: a warp's DFMA holds its
 // scheduler's unit for 64 cycles (33 ns measured, whatever the number of active
 // lanes), so a launch takes as long as the scheduler with the most FP64 instructions.
-// Warps work alone (their own double-buffered bulk copies of the table with bounded
-// waits, no CTA-wide barrier), and the host picks the shape that loads the fullest
-// scheduler least (f64_shape in dsp_api.cpp).  FP64 instructions of a warp per EXACT
-// step and its points:
+// Warps (in one shape, pairs of warps) work alone: their own double-buffered bulk copies
+// of the table with bounded waits, no CTA-wide barrier, and the host picks the shape that
+// loads the fullest scheduler least (f64_lanes in dsp_api.cpp).  FP64 instructions per
+// step of a tile (EXACT, STRANG_XY, MAGNUS4) and its points:
 //   rows   32 columns x 4 rows: the dt P_x part once per lane, the dt P_y part once per
-//          row and step in a shared table                                65 for 128
-//   flat 1 32 consecutive points                                         18 for 32
-//   flat 2 16 consecutive points, a lane pair per point: lane 0 holds a, lane 1 b;
-//          each forms one of P_x and P_y, of the two series, and of the two parts of
-//          q, and they trade by shuffles                                  9 for 16
-//   flat 4 8 points, a lane per real component                            6 for 8
-// (STRANG_XY: rows 62, flat 24; MAGNUS4: flat 26.)  Every FP64 operation of a point is the same in every shape (same operands, same
-// rounding), so its result is bitwise the same.  STRANG_XY takes rows or flat 1,
-// MAGNUS4 flat 1.  The projection is the projection kernel's, on the state these
-// leave.
+//          row and step in a shared table                       65, 62, - for 128
+//   flat   32 consecutive points, a lane each                   18, 24, 26 for 32
+//   pair   8 points, a lane per real component in one warp, the operators of four
+//          steps at once in the other                           4.5, 6, 6.5 for 8
+// Every FP64 operation of a point is the same in every shape (same operands, same
+// rounding), so its result is bitwise the same.  The projection is the projection
+// kernel's, on the state these leave.
 //
-// Measured: 64^2 x 2000 steps 9.48 -> 1.08 ms (1024-point CTAs held 4 of 152 SMs;
-// flat 4 holds 512 warps), 300 x 257 x 1700 steps 8.10 -> 4.20 ms; 1000 steps of 512^2:
-// MAGNUS4 19.8 -> 12.4 ms, STRANG_XY 9.48 -> 8.50 ms.
+// A step's operator is a chain of ~900 cycles before its update, and a warp cannot run
+// the one beside the other: its own FP64 instructions hold its issue.  Flat and rows
+// therefore need several warps per scheduler, and pairs take the launches that cannot
+// give them.  Measured, 2000 EXACT steps: 64^2 9.48 ms with 1024-point CTAs (4 of 152
+// SMs), 1.80 flat, 1.08 with 4 lanes a point on one warp, 0.40 on pairs (0.22 of FP64
+// work over the whole chip); 128^2 1.83 flat, 1.12 pairs; 256^2 4.83, 4.31; 300 x 257
+// 4.84 flat, 4.92 pairs; 512^2 17.1 rows, 16.5 flat and pairs.
 // ---------------------------------------------------------------------------
 
 constexpr int kF64Stage = 1024;  // bytes per staged table chunk and warp
@@ -342,165 +361,13 @@ __device__ __forceinline__ double shfl_x(double v, int mask)
 {
     return __shfl_xor_sync(0xffffffffu, v, mask);
 }
-__device__ __forceinline__ float shfl_x(float v, int mask)
-{
-    return __shfl_xor_sync(0xffffffffu, v, mask);
-}
 
-// sum_{k=K..D} c_k x^(k-K) in double-float as horner_df, for U steps at once, of the cos
-// series (odd = false: c_k = (-1)^k/(2k)!, to DC) or the sinc one (odd: (-1)^k/(2k +
-// 1)!, to DS); the shorter one starts from zero coefficients, which changes nothing.
-template <int DC, int DS, int K, int U>
-__device__ __forceinline__ void horner_either(bool odd, const float (&xh)[U], const float (&xl)[U],
-                                              float (&th)[U], float (&tl)[U])
-{
-    constexpr int D = DC > DS ? DC : DS;
-    constexpr double sign = (K & 1) ? -1.0 : 1.0;
-    constexpr DFConst c = df_const(K <= DC ? sign * inv_factorial<2 * K>() : 0.0);
-    constexpr DFConst s = df_const(K <= DS ? sign * inv_factorial<2 * K + 1>() : 0.0);
-    const float ch = odd ? s.h : c.h, cl = odd ? s.l : c.l;
-    if constexpr (K < D)
-        horner_either<DC, DS, K + 1, U>(odd, xh, xl, th, tl);
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        if constexpr (K == D) {
-            th[u] = ch;
-            tl[u] = cl;
-        } else {
-            float ph, pl;
-            df_mul(xh[u], xl[u], th[u], tl[u], ph, pl);
-            df_add(ph, pl, ch, cl);
-            th[u] = ph;
-            tl[u] = pl;
-        }
-    }
-}
-
-// EXACT steps on L = 2 or 4 lanes per point (step_f64_exact's operations).  Lane k of a
-// point: L = 2 holds a (k = 0) or b (k = 1) in v[0], v[1]; L = 4 holds Re a, Im a, Re b,
-// Im b.  An operator's entries as the lane applies them:
-template <int L, int U>
-struct LaneOps {
-    double m[U], sr[U], si[U];  // cos - 1; -+ Re q; +- Im q (L = 2: Im q)
-};
-
-// The operators of U steps, stage by stage for all of them (a step's own chain of
-// conversions, shuffles and double-float series takes ~900 cycles).  P: the lane's P_x
-// (k even) or P_y (k odd).
-template <int DC, int DS, int L, int U>
-__device__ __forceinline__ void lane_ops(LaneOps<L, U> &o, const double (&P)[U], int k)
-{
-    const bool odd = k & 1;
-    float2 own[U];
-    float xh[U], xl[U], th[U], tl[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-        own[u] = square_df(P[u]);
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        th[u] = shfl_x(own[u].x, 1);
-        tl[u] = shfl_x(own[u].y, 1);
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {  // P_x^2 + P_y^2
-        xh[u] = odd ? th[u] : own[u].x;
-        xl[u] = odd ? tl[u] : own[u].y;
-        df_add(xh[u], xl[u], odd ? own[u].x : th[u], odd ? own[u].y : tl[u]);
-    }
-    horner_either<DC, DS, 1, U>(odd, xh, xl, th, tl);
-    double mine[U], q[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        float ph, pl;
-        df_mul(xh[u], xl[u], th[u], tl[u], ph, pl);
-        mine[u] = df_to_f64(ph, pl);
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        const double other = shfl_x(mine[u], 1);
-        o.m[u] = odd ? other : mine[u];
-        q[u] = fma(odd ? mine[u] : other, P[u], P[u]);
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        const double p = shfl_x(q[u], 1);
-        const double qr = odd ? q[u] : p, qi = odd ? p : q[u];
-        if constexpr (L == 2) {
-            o.sr[u] = odd ? qr : -qr;
-            o.si[u] = qi;
-        } else {
-            o.sr[u] = (k & 2) ? qr : -qr;
-            o.si[u] = odd ? -qi : qi;
-        }
-    }
-}
-
-template <int L, int U>
-__device__ __forceinline__ void lane_apply(double (&v)[4 / L], const LaneOps<L, U> &o)
-{
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        if constexpr (L == 2) {
-            const double tr = shfl_x(v[0], 1), ti = shfl_x(v[1], 1);
-            const double nr = fma(o.m[u], v[0], fma(o.sr[u], tr, fma(o.si[u], ti, v[0])));
-            const double ni = fma(o.m[u], v[1], fma(o.sr[u], ti, fma(-o.si[u], tr, v[1])));
-            v[0] = nr;
-            v[1] = ni;
-        } else {
-            const double t1 = shfl_x(v[0], 2), t2 = shfl_x(v[0], 3);
-            v[0] = fma(o.m[u], v[0], fma(o.sr[u], t1, fma(o.si[u], t2, v[0])));
-        }
-    }
-}
-
-// A chunk's steps: the operators of the next kLaneSteps steps are formed beside the
-// current ones' updates.  A warp waits out the issue of its own FP64 instructions, so
-// this hides shuffles and FP32 latency only, and only 4 lanes per point, which run
-// where a scheduler has one warp or two, take it (64^2 x 2000: 1.29 -> 1.08 ms); on 2
-// lanes the registers push out warps that hide more (4 steps on 256^2: 4.84 -> 5.31
-// ms).  a: the lane's component of the chunk's entries (every second double).
-template <int L>
-constexpr int kLaneSteps = L == 4 ? 4 : 1;
-template <int DC, int DS, int L>
-__device__ __forceinline__ void lane_steps(double (&v)[4 / L], const double *a, double t, int len,
-                                           int k)
-{
-    constexpr int U = kLaneSteps<L>;
-    const auto block = [&](LaneOps<L, U> &o, int j) {
-        double P[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            P[u] = t + a[2 * (j + u)];
-        lane_ops<DC, DS, L, U>(o, P, k);
-    };
-    int j = 0;
-    if (len >= U) {
-        LaneOps<L, U> cur;
-        block(cur, 0);
-        for (j = U; j + U <= len; j += U) {
-            LaneOps<L, U> next;
-            block(next, j);
-            lane_apply<L, U>(v, cur);
-            cur = next;
-        }
-        lane_apply<L, U>(v, cur);
-    }
-    for (; j < len; ++j) {
-        LaneOps<L, 1> o;
-        const double P[1] = {t + a[2 * j]};
-        lane_ops<DC, DS, L, 1>(o, P, k);
-        lane_apply<L, 1>(v, o);
-    }
-}
-
-// A flat tile of 32 / L consecutive points.
-template <int SCHEME, int DC, int DS, int L>
+// A flat tile of 32 consecutive points.
+template <int SCHEME, int DC, int DS>
 __device__ void body_flat(const ReqDesc &R, int tile, F64Smem &sm, int *err)
 {
-    constexpr int PTS = 32 / L;
     const int lane = threadIdx.x & 31;
-    const int k = lane % L;
-    const int64_t idx = static_cast<int64_t>(tile) * PTS + lane / L;
+    const int64_t idx = static_cast<int64_t>(tile) * 32 + lane;
     const bool valid = idx < R.n_points;
     const double vs = R.valley > 0 ? 1.0 : -1.0;
     double px = 0.0, py = 0.0;
@@ -512,46 +379,164 @@ __device__ void body_flat(const ReqDesc &R, int tile, F64Smem &sm, int *err)
     pt.tx = vs * (R.dt * px);  // valley K- is stepped as K+ on -P
     pt.ty = vs * (R.dt * py);
     load_f64(R, idx, valid, px, py, vs, pt);
-    double2 *a_plane = static_cast<double2 *>(R.state);
-    if constexpr (L == 1) {
-        using E = typename std::conditional<SCHEME == 2, F64G2, double2>::type;
-        const WarpStager<E> st(R, &sm.stage[0][0], sm.bars);
-        if (!st.run(err, [&](const E *e, int len) {
+    using E = typename std::conditional<SCHEME == 2, F64G2, double2>::type;
+    const WarpStager<E> st(R, &sm.stage[0][0], sm.bars);
+    if (!st.run(err, [&](const E *e, int len) {
 #pragma unroll 2
-                for (int j = 0; j < len; ++j) {
-                    if constexpr (SCHEME == 2)
-                        step_f64<SCHEME, DC, DS>(pt, e[j].a, e[j].d);
-                    else
-                        step_f64<SCHEME, DC, DS>(pt, e[j], make_double2(0.0, 0.0));
-                }
-            }))
-            return;
-        if (valid) {
-            a_plane[idx] = make_double2(pt.ar, pt.ai);
-            a_plane[R.n_points + idx] = make_double2(pt.br, pt.bi);
-        }
+            for (int j = 0; j < len; ++j) {
+                if constexpr (SCHEME == 2)
+                    step_f64<SCHEME, DC, DS>(pt, e[j].a, e[j].d);
+                else
+                    step_f64<SCHEME, DC, DS>(pt, e[j], make_double2(0.0, 0.0));
+            }
+        }))
+        return;
+    double2 *a_plane = static_cast<double2 *>(R.state);
+    if (valid) {
+        a_plane[idx] = make_double2(pt.ar, pt.ai);
+        a_plane[R.n_points + idx] = make_double2(pt.br, pt.bi);
+    }
+}
+
+// 4 lanes per point and two warps per 8 points.  A warp waits out the issue of its own
+// FP64 instructions, so one warp cannot form a step's operator beside another step's
+// update; here one warp of the pair forms operators, the lanes of a point those of four
+// steps at once, and hands them through shared memory, kPairSteps at a time and double
+// buffered, to the other, whose lanes hold Re a, Im a, Re b, Im b of a point and only
+// apply them.  Waits between the two are bounded like those for the table.
+constexpr int kPairSteps = 16;
+static_assert(kF64Chunk % kPairSteps == 0 && kF64Chunk / 2 % kPairSteps == 0,
+              "table chunks are whole slots");
+struct PairSmem {
+    unsigned char stage[2][kF64Stage];
+    double ops[2][kPairSteps][4][8];  // per step: m or c, qr, qi, qz of the 8 points
+    uint64_t bars[2];                 // table chunks
+    uint64_t full[2], empty[2];       // slots of ops
+};
+
+// A step's operator into out: EXACT m, qr, qi; STRANG_XY c, qr, qi; MAGNUS4 c, qr, qi, qz.
+template <int SCHEME, int DC, int DS, typename E>
+__device__ __forceinline__ void form_operator(const E &e, double tx, double ty,
+                                              double (&out)[4][8], int pt)
+{
+    double c, qr, qi;
+    if constexpr (SCHEME == 2) {
+        double qz;
+        operator_f64_magnus<DC, DS>(tx + e.a.x, ty + e.a.y, e.d, c, qr, qi, qz);
+        out[3][pt] = qz;
     } else {
-        double v[4 / L];
-        if constexpr (L == 2) {
-            v[0] = k ? pt.br : pt.ar;
-            v[1] = k ? pt.bi : pt.ai;
+        const double Px = tx + e.x, Py = ty + e.y;
+        if constexpr (SCHEME == 0) {
+            operator_f64_exact<DC, DS>(Px, Py, square_df(Px), square_df(Py), c, qr, qi);
         } else {
-            v[0] = k < 2 ? (k == 0 ? pt.ar : pt.ai) : (k == 2 ? pt.br : pt.bi);
-        }
-        const double t = (k & 1) ? pt.ty : pt.tx;
-        const WarpStager<double2> st(R, &sm.stage[0][0], sm.bars);
-        if (!st.run(err, [&](const double2 *e, int len) {
-                lane_steps<DC, DS, L>(v, reinterpret_cast<const double *>(e) + (k & 1), t, len, k);
-            }))
-            return;
-        if (valid) {
-            if constexpr (L == 2)
-                a_plane[(k ? R.n_points : 0) + idx] = make_double2(v[0], v[1]);
-            else
-                reinterpret_cast<double *>(a_plane)[2 * ((k < 2 ? 0 : R.n_points) + idx) + (k & 1)] =
-                    v[0];
+            const double2 x = strang_part<DC, DS>(Px), y = strang_part<DC, DS>(Py);
+            c = y.x * x.x;
+            qr = y.y;
+            qi = y.x * x.y;
         }
     }
+    out[0][pt] = c;
+    out[1][pt] = qr;
+    out[2][pt] = qi;
+}
+
+template <int SCHEME, int DC, int DS>
+__device__ void pair_operators(const ReqDesc &R, double tx, double ty, PairSmem &sm, int *err)
+{
+    const int lane = threadIdx.x & 31, s = lane & 3;
+    using E = typename std::conditional<SCHEME == 2, F64G2, double2>::type;
+    const WarpStager<E> st(R, &sm.stage[0][0], sm.bars);
+    int q = 0;
+    bool ok = true;
+    st.run(err, [&](const E *e, int len) {
+        for (int b = 0; b < len; b += kPairSteps, ++q) {
+            if (ok && q >= 2)  // the other warp is done with the slot
+                ok = __all_sync(0xffffffffu, mbar_wait_bounded(&sm.empty[q & 1], ((q >> 1) - 1) & 1));
+            if (!ok)
+                continue;
+#pragma unroll
+            for (int p = 0; p < kPairSteps; p += 4) {
+                const int j = b + p + s;  // past the end: the last one's, not applied
+                form_operator<SCHEME, DC, DS>(e[j < len ? j : len - 1], tx, ty,
+                                              sm.ops[q & 1][p + s], lane >> 2);
+            }
+            __syncwarp();
+            if (lane == 0)
+                mbar_arrive(&sm.full[q & 1]);
+        }
+    });
+    if (!ok && lane == 0)
+        atomicOr(err, kErrTimeout);
+}
+
+// v with its sign bit flipped where mask is 1 << 31: an integer operation (choosing
+// between x and -x negates on the FP64 pipe: 64^2 x 2000 took 0.56 ms, not 0.40).
+__device__ __forceinline__ double flip_sign(double v, int mask)
+{
+    return __hiloint2double(__double2hiint(v) ^ mask, __double2loint(v));
+}
+
+template <int SCHEME>
+__device__ __forceinline__ bool pair_updates(double &v, int64_t nsteps, PairSmem &sm, int *err)
+{
+    constexpr int kSign = static_cast<int>(0x80000000u);
+    const int lane = threadIdx.x & 31, k = lane & 3;
+    const int sr_mask = (k & 2) ? 0 : kSign, si_mask = (k & 1) ? kSign : 0;
+    const int sz_mask = k == 1 || k == 2 ? kSign : 0;
+    for (int q = 0; static_cast<int64_t>(q) * kPairSteps < nsteps; ++q) {
+        if (!__all_sync(0xffffffffu, mbar_wait_bounded(&sm.full[q & 1], (q >> 1) & 1))) {
+            if (lane == 0)
+                atomicOr(err, kErrTimeout);
+            return false;
+        }
+        const int64_t left = nsteps - static_cast<int64_t>(q) * kPairSteps;
+        const int len = left < kPairSteps ? static_cast<int>(left) : kPairSteps;
+        const double *o = &sm.ops[q & 1][0][0][lane >> 2];
+#pragma unroll 4
+        for (int u = 0; u < len; ++u, o += 4 * 8) {
+            const double c = o[0];
+            const double sr = flip_sign(o[8], sr_mask), si = flip_sign(o[16], si_mask);
+            const double t1 = shfl_x(v, 2), t2 = shfl_x(v, 3);
+            if constexpr (SCHEME == 0) {
+                v = fma(c, v, fma(sr, t1, fma(si, t2, v)));
+            } else if constexpr (SCHEME == 1) {
+                v = fma(c, v, fma(sr, t1, si * t2));
+            } else {
+                const double t0 = shfl_x(v, 1);
+                v = fma(c, v, fma(flip_sign(o[24], sz_mask), t0, fma(sr, t1, si * t2)));
+            }
+        }
+        __syncwarp();
+        if (lane == 0)
+            mbar_arrive(&sm.empty[q & 1]);
+    }
+    return true;
+}
+
+// A tile of 8 consecutive points; `forms`: this warp forms the operators.
+template <int SCHEME, int DC, int DS>
+__device__ void body_pair(const ReqDesc &R, int tile, PairSmem &sm, int *err, bool forms)
+{
+    const int lane = threadIdx.x & 31, k = lane & 3;
+    const int64_t idx = static_cast<int64_t>(tile) * 8 + (lane >> 2);
+    const bool valid = idx < R.n_points;
+    const double vs = R.valley > 0 ? 1.0 : -1.0;
+    double px = 0.0, py = 0.0;
+    if (valid) {
+        px = grid_node(R.px_min, R.hx, idx % R.nx);
+        py = grid_node(R.py_min, R.hy, R.row0 + idx / R.nx);
+    }
+    if (forms) {  // valley K- is stepped as K+ on -P
+        pair_operators<SCHEME, DC, DS>(R, vs * (R.dt * px), vs * (R.dt * py), sm, err);
+        return;
+    }
+    F64Point pt;
+    load_f64(R, idx, valid, px, py, vs, pt);
+    double v = k < 2 ? (k == 0 ? pt.ar : pt.ai) : (k == 2 ? pt.br : pt.bi);
+    if (!pair_updates<SCHEME>(v, R.step_end > R.step_begin ? R.step_end - R.step_begin : 0, sm, err))
+        return;
+    if (valid)
+        static_cast<double *>(R.state)[2 * ((k < 2 ? 0 : R.n_points) + idx) + (k & 1)] = v;
 }
 
 // A tile of 32 columns x 4 rows (EXACT and STRANG_XY).
@@ -601,23 +586,32 @@ __device__ void body_rows(const ReqDesc &R, int tile, F64Smem &sm, int *err)
     }
 }
 
-// Warp-uniform dispatch on the request's series level (compile-time degrees).  L: 1, 2,
-// 4 flat; 0 rows.
-template <int SCHEME, int L, int V>
-__device__ __forceinline__ void dispatch_f64(const ReqDesc &R, int tile, F64Smem &sm, int *err)
+// Warp-uniform dispatch on the request's scheme and series level (compile-time
+// degrees): body(scheme, dc, ds) as integral constants.
+template <int SCHEME, int V, typename Body>
+__device__ __forceinline__ void dispatch_level(const ReqDesc &R, Body body)
 {
-    if (R.level == V || V + 1 == kNumLevels) {
-        if constexpr (L == 0)
-            body_rows<SCHEME, kLevelsF64[V].dc, kLevelsF64[V].ds>(R, tile, sm, err);
-        else
-            body_flat<SCHEME, kLevelsF64[V].dc, kLevelsF64[V].ds, L>(R, tile, sm, err);
-    } else if constexpr (V + 1 < kNumLevels) {
-        dispatch_f64<SCHEME, L, V + 1>(R, tile, sm, err);
-    }
+    if (R.level == V || V + 1 == kNumLevels)
+        body(std::integral_constant<int, SCHEME>{},
+             std::integral_constant<int, kLevelsF64[V].dc>{},
+             std::integral_constant<int, kLevelsF64[V].ds>{});
+    else if constexpr (V + 1 < kNumLevels)
+        dispatch_level<SCHEME, V + 1>(R, body);
+}
+template <bool MAGNUS, typename Body>
+__device__ __forceinline__ void dispatch_f64(const ReqDesc &R, Body body)
+{
+    if (R.scheme == 0)
+        dispatch_level<0, 0>(R, body);
+    else if (R.scheme == 1)
+        dispatch_level<1, 0>(R, body);
+    else if constexpr (MAGNUS)
+        dispatch_level<2, 0>(R, body);
 }
 
-template <int L>
-__global__ void __launch_bounds__(32 * kF64Warps, L == 4 ? 2 : L == 0 ? 4 : 5)
+// Tiles on one warp: ROWS 32 columns x 4 rows, otherwise flat.
+template <bool ROWS>
+__global__ void __launch_bounds__(32 * kF64Warps, ROWS ? 4 : 5)
     evolve_f64_kernel(const __grid_constant__ EvolveArgs args)
 {
     __shared__ __align__(128) F64Smem smem[kF64Warps];
@@ -636,22 +630,45 @@ __global__ void __launch_bounds__(32 * kF64Warps, L == 4 ? 2 : L == 0 ? 4 : 5)
     const int tile = t - R.tile_begin;
     if (!tile_ok(R, tile, R.err) || !table_range_ok(R, R.step_begin, R.err))
         return;
-    if (L > 1 || R.scheme == 0)
-        dispatch_f64<0, L, 0>(R, tile, sm, R.err);
-    else if constexpr (L <= 1) {
-        if (R.scheme == 1)
-            dispatch_f64<1, L, 0>(R, tile, sm, R.err);
-        else if constexpr (L == 1)
-            dispatch_f64<2, L, 0>(R, tile, sm, R.err);
-    }
+    dispatch_f64<!ROWS>(R, [&](auto scheme, auto dc, auto ds) {
+        if constexpr (ROWS)
+            body_rows<decltype(scheme)::value, decltype(dc)::value, decltype(ds)::value>(R, tile,
+                                                                                         sm, R.err);
+        else
+            body_flat<decltype(scheme)::value, decltype(dc)::value, decltype(ds)::value>(R, tile,
+                                                                                         sm, R.err);
+    });
 }
 
-template <int L>
-cudaError_t launch_lanes(const EvolveArgs &args, int warps, cudaStream_t stream)
+// Warp pairs, kF64Warps / 2 of them or one per CTA.  The CTAs are dealt to the SMs in
+// turn, so that swapping the warps' roles from one round of SMs to the next puts both
+// kinds on every scheduler.
+__global__ void __launch_bounds__(32 * kF64Warps, 4)
+    evolve_f64_pair_kernel(const __grid_constant__ EvolveArgs args, int sms)
 {
-    const int grid = (args.total_tiles + warps - 1) / warps;
-    evolve_f64_kernel<L><<<grid, 32 * warps, 0, stream>>>(args);
-    return cudaGetLastError();
+    __shared__ __align__(128) PairSmem smem[kF64Warps / 2];
+    const int w = threadIdx.x >> 5;
+    PairSmem &sm = smem[w >> 1];
+    if ((threadIdx.x & 63) == 0) {
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&sm.bars[i], 1);
+            mbar_init(&sm.full[i], 1);
+            mbar_init(&sm.empty[i], 1);
+        }
+        fence_mbar_init();
+    }
+    __syncthreads();
+    const int t = static_cast<int>(blockIdx.x) * static_cast<int>(blockDim.x >> 6) + (w >> 1);
+    if (t >= args.total_tiles)
+        return;
+    const ReqDesc &R = args.r[find_request(args, t)];
+    const int tile = t - R.tile_begin;
+    if (!tile_ok(R, tile, R.err) || !table_range_ok(R, R.step_begin, R.err))
+        return;
+    const bool forms = (w & 1) != ((blockIdx.x / sms) & 1);
+    dispatch_f64<true>(R, [&](auto scheme, auto dc, auto ds) {
+        body_pair<decltype(scheme)::value, decltype(dc)::value, decltype(ds)::value>(R, tile, sm, R.err, forms);
+    });
 }
 
 }  // namespace
@@ -660,10 +677,24 @@ cudaError_t launch_evolve_f64(const EvolveArgs &args, int lanes, int warps, cuda
 {
     if (args.nreq <= 0 || args.total_tiles <= 0)
         return cudaSuccess;
-    return lanes == 0   ? launch_lanes<0>(args, warps, stream)
-           : lanes == 1 ? launch_lanes<1>(args, warps, stream)
-           : lanes == 2 ? launch_lanes<2>(args, warps, stream)
-                        : launch_lanes<4>(args, warps, stream);
+    if (lanes == 4) {
+        int dev = 0, sms = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess)
+            e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess)
+            return e;
+        const int pairs = warps > 1 ? warps / 2 : 1;
+        evolve_f64_pair_kernel<<<(args.total_tiles + pairs - 1) / pairs, 64 * pairs, 0, stream>>>(
+            args, sms);
+        return cudaGetLastError();
+    }
+    const int grid = (args.total_tiles + warps - 1) / warps;
+    if (lanes == 0)
+        evolve_f64_kernel<true><<<grid, 32 * warps, 0, stream>>>(args);
+    else
+        evolve_f64_kernel<false><<<grid, 32 * warps, 0, stream>>>(args);
+    return cudaGetLastError();
 }
 
 }  // namespace dsp

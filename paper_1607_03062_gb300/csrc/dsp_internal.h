@@ -253,10 +253,10 @@ struct CombineArgs {
     int32_t row0;  // global row index of the grid's first row
 };
 
-// Evolve launches, one kernel per kind of request.  FP64: `lanes` 0 tiles of 32
-// columns x 4 rows (no MAGNUS4), 1, 2 or 4 lanes per point on tiles of 32 / lanes
-// consecutive points (2, 4: EXACT only); n_tiles counts those, `warps` tiles per CTA.
-// Does not project.
+// Evolve launches, one kernel per kind of request (every FP64 request in args has the
+// same scheme).  FP64: `lanes` 0 tiles of 32 columns x 4 rows (no MAGNUS4), 1 of 32
+// consecutive points, 4 of 8 points on a warp pair; n_tiles counts those, `warps` warps
+// per CTA.  Does not project.
 cudaError_t launch_evolve_f64(const EvolveArgs &args, int lanes, int warps, cudaStream_t stream);
 // FP32_MIXED on contiguous tiles.
 cudaError_t launch_evolve_mixed(const EvolveArgs &args, cudaStream_t stream);

@@ -1,6 +1,6 @@
-"""The FP64 kernels' shapes -- 32 columns x 4 rows per warp, or 32, 16 or 8 consecutive points on 1,
-2 or 4 lanes each -- give bitwise the same map, density and state.  The tiling hook forces the
-first two; sizes from one point to a few thousand take 4 and 2 lanes by themselves."""
+"""The FP64 kernels' shapes -- 32 columns x 4 rows or 32 consecutive points per warp, or 8 points per
+warp pair, one warp forming the operators and one applying them -- give bitwise the same map, density
+and state.  The tiling hook forces the first two; sizes up to a few thousand points take pairs."""
 import numpy as np
 import pytest
 import torch
@@ -33,7 +33,7 @@ def solve(size, table, scheme, tiling, valley=1, pieces=()):
     return out
 
 
-# one point; a lane pair and a warp not full; a lane-quad launch; a lane-pair one; several waves
+# one point; warps not full; one pair per scheduler; several; several warps per scheduler
 @pytest.mark.parametrize("size", [(1, 1), (7, 3), (64, 65), (131, 90), (300, 257)])
 @pytest.mark.parametrize("scheme", ["exact", "strang_xy", "magnus4"])
 @pytest.mark.parametrize("steps", [1, 67, 130])
