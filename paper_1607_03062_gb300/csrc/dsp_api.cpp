@@ -571,7 +571,7 @@ int f64_lanes(const std::vector<ReqDesc> &reqs, int scheme)
     };
     constexpr Shape shapes[3] = {{1, {18.2, 24.2, 26.2}, {27.5, 39.0, 38.5}},
                                  {0, {65.0, 62.0, 0.0}, {93.0, 72.0, 0.0}},
-                                 {4, {4.8, 7.0, 6.9}, {6.0, 10.0, 9.0}}};
+                                 {4, {4.8, 6.6, 6.9}, {6.0, 10.0, 9.0}}};
     int best = 1;
     double best_t = 0.0;
     for (const Shape &sh : shapes) {
