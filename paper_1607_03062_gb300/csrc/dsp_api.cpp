@@ -466,7 +466,7 @@ ReqDesc projection_of(const ReqDesc &r)
 template <typename Tiles>
 size_t fill_launch(const std::vector<ReqDesc> &reqs, size_t i, EvolveArgs &a, Tiles tiles)
 {
-    std::memset(&a, 0, sizeof(EvolveArgs));
+    a.nreq = a.total_tiles = 0;  // (the descriptors past nreq are never read)
     for (; i < reqs.size() && a.nreq < dsp::kMaxReqPerLaunch; ++i) {
         ReqDesc &r = a.r[a.nreq++];
         r = reqs[i];
@@ -480,7 +480,7 @@ size_t fill_launch(const std::vector<ReqDesc> &reqs, size_t i, EvolveArgs &a, Ti
 cudaError_t launch_projections(const std::vector<ReqDesc> &reqs, int precision,
                                cudaStream_t stream)
 {
-    std::unique_ptr<EvolveArgs> a(new EvolveArgs());
+    std::unique_ptr<EvolveArgs> a(new EvolveArgs);  // filled by fill_launch
     for (size_t i = 0; i < reqs.size();) {
         i = fill_launch(reqs, i, *a, [](const ReqDesc &r) { return r.n_tiles; });
         const cudaError_t e = dsp::launch_project(*a, precision, stream);
@@ -539,7 +539,7 @@ int group_rows(const std::vector<ReqDesc> &reqs)
 cudaError_t launch_groups(const std::vector<ReqDesc> &reqs, cudaStream_t stream)
 {
     const int rows = group_rows(reqs);
-    std::unique_ptr<EvolveArgs> a(new EvolveArgs());
+    std::unique_ptr<EvolveArgs> a(new EvolveArgs);  // filled by fill_launch
     for (size_t i = 0; i < reqs.size();) {
         i = fill_launch(reqs, i, *a, [&](const ReqDesc &r) { return row_tiles(r, rows); });
         const cudaError_t e = dsp::launch_evolve_group(
@@ -595,7 +595,7 @@ int f64_lanes(const std::vector<ReqDesc> &reqs, int scheme)
 // Queues the evolution of FP64 requests, one launch per scheme (and 96 requests).
 cudaError_t launch_f64(const std::vector<ReqDesc> &reqs, cudaStream_t stream)
 {
-    std::unique_ptr<EvolveArgs> a(new EvolveArgs());
+    std::unique_ptr<EvolveArgs> a(new EvolveArgs);  // filled by fill_launch
     for (int scheme = 0; scheme < 3; ++scheme) {
         std::vector<ReqDesc> sel;
         for (const ReqDesc &r : reqs)
@@ -622,7 +622,7 @@ cudaError_t launch_steps_mixed(const std::vector<ReqDesc> &reqs, cudaStream_t st
     if (reqs.size() == 1)
         split = split_last_wave(reqs[0]);
     const std::vector<ReqDesc> &all = split.empty() ? reqs : split;
-    std::unique_ptr<EvolveArgs> a(new EvolveArgs());
+    std::unique_ptr<EvolveArgs> a(new EvolveArgs);  // filled by fill_launch
     // kernel kinds: 0 contiguous tiles; 1 + 2 scheme + (strip_h == 2): row strips
     for (int kind = 0; kind < 7; ++kind) {
         std::vector<ReqDesc> sel;
@@ -666,10 +666,16 @@ cudaError_t launch_requests(const std::vector<ReqDesc> &given, int precision, cu
                 after.push_back(projection_of(r));
         }
     }
-    cudaError_t e = launch_groups(grouped, stream);
-    if (e == cudaSuccess)
+    // (a launch's 27 KB of parameters cost ~0.5 us to allocate and clear: a projection
+    // alone, 6.2 us on a small grid, does not pay for the empty ones)
+    cudaError_t e = cudaSuccess;
+    if (!grouped.empty())
+        e = launch_groups(grouped, stream);
+    if (e == cudaSuccess && !steps.empty())
         e = precision == DSP_FP64 ? launch_f64(steps, stream) : launch_steps_mixed(steps, stream);
-    return e == cudaSuccess ? launch_projections(after, precision, stream) : e;
+    if (e == cudaSuccess && !after.empty())
+        e = launch_projections(after, precision, stream);
+    return e;
 }
 
 cudaError_t launch_finalizes(const std::vector<dsp::FinDesc> &fins, cudaStream_t stream)
