@@ -246,10 +246,10 @@ def ops_strang(dc, ds, group=1, strips=False, tdeg=0):
 
 def ops_groups(steps, level, strang=False):
     """FP32 lane instructions per spinor-step of expanded groups of `steps` steps: per
-    group 42 (level 0), 64 (1) or 76 (2) for the operator and the compensated update, 11
+    group 42 (level 0), 64 (1) or 75 (2) for the operator and the compensated update, 11
     more for STRANG_XY's momentum, and the column part (9 scalar ops per lane) shared by
     its 4 rows."""
-    return ((42, 64, 76)[level] + (11 if strang else 0) + 9 / 4.0) / steps
+    return ((42, 64, 75)[level] + (11 if strang else 0) + 9 / 4.0) / steps
 
 
 def ops_fp64(dc, ds, strips=False):
