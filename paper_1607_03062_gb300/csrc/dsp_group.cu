@@ -577,7 +577,8 @@ static_assert(kGroupWarps * sizeof(WarpSmem) <= 48 * 1024, "dynamic shared memor
 //     K S from L_ij = int int_{t1>t2} (t1 d1_i d2_j - t2 d2_i d1_j).
 // (Magnus series; Blanes, Casas, Oteo and Ros, Phys. Rep. 470 (2009) 151.)  MAGNUS4
 // steps exp(-i (sigma.P_n + sigma_z P_n x D_n)) add the sigma_z parts of their
-// commutators to the disturbance: the same polynomials with other coefficients.
+// commutators, z D/2, to the disturbance: the same integrals one power of z higher, so
+// the odd moments of D enter the plane (u2, u4) and the even ones w_z (n1, n3, n5).
 // STRANG_XY's P' adds the second derivative of its cubic terms, sum d d, to K (the rest
 // of P' depends on S alone and is the evolve kernel's).
 // The next power of x = |S|^2 is folded into the kept ones (its Chebyshev
@@ -587,7 +588,8 @@ static_assert(kGroupWarps * sizeof(WarpSmem) <= 48 * 1024, "dynamic shared memor
 // run.  Against the true sum of the groups' largest errors over the box (FP64, CPU):
 // smooth pulses 0.7e-6 (Gaussian pulse, eps 0.63), 9e-8 (two colours, 0.36), 2e-10
 // (sin^2, 0.16) for estimates about three times that; tables of noise, steps, spikes
-// and kinks: at most 0.69 of the estimate.
+// and kinks, and for MAGNUS4 of noise in D alone: at most 0.7 of the estimate (EXACT
+// 1.2 where a group drops less than 1e-9).
 //
 // One thread per group, and one per 16 steps for the per-step table (dt A rounded
 // to FP32 with error feedback inside the 16); FP64 only where the group's sum and
@@ -691,12 +693,12 @@ __device__ __forceinline__ void expand_group(const PrepArgs &args, int64_t g, fl
                   static_cast<float>(k7 * 7.0 * G4 / 34560.0) * M3 -
                   static_cast<float>(k7 * 31.0 * G6 / 967680.0) * M1;
     F2 u2 = static_cast<float>(0.5 * k2) * M2;
-    const F2 u4 = static_cast<float>(k4 * G2 / 48.0) * M2 - static_cast<float>(k4 / 24.0) * M4;
+    F2 u4 = static_cast<float>(k4 * G2 / 48.0) * M2 - static_cast<float>(k4 / 24.0) * M4;
     const float X = eps * eps, e3 = X * eps, e5 = e3 * X, e7 = e5 * X;
     const float s = s_odd + s_even;
     wide = 0.0f;
     if (args.scheme == 2) {
-        F2 D0{0, 0}, D1{0, 0}, D2{0, 0}, D4{0, 0};
+        F2 D0{0, 0}, D1{0, 0}, D2{0, 0}, D3{0, 0}, D4{0, 0};  // int tau^k D dtau
         float sD = 0.0f;
 #pragma unroll
         for (int n = 0; n < G; ++n) {
@@ -704,6 +706,7 @@ __device__ __forceinline__ void expand_group(const PrepArgs &args, int64_t g, fl
             D0 = D0 + D[n];
             D1 = D1 + tau * D[n];
             D2 = D2 + (t2 + 1.0f / 12.0f) * D[n];
+            D3 = D3 + (tau * (t2 + 0.25f)) * D[n];
             D4 = D4 + (t2 * t2 + 0.5f * t2 + 1.0f / 80.0f) * D[n];
             C += cross(d[n], D[n]);
             sD += size1(D[n]);
@@ -714,7 +717,11 @@ __device__ __forceinline__ void expand_group(const PrepArgs &args, int64_t g, fl
         n5 = n5 + static_cast<float>(k4 * i * 7.0 * G4 / 5760.0) * D0 -
              static_cast<float>(k4 * i * G2 / 48.0) * D2 + static_cast<float>(k4 * i / 24.0) * D4;
         u2 = u2 - static_cast<float>(k * i) * D1;
-        wide += static_cast<float>(i) * sD * (s * eps + 0.03f * e7);
+        u4 = u4 + static_cast<float>(k4 / 12.0) * D3 - static_cast<float>(k4 * G2 / 48.0) * D1;
+        // the next orders of D: z^7 along sigma_z; z^6 in the plane, whose coefficient is
+        // at most 0.0065 whatever the D's signs; and D with D, (sD/G)^2 |S|^3
+        const float mD = static_cast<float>(i) * sD;
+        wide += mD * (s * eps + 0.03f * e7 + 0.01f * e3 * e3) + 0.25f * mD * mD * e3;
     }
     // (the next power of K S, fitted to smooth pulses, at half the box's x)
     const float kk = static_cast<float>(k) * (1.0f + 0.08f * X);
