@@ -556,33 +556,47 @@ int64_t f64_tiles(const ReqDesc &r, int lanes)
     return lanes == 0 ? row_tiles(r, 4) : (r.n_points + 32 / lanes - 1) / (32 / lanes);
 }
 
-// Shape of an FP64 launch (launch_evolve_f64's lanes) by the FP64 work of its fullest
-// scheduler (dsp_f64.cu), in units of 33 ns per step: 32 points flat, 4 rows x 32 columns
-// (EXACT, STRANG_XY), or 8 points on a warp pair.  `cost` is a tile's share of a busy
-// scheduler, its FP64 instructions and, for pairs, the waits between the two warps;
-// `alone` what a step takes when a scheduler has one tile, whose operators then wait for
-// its own updates.  Both measured, on grids of 16^2 to 512^2: EXACT flat at 0.8 and 2.5
-// tiles a scheduler 27.6 and 18.1, rows 93 and 64.7, pairs 6.1 and 4.8.
+// A tile's share of a busy scheduler per step of an FP64 launch (launch_evolve_f64's
+// lanes), in units of 33 ns: its FP64 instructions and, for pairs, the waits between the
+// two warps; n = the series' degrees together.  Measured on grids of 16^2 to 512^2, 1000
+// steps, n of 6 to 12, to within 1%.  EXACT forms its series in FP32: no n.
+double f64_cost(const ReqDesc &r, int lanes)
+{
+    const int n = dsp::kLevelsF64[r.level].dc + dsp::kLevelsF64[r.level].ds;
+    if (r.scheme == DSP_SCHEME_EXACT)
+        return lanes == 1 ? 18.0 : lanes == 0 ? 64.2 : 4.55;
+    if (r.scheme == DSP_SCHEME_STRANG_XY)
+        return lanes == 1 ? 20.9 + 2.23 * n : lanes == 0 ? 60.6 + 1.25 * n : 5.3 + 0.555 * n;
+    return lanes == 1 ? 26.4 + 1.12 * n : 6.7 + 0.28 * n;
+}
+
+// Shape of an FP64 launch by the FP64 work of its fullest scheduler (dsp_f64.cu): 32
+// points flat, 4 rows x 32 columns (EXACT, STRANG_XY), or 8 points on a warp pair.
+// `alone` is what an EXACT step takes when a scheduler has one tile, whose operators then
+// wait for its own updates (the other schemes' operators are FP64 work themselves, in
+// f64_cost).
 int f64_lanes(const std::vector<ReqDesc> &reqs, int scheme)
 {
-    struct Shape {
-        int lanes;
-        double cost[3], alone[3];  // EXACT, STRANG_XY, MAGNUS4 (0: no such kernel)
-    };
-    constexpr Shape shapes[3] = {{1, {18.2, 24.2, 26.2}, {27.5, 39.0, 38.5}},
-                                 {0, {65.0, 62.0, 0.0}, {93.0, 72.0, 0.0}},
-                                 {4, {4.8, 6.6, 6.9}, {6.0, 10.0, 9.0}}};
+    constexpr int shapes[3] = {1, 0, 4};
+    constexpr double alone[3] = {26.6, 84.6, 5.5};
     int best = 1;
     double best_t = 0.0;
-    for (const Shape &sh : shapes) {
-        if (sh.cost[scheme] == 0.0)
+    for (int k = 0; k < 3; ++k) {
+        const int lanes = shapes[k];
+        if (lanes == 0 && scheme == DSP_SCHEME_MAGNUS4)
             continue;
         int64_t tiles = 0;
-        for (const ReqDesc &r : reqs)
-            tiles += f64_tiles(r, sh.lanes);
-        const double t = std::max(sh.alone[scheme], launch_time(tiles, sh.cost[scheme]));
-        if (sh.lanes == 1 || t < 0.99 * best_t) {
-            best = sh.lanes;
+        double work = 0.0;
+        for (const ReqDesc &r : reqs) {
+            tiles += f64_tiles(r, lanes);
+            work += static_cast<double>(f64_tiles(r, lanes)) * f64_cost(r, lanes);
+        }
+        if (tiles == 0)
+            break;
+        const double t = std::max(scheme == DSP_SCHEME_EXACT ? alone[k] : 0.0,
+                                  launch_time(tiles, work / static_cast<double>(tiles)));
+        if (lanes == 1 || t < 0.99 * best_t) {
+            best = lanes;
             best_t = t;
         }
     }

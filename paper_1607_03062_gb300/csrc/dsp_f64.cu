@@ -24,7 +24,8 @@ struct F64Point {
 // The small parts m = cos(theta) - 1 and s1 = sin(theta)/theta - 1 of theta^2 =
 // |dt P|^2 are evaluated in double-float FP32 arithmetic (pairs of floats, ~2^-46
 // relative): being small (~theta^2/2, ~theta^2/6), they come out to ~1e-19
-// absolute, far below an FP64 ulp of the state, so the step is FP64-accurate.
+// absolute at theta 0.005 (below theta^2 2^-47, 7e-17 at 0.1): below an FP64 ulp of the
+// state.
 // FP64 operations per spinor-step: 2 (dt P) + 2 (m, s1 to double) + 2 (q) + 12
 // (update) = 18 instead of 18 + dc + ds; the ~100 FP32 operations of the series
 // issue beside them.
@@ -102,42 +103,21 @@ __device__ __forceinline__ double horner_f64(double x)
         return fma(horner_f64<D, K + 1, ODD>(x), x, c);
 }
 
-// STRANG_XY and MAGNUS4 form their small parts in double-float up to this cosine
-// degree (theta below ~0.2, where their ~2^-46 relative error is below an FP64 ulp of
-// the state), in FP64 above.
-constexpr int kDfDegree = 5;
-
-// The FP64 MAGNUS4 step in the same way: n = (dt Pbar, n_z), n_z = Pbar x D, |n|^2 and
-// the small parts in double-float (kDfDegree), the update and q in FP64.  26 FP64
-// operations where the FP64 series took 26 + dc + ds.
+// The FP64 MAGNUS4 step's operator: n = (dt Pbar, n_z), n_z = Pbar x D; c = cos|n|, q and
+// qz = sinc|n| n, all in FP64: 26 + dc + ds FP64 operations a step.  (Its small parts as
+// pairs of floats, 26, are off by ~2^-50 of theta^2/2 with one sign: 1e5 steps at theta
+// 0.06 put 1.6e-13 into the state instead of 1.7e-14.)
 template <int DC, int DS>
 __device__ __forceinline__ void operator_f64_magnus(double Px, double Py, double2 d, double &c,
                                                     double &qr, double &qi, double &qz)
 {
     const double nz = fma(Px, d.y, -(Py * d.x));
-    if constexpr (DC <= kDfDegree) {
-        const float2 px2 = square_df(Px), py2 = square_df(Py), nz2 = square_df(nz);
-        float xh = px2.x, xl = px2.y;
-        df_add(xh, xl, py2.x, py2.y);
-        df_add(xh, xl, nz2.x, nz2.y);  // |n|^2
-        float th, tl, uh, ul;
-        horner_df<DC, 1, 0>(xh, xl, th, tl);
-        df_mul(xh, xl, th, tl, uh, ul);
-        c = 1.0 + df_to_f64(uh, ul);
-        horner_df<DS, 1, 1>(xh, xl, th, tl);
-        df_mul(xh, xl, th, tl, uh, ul);
-        const double s1 = df_to_f64(uh, ul);
-        qr = fma(s1, Py, Py);
-        qi = fma(s1, Px, Px);
-        qz = fma(s1, nz, nz);
-    } else {
-        const double x = fma(Px, Px, fma(Py, Py, nz * nz));
-        c = horner_f64<DC, 0, 0>(x);
-        const double sn = horner_f64<DS, 0, 1>(x);
-        qr = sn * Py;
-        qi = sn * Px;
-        qz = sn * nz;
-    }
+    const double x = fma(Px, Px, fma(Py, Py, nz * nz));
+    c = horner_f64<DC, 0, 0>(x);
+    const double sn = horner_f64<DS, 0, 1>(x);
+    qr = sn * Py;
+    qi = sn * Px;
+    qz = sn * nz;
 }
 template <int DC, int DS>
 __device__ __forceinline__ void step_f64_magnus(F64Point &s, double Px, double Py, double2 d)
@@ -145,8 +125,7 @@ __device__ __forceinline__ void step_f64_magnus(F64Point &s, double Px, double P
     double c, qr, qi, qz;
     operator_f64_magnus<DC, DS>(Px, Py, d, c, qr, qi, qz);
     // a' = (c - i qz) a - q b ; b' = conj(q) a + (c + i qz) b, q = qr + i qi: the small
-    // terms first, one rounding at the state's size (from psi + m psi each term would
-    // round there: 1.2 to 1.6 times the error over 12000 and 50000 steps)
+    // terms first, one rounding at the state's size
     const double nar = fma(c, s.ar, fma(qz, s.ai, fma(-qr, s.br, qi * s.bi)));
     const double nai = fma(c, s.ai, fma(-qz, s.ar, fma(-qr, s.bi, -(qi * s.br))));
     const double nbr = fma(c, s.br, fma(-qz, s.bi, fma(qr, s.ar, qi * s.ai)));
@@ -164,26 +143,15 @@ __device__ __forceinline__ void apply_f64(F64Point &s, double c, double qr, doub
     s.ar = nar; s.ai = nai; s.br = nbr; s.bi = nbi;
 }
 
-// STRANG_XY's parts of one coordinate: {cos P, sin P} (the small parts by kDfDegree);
-// and its step from those of x and y, c = cos y cos x, q = sin y + i cos y sin x.  24
-// FP64 operations where the FP64 series took 20 + 2 dc + 2 ds; on row tiles the parts
-// of a row and of a column are formed once.
+// STRANG_XY's parts of one coordinate, {cos P, sin P}, in FP64 (as MAGNUS4's; pairs of
+// floats put 1.6e-13 instead of 2.2e-14 into the state there); and its step from those of
+// x and y, c = cos y cos x, q = sin y + i cos y sin x.  20 + 2 dc + 2 ds FP64 operations;
+// on row tiles the parts of a row and of a column are formed once.
 template <int DC, int DS>
 __device__ __forceinline__ double2 strang_part(double P)
 {
-    if constexpr (DC <= kDfDegree) {
-        const float2 x = square_df(P);
-        float th, tl, uh, ul;
-        horner_df<DC, 1, 0>(x.x, x.y, th, tl);
-        df_mul(x.x, x.y, th, tl, uh, ul);
-        const double c1 = df_to_f64(uh, ul);
-        horner_df<DS, 1, 1>(x.x, x.y, th, tl);
-        df_mul(x.x, x.y, th, tl, uh, ul);
-        return make_double2(1.0 + c1, fma(df_to_f64(uh, ul), P, P));
-    } else {
-        const double x = P * P;
-        return make_double2(horner_f64<DC, 0, 0>(x), P * horner_f64<DS, 0, 1>(x));
-    }
+    const double x = P * P;
+    return make_double2(horner_f64<DC, 0, 0>(x), P * horner_f64<DS, 0, 1>(x));
 }
 __device__ __forceinline__ void step_f64_strang(F64Point &s, double2 x, double2 y)
 {
@@ -253,12 +221,12 @@ __device__ __forceinline__ void strip64_step(F64Point (&pt)[H], double tx, doubl
 // Warps (in one shape, pairs of warps) work alone: their own double-buffered bulk copies
 // of the table with bounded waits, no CTA-wide barrier, and the host picks the shape that
 // loads the fullest scheduler least (f64_lanes in dsp_api.cpp).  FP64 instructions per
-// step of a tile (EXACT, STRANG_XY, MAGNUS4) and its points:
+// step of a tile (EXACT; STRANG_XY and MAGNUS4 at series degrees 4 and 3) and its points:
 //   rows   32 columns x 4 rows: the dt P_x part once per lane, the dt P_y part once per
-//          row and step in a shared table                       65, 62, - for 128
-//   flat   32 consecutive points, a lane each                   18, 24, 26 for 32
+//          row and step in a shared table                       65, 67, - for 128
+//   flat   32 consecutive points, a lane each                   18, 34, 33 for 32
 //   pair   8 points, a lane per real component in one warp, the operators of four
-//          steps at once in the other                           4.5, 6, 6.5 for 8
+//          steps at once in the other                           4.5, 8.5, 8.3 for 8
 // Every FP64 operation of a point is the same in every shape (same operands, same
 // rounding), so its result is bitwise the same.  The projection is the projection
 // kernel's, on the state these leave.
