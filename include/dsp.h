@@ -61,8 +61,9 @@ typedef int32_t dsp_status;
                             (7e-17 at theta = 0.1, an ulp of the state at 0.18)     */
 #define DSP_FP32_MIXED 1 /* spinor in compensated FP32 (hi + lo); dt P_n formed as
                             dt p_hi + (dt A_n + dt p_lo) with dt p an FP32 hi/lo
-                            pair and dt A_n one FP32 per step, rounded on the host
-                            with error feedback; the trigonometric factors of
+                            pair and dt A_n one FP32 per step, rounded so that
+                            their running sum stays within half an ulp of the
+                            exact one; the trigonometric factors of
                             the phase argument dt|P| (cos/sin series, or the tan
                             series of step groups) in FP32; initial state in FP64 */
 

@@ -62,7 +62,8 @@ def _stale(lib: str = LIB) -> bool:
         return True
     t = os.path.getmtime(lib)
     deps = sources() + [os.path.join(CSRC, h) for h in ("dsp_internal.h", "dsp_df.cuh",
-                                                        "dsp_device.cuh")] + [
+                                                        "dsp_device.cuh",
+                                                        "dsp_steptable.h")] + [
                         os.path.join(INCLUDE, "dsp.h"),
                         os.path.abspath(__file__)]
     return any(os.path.getmtime(d) > t for d in deps)

@@ -21,6 +21,7 @@
 
 #include "dsp.h"
 #include "dsp_internal.h"
+#include "dsp_steptable.h"
 
 using dsp::EvolveArgs;
 using dsp::FinalizeArgs;
@@ -287,12 +288,14 @@ int32_t first_group_size(double theta_max)
 }
 
 // Layout of a grid's expanded-group memory: what one copy uploads (the caller's table
-// in FP64, the sums as zeros, the projection nodes), then the entries of every group
-// size it may use.
+// in FP64, its running sums, the groups' sums as zeros, the projection nodes), then the
+// entries of every group size it may use.
 struct GroupMemory {
-    size_t raw_bytes, node_bytes, entry_bytes;
+    size_t raw_bytes, prefix_bytes, node_bytes, entry_bytes;
     explicit GroupMemory(const dsp_grid *g)
         : raw_bytes((g->scheme == DSP_SCHEME_MAGNUS4 ? 32 : 16) * static_cast<size_t>(g->n_steps)),
+          prefix_bytes(16 * (static_cast<size_t>(g->n_steps + dsp::kTableBlock - 1) /
+                                 dsp::kTableBlock + 1)),
           node_bytes((sizeof(float2) * (static_cast<size_t>(g->nx) + static_cast<size_t>(g->ny)) +
                       15) & ~static_cast<size_t>(15)),
           entry_bytes(0)
@@ -302,10 +305,11 @@ struct GroupMemory {
                 sizeof(dsp::GroupEntry) * static_cast<size_t>(g->n_steps / dsp::group_size(i));
     }
     static constexpr size_t kSums = 64;
-    size_t upload() const { return raw_bytes + kSums + node_bytes; }
+    size_t upload() const { return nodes() + node_bytes; }
     size_t total() const { return upload() + entry_bytes; }
-    size_t sums() const { return raw_bytes; }
-    size_t nodes() const { return raw_bytes + kSums; }
+    size_t prefix() const { return raw_bytes; }
+    size_t sums() const { return raw_bytes + prefix_bytes; }
+    size_t nodes() const { return sums() + kSums; }
     size_t entries() const { return upload(); }
 };
 static_assert(sizeof(dsp::GroupSums) <= GroupMemory::kSums, "the sums' slot");
@@ -1009,7 +1013,7 @@ dsp_status create_grid_impl(int32_t nx, int32_t ny, double px_min, double px_max
 // piece rule of dsp_evolve) allow it, a group size is within the expansion's angle, the
 // rows fill a good part of the kernel's 32 columns (below 8 columns the step-by-step
 // kernels' contiguous tiles do less work than a quarter-filled warp), and the memory
-// (67 bytes a step and less) stays small.
+// (68 bytes a step and less) stays small.
 bool may_expand(const dsp_grid *g)
 {
     return g->group > 1 && g->nx >= 8 &&
@@ -1050,7 +1054,9 @@ dsp_status prepare_pulse(dsp_grid *g, const double *a_mid, int64_t n_steps, doub
     if (g->by_groups) {
         const GroupMemory m(g);
         host.alloc(m.upload());
-        std::memcpy(host.data(), a_mid, m.raw_bytes);
+        dsp::copy_with_prefix(a_mid, n_steps, samples_per_step(g->scheme),
+                              reinterpret_cast<double *>(host.data()),
+                              reinterpret_cast<double *>(host.data() + m.prefix()));
         std::memset(host.data() + m.sums(), 0, m.kSums);
         build_nodes(g, reinterpret_cast<float2 *>(host.data() + m.nodes()));
     } else {
@@ -1077,6 +1083,7 @@ cudaError_t prep_groups(const dsp_grid *g, cudaStream_t stream)
     a.eps = static_cast<float>(dsp::group_size(0) * g->theta_max);
     a.table = g->table;
     unsigned char *base = static_cast<unsigned char *>(g->groups);
+    a.prefix = reinterpret_cast<const double *>(base + m.prefix());
     a.entries = reinterpret_cast<dsp::GroupEntry *>(base + m.entries());
     a.sums = reinterpret_cast<dsp::GroupSums *>(base + m.sums());
     return dsp::launch_prep_groups(a, stream);

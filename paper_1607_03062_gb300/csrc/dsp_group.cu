@@ -2,6 +2,7 @@
 // that expands a pulse's groups.  Shared device code is in dsp_device.cuh.
 
 #include "dsp_device.cuh"
+#include "dsp_steptable.h"
 
 namespace dsp {
 namespace {
@@ -592,8 +593,8 @@ static_assert(kGroupWarps * sizeof(WarpSmem) <= 48 * 1024, "dynamic shared memor
 // 1.2 where a group drops less than 1e-9).
 //
 // One thread per group, and one per 16 steps for the per-step table (dt A rounded
-// to FP32 with error feedback inside the 16); FP64 only where the group's sum and
-// mean need it.  A 1e5-step table takes microseconds, where the host took 18 ns a step.
+// to FP32 so that its running sum keeps to the exact one, dsp_steptable.h); FP64 only
+// where those sums and the group's mean need it.  A 1e5-step table takes microseconds, where the host took 18 ns a step.
 // ---------------------------------------------------------------------------
 
 struct F2 {
@@ -798,24 +799,21 @@ __global__ void __launch_bounds__(kPrepThreads) prep_groups_kernel(const __grid_
         add_estimate(&a.sums->lite[what], lite);
         return;
     }
-    // dt A per step, rounded to FP32 with error feedback inside 16 steps
-    float rx = 0.0f, ry = 0.0f;
-    for (int64_t n = kGroupMax * g; n < kGroupMax * (g + 1) && n < a.n_steps; ++n) {
-        const StepA s = step_potential(a, n);
-        float h, l;
-        split_f64(s.x, h, l);
-        rx = __fadd_rn(l, rx);
-        const float fx = __fadd_rn(h, rx);
-        rx = __fadd_rn(__fadd_rn(h, -fx), rx);
-        split_f64(s.y, h, l);
-        ry = __fadd_rn(l, ry);
-        const float fy = __fadd_rn(h, ry);
-        ry = __fadd_rn(__fadd_rn(h, -fy), ry);
-        if (a.scheme == 2)
-            static_cast<float4 *>(a.table)[n] = make_float4(fx, fy, s.D.x, s.D.y);
-        else
-            static_cast<float2 *>(a.table)[n] = make_float2(fx, fy);
-    }
+    // dt A per step, rounded to FP32 (table_block)
+    if (kTableBlock * g >= a.n_steps)
+        return;
+    const double half = a.scheme == 2 ? 0.5 * a.sdt : a.sdt;  // times the sum of the samples
+    const double2 s0 = reinterpret_cast<const double2 *>(a.prefix)[g];
+    const double2 s1 = reinterpret_cast<const double2 *>(a.prefix)[g + 1];
+    table_block(g, a.n_steps, __dmul_rn(half, s0.x), __dmul_rn(half, s0.y),
+                __dmul_rn(half, s1.x), __dmul_rn(half, s1.y),
+                [&](int64_t k) { return step_potential(a, k); },
+                [&](int64_t k, const StepA &s, float fx, float fy) {
+                    if (a.scheme == 2)
+                        static_cast<float4 *>(a.table)[k] = make_float4(fx, fy, s.D.x, s.D.y);
+                    else
+                        static_cast<float2 *>(a.table)[k] = make_float2(fx, fy);
+                });
 }
 
 }  // namespace

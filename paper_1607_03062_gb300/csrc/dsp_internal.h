@@ -114,6 +114,7 @@ struct GroupTable {
 
 struct PrepArgs {
     const double *raw;  // the caller's table: (A_x, A_y) per step, MAGNUS4 two per step
+    const double *prefix;  // its running sums (copy_with_prefix)
     int64_t n_steps;
     double sdt;         // valley * dt
     int32_t scheme;
