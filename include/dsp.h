@@ -404,8 +404,9 @@ typedef struct {
 #define DSP_REQ_CANCELLED 4
 
 /* hbm_budget_bytes > 0: admission limit on the sum of device footprints
- * (state + table + map + partial sums; the expanded step groups of a request, at
- * most 67 bytes a step, are not counted) of the active requests; max_active
+ * (state + table + map + partial sums, and the expanded step groups of a request, at
+ * most 68 bytes a step; a request that fits the budget only without them goes step
+ * by step) of the active requests; max_active
  * >= 1; chunk_steps >= 1: steps per batched launch, rounded down to a multiple
  * of 16 when it is 16 or more (a request's result is then bitwise the same alone
  * or in any mix, see dsp_evolve).

@@ -1021,6 +1021,18 @@ bool may_expand(const dsp_grid *g)
            GroupMemory(g).total() <= (static_cast<size_t>(4) << 30);
 }
 
+// What follows from a pulse's length and theta_max: series degrees, step groups, and
+// whether they may be evaluated expanded.
+void choose_steps(dsp_grid *g, int64_t n_steps, double theta_max)
+{
+    g->n_steps = n_steps;
+    g->theta_max = theta_max;
+    g->level = choose_level(g->precision, theta_max, n_steps);
+    g->tdeg = g->precision == DSP_FP32_MIXED ? choose_tan_degree(g->scheme, theta_max, n_steps) : 0;
+    g->group = choose_group(g->precision, g->scheme, g->tdeg, theta_max);
+    g->by_groups = g->expand && may_expand(g);
+}
+
 // Host part of setting a pulse: validates, fills the grid's pulse fields, and lays out
 // in `host` what is uploaded: for expanded groups GroupMemory's upload (the device makes
 // the per-step table from it), else the per-step table, padded to 16 bytes, and the
@@ -1035,22 +1047,16 @@ dsp_status prepare_pulse(dsp_grid *g, const double *a_mid, int64_t n_steps, doub
     if (s != DSP_OK)
         return s;
     g->has_pulse = true;
-    g->n_steps = n_steps;
     g->cursor = 0;
     g->dt = dt;
     g->a_in[0] = a_in[0];
     g->a_in[1] = a_in[1];
     g->a_out[0] = a_out[0];
     g->a_out[1] = a_out[1];
-    g->theta_max = tmax;
-    g->level = choose_level(g->precision, tmax, n_steps);
-    g->tdeg = g->precision == DSP_FP32_MIXED ? choose_tan_degree(g->scheme, tmax, n_steps) : 0;
-    g->group = choose_group(g->precision, g->scheme, g->tdeg, tmax);
+    choose_steps(g, n_steps, tmax);
     g->fresh = true;
     g->projected = false;
     g->state_stale = false;
-    // groups that the grid's piece rule allows may be evaluated expanded
-    g->by_groups = g->expand && may_expand(g);
     if (g->by_groups) {
         const GroupMemory m(g);
         host.alloc(m.upload());
@@ -1882,7 +1888,8 @@ struct ServerReq {
     void *block = nullptr;    // one pool allocation: state | table, nodes, groups | partials |
                               // scalars | map
     void *map_dev = nullptr;
-    int64_t footprint = 0;
+    int64_t footprint = 0;    // bytes of `block`
+    bool expand = true;       // its groups may be expanded: their memory is within the budget
     int64_t finish_iter = -1;  // iteration whose launch holds the last steps
     bool cancel_pending = false;
     int32_t slot = -1;                   // index into the server's pinned result slots
@@ -1892,17 +1899,22 @@ struct ServerReq {
 
 size_t align256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
 
-int64_t footprint_of(const dsp_request &p)
-{
-    const int64_t pts = static_cast<int64_t>(p.nx) * p.ny;
-    const int64_t parts = (pts + dsp::kGranule - 1) / dsp::kGranule;
-    const size_t nodes = sizeof(float2) * (static_cast<size_t>(p.nx) + static_cast<size_t>(p.ny));
-    return static_cast<int64_t>(align256(32 * static_cast<size_t>(pts)) +
-                                align256(table_bytes(p.precision, p.scheme, p.n_steps) + nodes) +
-                                align256(8 * static_cast<size_t>(parts)) +
-                                align256(sizeof(DeviceScalars)) +
-                                align256(map_elem_bytes(p.precision) * static_cast<size_t>(pts)));
-}
+// Layout of a request's device block.
+struct RequestMemory {
+    size_t table, upload, partials, scalars, map, total;  // offsets (the state is at 0)
+    // `g` after choose_steps.  With expanded groups the table, which the device fills, comes first, then the groups' memory.
+    explicit RequestMemory(const dsp_grid &g)
+    {
+        const size_t pts = static_cast<size_t>(g.n_points);
+        const size_t tb = table_bytes(g.precision, g.scheme, g.n_steps);
+        table = align256(32 * pts);
+        upload = table + (g.by_groups ? tb : 0);
+        partials = table + align256(tb + (g.by_groups ? GroupMemory(&g).total() : node_bytes(&g)));
+        scalars = partials + align256(8 * static_cast<size_t>(g.n_parts));
+        map = scalars + align256(sizeof(DeviceScalars));
+        total = map + align256(map_elem_bytes(g.precision) * pts);
+    }
+};
 
 }  // namespace
 
@@ -1944,14 +1956,13 @@ void server_release(dsp_server *s, ServerReq *r)
     }
     r->map_dev = nullptr;
     s->used -= r->footprint;
-    r->footprint = 0;
 }
 
 // Allocates from the pool and queues the table upload of one request.
-dsp_status server_admit(dsp_server *s, ServerReq *r, bool expand = true)
+dsp_status server_admit(dsp_server *s, ServerReq *r)
 {
     const dsp_request &p = r->p;
-    r->g.expand = expand;
+    r->g.expand = r->expand;
     fill_grid(&r->g, p.nx, p.ny, p.px_min, p.px_max, p.py_min, p.py_max, p.precision, p.scheme,
               p.valley, s->stream);
     HostBytes host;
@@ -1959,36 +1970,30 @@ dsp_status server_admit(dsp_server *s, ServerReq *r, bool expand = true)
     if (st != DSP_OK)
         return st;
     r->g.keep_final_state = false;  // a finished request's state is never read again
-    // One copy uploads the table and the projection nodes, or what the expanded groups
-    // start from, which then lies behind the table that the device fills.
-    const size_t tb = table_bytes(p.precision, p.scheme, p.n_steps);
+    // one copy uploads the table and the projection nodes, or what the expanded groups
+    // start from
+    const RequestMemory m(r->g);
     const bool by_groups = r->g.by_groups;
-    const size_t o_up = by_groups ? tb : 0;  // where the upload lands after o_table
-    const size_t region = by_groups ? tb + GroupMemory(&r->g).total() : host.size();
+    const size_t tb = table_bytes(p.precision, p.scheme, p.n_steps);
     const size_t pts = static_cast<size_t>(r->g.n_points);
-    const size_t o_table = align256(32 * pts);
-    const size_t o_part = o_table + align256(region);
-    const size_t o_scal = o_part + align256(8 * static_cast<size_t>(r->g.n_parts));
-    const size_t o_map = o_scal + align256(sizeof(DeviceScalars));
-    const size_t total = o_map + align256(map_elem_bytes(p.precision) * pts);
     // allocated in stream order on the copy stream, so the upload does not wait for
     // the iteration in flight on the compute stream; the compute stream waits for
     // the upload before its first use, and frees the block after its last use
     void *block = nullptr;
-    if (cudaMallocAsync(&block, total, s->copy_stream) != cudaSuccess) {
+    if (cudaMallocAsync(&block, m.total, s->copy_stream) != cudaSuccess) {
         cudaGetLastError();
-        return by_groups ? server_admit(s, r, false) : DSP_E_NOMEM;
+        return DSP_E_NOMEM;
     }
     unsigned char *b = static_cast<unsigned char *>(block);
     r->block = block;
     r->g.state = b;
-    r->g.table = b + o_table;
+    r->g.table = b + m.table;
     r->g.table_cap = p.n_steps;
-    r->g.nodes = by_groups ? nullptr : reinterpret_cast<float2 *>(b + o_table + tb);
-    r->g.groups = by_groups ? b + o_table + tb : nullptr;
-    r->g.partials = reinterpret_cast<double *>(b + o_part);
-    r->g.scal = reinterpret_cast<DeviceScalars *>(b + o_scal);
-    r->map_dev = b + o_map;
+    r->g.nodes = by_groups ? nullptr : reinterpret_cast<float2 *>(b + m.table + tb);
+    r->g.groups = by_groups ? b + m.upload : nullptr;
+    r->g.partials = reinterpret_cast<double *>(b + m.partials);
+    r->g.scal = reinterpret_cast<DeviceScalars *>(b + m.scalars);
+    r->map_dev = b + m.map;
     if (p.keep_map && !r->map_host) {
         if (cudaMallocHost(&r->map_host, map_elem_bytes(p.precision) * pts) != cudaSuccess) {
             cudaGetLastError();
@@ -2013,14 +2018,13 @@ dsp_status server_admit(dsp_server *s, ServerReq *r, bool expand = true)
             s->staging_cap = host.size();
         }
         std::memcpy(s->staging, host.data(), host.size());
-        if (cudaMemcpyAsync(b + o_table + o_up, s->staging, host.size(), cudaMemcpyHostToDevice,
+        if (cudaMemcpyAsync(b + m.upload, s->staging, host.size(), cudaMemcpyHostToDevice,
                             s->copy_stream) != cudaSuccess ||
             (by_groups && prep_groups(&r->g, s->copy_stream) != cudaSuccess) ||
             cudaEventRecord(s->upload_done, s->copy_stream) != cudaSuccess ||
             cudaStreamWaitEvent(s->stream, s->upload_done, 0) != cudaSuccess)
             return server_fail(s, DSP_E_CUDA);
     }
-    r->footprint = footprint_of(p);
     s->used += r->footprint;
     r->state = DSP_REQ_ACTIVE;
     std::vector<double>().swap(r->a_mid);  // the device holds the table now
@@ -2101,22 +2105,31 @@ dsp_status dsp_server_submit(dsp_server *s, const dsp_request *req, const double
         return st;
     if (p.keep_map != 0 && p.keep_map != 1)
         return DSP_E_INVALID;
-    dsp_grid probe;  // only the box matters for the step condition
-    probe.px_min = p.px_min;
-    probe.px_max = p.px_max;
-    probe.py_min = p.py_min;
-    probe.py_max = p.py_max;
+    dsp_grid probe;
+    fill_grid(&probe, p.nx, p.ny, p.px_min, p.px_max, p.py_min, p.py_max, p.precision, p.scheme,
+              p.valley, s->stream);
     const int64_t n_samples = p.n_steps * samples_per_step(p.scheme);
-    st = validate_pulse_args(&probe, a_mid, n_samples, p.dt, p.a_in, p.a_out);
+    double tmax = 0.0;
+    st = validate_pulse_args(&probe, a_mid, n_samples, p.dt, p.a_in, p.a_out, &tmax);
     if (st != DSP_OK)
         return st;
-    if (footprint_of(p) > s->budget)
+    // The request's own footprint and the budget decide whether its groups may be expanded,
+    // not what else is active: its result is the same alone and in any mix.
+    choose_steps(&probe, p.n_steps, tmax);
+    size_t footprint = RequestMemory(probe).total;
+    if (probe.by_groups && footprint > static_cast<size_t>(s->budget)) {
+        probe.by_groups = probe.expand = false;
+        footprint = RequestMemory(probe).total;
+    }
+    if (footprint > static_cast<size_t>(s->budget))
         return DSP_E_NOMEM;
     std::unique_ptr<ServerReq> r(new (std::nothrow) ServerReq());
     if (!r)
         return DSP_E_NOMEM;
     r->id = static_cast<int64_t>(s->reqs.size());
     r->p = p;
+    r->footprint = static_cast<int64_t>(footprint);
+    r->expand = probe.expand;
     try {
         r->a_mid.assign(a_mid, a_mid + 2 * n_samples);
     } catch (...) {
@@ -2152,7 +2165,7 @@ dsp_status dsp_server_step(dsp_server *s, int32_t *n_active, int32_t *n_queued,
         Range admit_range_("server admit");
         while (!s->queue.empty() && static_cast<int32_t>(s->active.size()) < s->max_active) {
             ServerReq *r = s->reqs[s->queue.front()].get();
-            if (s->used + footprint_of(r->p) > s->budget)
+            if (s->used + r->footprint > s->budget)
                 break;
             s->queue.pop_front();
             dsp_status st = server_admit(s, r);
