@@ -138,7 +138,11 @@ dsp_status dsp_set_keep_final_state(dsp_grid *g, int32_t keep);
  * each).  All values finite, dt > 0 (dt >= 0 when n_steps == 0), n_steps >= 0.
  * Copies and converts the table to the device, resets the state to
  * v(p + A_in) and the step cursor to 0.  Returns DSP_E_CFL when
- * dt * max_{n, p in box} |p + A_n| > pi (the step condition of Sec. III).
+ * dt * max_{n, p in box} |p + A_n| > pi (the step condition of Sec. III), and
+ * DSP_E_NOMEM when the device has no room for the table (the pulse before is then
+ * gone).  Where it has no room for the expanded step groups (dsp_get_info; at most
+ * 68 bytes a step), the pulse goes step by step: dsp_get_groups then says so, and
+ * the result differs in rounding from one with room.
  * Not ordered against work already queued that still reads the old table:
  * the library orders it on the grid's stream. */
 dsp_status dsp_set_pulse(dsp_grid *g, const double *a_mid, int64_t n_steps, double dt,
@@ -326,6 +330,11 @@ dsp_status dsp_test_tiling(dsp_grid *g, int32_t tiling);
  * rounding; the hook exists so that a test can show it. */
 dsp_status dsp_test_expansion(dsp_grid *g, int32_t on);
 
+/* Test hook (not in the paper): of the device allocations that dsp_set_pulse makes on
+ * this grid (the step groups' memory, then the table's, as far as they have to grow),
+ * the next `skip` go through and `fail` more are answered as if the device were full. */
+dsp_status dsp_test_fail_alloc(dsp_grid *g, int32_t skip, int32_t fail);
+
 /* Copies the raw spinor state (dsp_state_bytes bytes) to the host, or back
  * from the host, with the step cursor, for checkpoint / resume.  Synchronise.
  * Checkpointing only: the paper has no counterpart. */
@@ -425,7 +434,9 @@ dsp_status dsp_server_submit(dsp_server *s, const dsp_request *req, const double
  * launch that advances every admitted request by up to chunk_steps (with the
  * projection, density and result copies of those whose last steps are in it),
  * then waits only for the PREVIOUS iteration and retires the requests that
- * finished there (so the device always has the next iteration queued).  Device
+ * finished there (so the device always has the next iteration queued).  A request
+ * within the budget for which the device has no room waits for the active ones; if
+ * there are none it fails (DSP_REQ_FAILED).  Device
  * memory comes from the stream-ordered pool; nothing blocks on an allocation.
  * Outputs may be NULL: requests admitted and not yet retired, requests still
  * queued, requests retired by this call. */
@@ -441,6 +452,10 @@ dsp_status dsp_server_query(dsp_server *s, int64_t id, int32_t *state, double *d
 /* Cancels a queued or active request; its device memory is freed at the next
  * step.  Other requests are unaffected. */
 dsp_status dsp_server_cancel(dsp_server *s, int64_t id);
+
+/* Test hook (serving only, the paper has no counterpart): dsp_test_fail_alloc for the
+ * device memory of the requests that are admitted next. */
+dsp_status dsp_server_test_fail_alloc(dsp_server *s, int32_t skip, int32_t fail);
 
 /* Frees everything.  NULL is OK.  (Like every dsp_server_* call: serving
  * only, the paper has no counterpart.) */

@@ -41,7 +41,8 @@ EXPORTS = (
     "dsp_server_query", "dsp_server_cancel", "dsp_server_destroy", "dsp_density_noalloc",
     "dsp_get_info", "dsp_solve_segmented", "dsp_sample_pulse_gauss",
     "dsp_test_withhold_next_copy", "dsp_create_band", "dsp_set_keep_final_state",
-    "dsp_test_tiling", "dsp_test_expansion", "dsp_get_groups",
+    "dsp_test_tiling", "dsp_test_expansion", "dsp_get_groups", "dsp_test_fail_alloc",
+    "dsp_server_test_fail_alloc",
 )
 
 
@@ -130,6 +131,8 @@ def lib() -> ctypes.CDLL:
                 "dsp_test_tiling": (i32, [p, i32]),
                 "dsp_test_expansion": (i32, [p, i32]),
                 "dsp_get_groups": (i32, [p, pi32, pi32]),
+                "dsp_test_fail_alloc": (i32, [p, i32, i32]),
+                "dsp_server_test_fail_alloc": (i32, [p, i32, i32]),
             }
             for name, (res, args) in sig.items():
                 fn = getattr(L, name)
@@ -332,6 +335,12 @@ def test_expansion(h: int, on: bool):
     _check(lib().dsp_test_expansion(ctypes.c_void_p(h), 1 if on else 0), "test_expansion")
 
 
+def test_fail_alloc(h: int, skip: int, fail: int):
+    """Test hook: of the device allocations that set_pulse makes on the grid, `skip` go through
+    and the next `fail` are answered as if the device were full."""
+    _check(lib().dsp_test_fail_alloc(ctypes.c_void_p(h), int(skip), int(fail)), "test_fail_alloc")
+
+
 def status_string(code: int) -> str:
     return lib().dsp_status_string(int(code)).decode()
 
@@ -424,6 +433,12 @@ def server_query(s: int, rid: int, map_out: np.ndarray | None = None):
 
 def server_cancel(s: int, rid: int):
     _check(lib().dsp_server_cancel(ctypes.c_void_p(s), int(rid)), "server_cancel")
+
+
+def server_test_fail_alloc(s: int, skip: int, fail: int):
+    """test_fail_alloc for the device memory of the requests admitted next."""
+    _check(lib().dsp_server_test_fail_alloc(ctypes.c_void_p(s), int(skip), int(fail)),
+           "server_test_fail_alloc")
 
 
 def server_destroy(s: int):

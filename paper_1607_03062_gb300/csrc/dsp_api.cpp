@@ -39,6 +39,19 @@ struct Range {
     Range &operator=(const Range &) = delete;
 };
 
+// Test hook (dsp_test_fail_alloc): lets `skip` device allocations through, then fails `fail`.
+struct AllocHook {
+    int32_t skip = 0, fail = 0;
+    bool fails()
+    {
+        if (fail <= 0 || skip-- > 0)
+            return false;
+        --fail;
+        skip = 0;
+        return true;
+    }
+};
+
 struct DeviceScalars {
     double density;
     int err;
@@ -81,6 +94,7 @@ struct dsp_grid {
     bool expand = true;  // test hook, see dsp_test_expansion
     int32_t tdeg = 0;   // FP32_MIXED: tan series degree of the step groups (choose_tan_degree)
     bool withhold_next = false;  // test hook, see dsp_test_withhold_next_copy
+    AllocHook hook;
     bool fresh = true;      // state not yet written on the device
     bool projected = false;  // partial sums valid for the current pulse
     bool keep_final_state = true;  // dsp_set_keep_final_state
@@ -1095,6 +1109,44 @@ cudaError_t prep_groups(const dsp_grid *g, cudaStream_t stream)
     return dsp::launch_prep_groups(a, stream);
 }
 
+// Makes room for `need` bytes at *p, which has room for *cap; need 0 gives it back.  What
+// was there is dropped, and with it the pulse before.
+cudaError_t reserve(dsp_grid *g, void **p, size_t *cap, size_t need)
+{
+    if (need > 0 && need <= *cap)
+        return cudaSuccess;
+    if (*p) {
+        cudaError_t e = cudaStreamSynchronize(g->stream);  // it may still be read
+        if (e == cudaSuccess)
+            e = cudaFree(*p);
+        *p = nullptr;
+        *cap = 0;
+        g->has_pulse = false;
+        if (e != cudaSuccess)
+            return e;
+    }
+    if (need == 0)
+        return cudaSuccess;
+    const cudaError_t e =
+        g->hook.fails() ? cudaErrorMemoryAllocation : cudaMalloc(p, need);
+    if (e != cudaSuccess)
+        *p = nullptr;
+    else
+        *cap = need;
+    return e;
+}
+
+// The same for the table, whose capacity is counted in steps.
+cudaError_t reserve_table(dsp_grid *g, int64_t n_steps)
+{
+    if (n_steps <= g->table_cap)
+        return cudaSuccess;
+    size_t cap = 0;
+    const cudaError_t e = reserve(g, &g->table, &cap, table_bytes(g->precision, g->scheme, n_steps));
+    g->table_cap = e == cudaSuccess ? n_steps : 0;
+    return e;
+}
+
 dsp_status set_pulse_impl(dsp_grid *g, const double *a_mid, int64_t n_steps, double dt,
                           const double a_in[2], const double a_out[2])
 {
@@ -1103,53 +1155,27 @@ dsp_status set_pulse_impl(dsp_grid *g, const double *a_mid, int64_t n_steps, dou
     dsp_status s = prepare_pulse(&staged, a_mid, n_steps, dt, a_in, a_out, host);
     if (s != DSP_OK)
         return s;
+    // the groups' memory first: where the device has no room for it, or for the table
+    // beside it, the pulse goes step by step
     cudaError_t e = cudaSuccess;
-    size_t gbytes = staged.by_groups ? GroupMemory(&staged).total() : 0;
-    if (gbytes > g->groups_cap) {
-        if (g->groups) {
-            e = cudaStreamSynchronize(g->stream);  // the old groups may still be read
-            if (e == cudaSuccess)
-                e = cudaFree(g->groups);
-            g->groups = nullptr;
-            g->groups_cap = 0;
-            g->has_pulse = false;  // the pulse before is gone
-        }
+    if (staged.by_groups)
+        e = reserve(g, &g->groups, &g->groups_cap, GroupMemory(&staged).total());
+    if (e == cudaSuccess)
+        e = reserve_table(g, n_steps);
+    if (e == cudaErrorMemoryAllocation && staged.by_groups) {
+        cudaGetLastError();
+        e = reserve(g, &g->groups, &g->groups_cap, 0);
+        staged.expand = false;
+        s = prepare_pulse(&staged, a_mid, n_steps, dt, a_in, a_out, host);
+        staged.expand = g->expand;
+        if (s != DSP_OK)
+            return s;
         if (e == cudaSuccess)
-            e = cudaMalloc(&g->groups, gbytes);
-        if (e == cudaErrorMemoryAllocation) {  // no room: step by step
-            cudaGetLastError();
-            g->groups = nullptr;
-            gbytes = 0;
-            staged.expand = false;
-            s = prepare_pulse(&staged, a_mid, n_steps, dt, a_in, a_out, host);
-            staged.expand = g->expand;
-            e = cudaSuccess;
-            if (s != DSP_OK)
-                return s;
-        } else if (e != cudaSuccess) {
-            cudaGetLastError();
-            g->groups = nullptr;
-            return latch_cuda(g, e);
-        } else {
-            g->groups_cap = gbytes;
-        }
+            e = reserve_table(g, n_steps);
     }
-    if (n_steps > g->table_cap) {
-        if (g->table) {
-            e = cudaStreamSynchronize(g->stream);  // old table may still be read
-            if (e == cudaSuccess)
-                e = cudaFree(g->table);
-            g->table = nullptr;
-            g->table_cap = 0;
-            g->has_pulse = false;  // the pulse before is gone
-        }
-        if (e == cudaSuccess)
-            e = cudaMalloc(&g->table, table_bytes(g->precision, g->scheme, n_steps));
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            return e == cudaErrorMemoryAllocation ? DSP_E_NOMEM : latch_cuda(g, e);
-        }
-        g->table_cap = n_steps;
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return e == cudaErrorMemoryAllocation ? DSP_E_NOMEM : latch_cuda(g, e);
     }
     if (staged.by_groups) {
         e = cudaMemcpyAsync(g->groups, host.data(), host.size(), cudaMemcpyHostToDevice, g->stream);
@@ -1172,6 +1198,7 @@ dsp_status set_pulse_impl(dsp_grid *g, const double *a_mid, int64_t n_steps, dou
     staged.table_cap = g->table_cap;
     staged.groups = g->groups;
     staged.groups_cap = g->groups_cap;
+    staged.hook = g->hook;
     *g = staged;
     return DSP_OK;
 }
@@ -1568,6 +1595,18 @@ dsp_status dsp_test_expansion(dsp_grid *g, int32_t on)
     return DSP_OK;
 }
 
+dsp_status dsp_test_fail_alloc(dsp_grid *g, int32_t skip, int32_t fail)
+{
+    dsp_status s = check_usable(g);
+    if (s != DSP_OK)
+        return s;
+    if (skip < 0 || fail < 0)
+        return DSP_E_INVALID;
+    g->hook.skip = skip;
+    g->hook.fail = fail;
+    return DSP_OK;
+}
+
 dsp_status dsp_get_groups(dsp_grid *g, int32_t *steps, int32_t *level)
 {
     dsp_status s = check_usable(g);
@@ -1935,6 +1974,7 @@ struct dsp_server {
     std::vector<std::unique_ptr<ServerReq>> reqs;  // by id
     std::deque<int64_t> queue;
     std::vector<int64_t> active;         // admitted, not yet retired
+    AllocHook hook;
     dsp_status latched = DSP_OK;
 };
 
@@ -1980,7 +2020,7 @@ dsp_status server_admit(dsp_server *s, ServerReq *r)
     // the iteration in flight on the compute stream; the compute stream waits for
     // the upload before its first use, and frees the block after its last use
     void *block = nullptr;
-    if (cudaMallocAsync(&block, m.total, s->copy_stream) != cudaSuccess) {
+    if (s->hook.fails() || cudaMallocAsync(&block, m.total, s->copy_stream) != cudaSuccess) {
         cudaGetLastError();
         return DSP_E_NOMEM;
     }
@@ -2169,6 +2209,17 @@ dsp_status dsp_server_step(dsp_server *s, int32_t *n_active, int32_t *n_queued,
                 break;
             s->queue.pop_front();
             dsp_status st = server_admit(s, r);
+            if (st == DSP_E_NOMEM && s->latched == DSP_OK) {
+                // no room on the device within the budget: the request waits for the active
+                // ones (its steps are taken as they would be alone), or for what finished
+                if (!s->active.empty()) {
+                    s->queue.push_front(r->id);
+                    break;
+                }
+                if (cudaStreamSynchronize(s->stream) != cudaSuccess)
+                    return server_fail(s, DSP_E_CUDA);
+                st = server_admit(s, r);
+            }
             if (s->latched != DSP_OK)
                 return s->latched;
             if (st != DSP_OK) {
@@ -2297,6 +2348,15 @@ dsp_status dsp_server_cancel(dsp_server *s, int64_t id)
         return DSP_OK;
     }
     return DSP_E_STATE;
+}
+
+dsp_status dsp_server_test_fail_alloc(dsp_server *s, int32_t skip, int32_t fail)
+{
+    if (!s || skip < 0 || fail < 0)
+        return DSP_E_INVALID;
+    s->hook.skip = skip;
+    s->hook.fail = fail;
+    return DSP_OK;
 }
 
 dsp_status dsp_server_destroy(dsp_server *s)
