@@ -473,7 +473,7 @@ __device__ __forceinline__ bool table_range_ok(const ReqDesc &R, int64_t first, 
 #ifdef DSP_BOUNDS_CHECK
     const bool ok = first >= 0 && R.step_end >= R.step_begin &&
                     (R.step_end == R.step_begin || R.step_end <= R.table_steps);
-    if (!ok && threadIdx.x == 0)
+    if (!ok && (threadIdx.x & 31) == 0)  // a warp may have a tile of its own
         atomicOr(err, kErrBounds);
     return ok;
 #else
@@ -520,12 +520,12 @@ __device__ __forceinline__ bool left_to_groups(const ReqDesc &R)
     return R.by_groups && pick_plan(R.groups).size < kNumGroupSizes;
 }
 
-// Bounds-check builds verify a CTA's tile index; a bad one sets kErrBounds.
+// Bounds-check builds verify a CTA's or a warp's tile index; a bad one sets kErrBounds.
 __device__ __forceinline__ bool tile_ok(const ReqDesc &R, int tile, int *err)
 {
 #ifdef DSP_BOUNDS_CHECK
     const bool ok = tile >= 0 && tile < R.n_tiles;
-    if (!ok && threadIdx.x == 0)
+    if (!ok && (threadIdx.x & 31) == 0)  // a warp may have a tile of its own
         atomicOr(err, kErrBounds);
     return ok;
 #else
