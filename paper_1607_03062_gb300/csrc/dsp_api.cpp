@@ -678,8 +678,9 @@ cudaError_t launch_steps_mixed(const std::vector<ReqDesc> &reqs, cudaStream_t st
 // device errors in its own error word (ReqDesc::err).  The step-by-step FP32_MIXED
 // kernels project in the same launch; the FP64 kernels and the expanded groups leave
 // the projection to a launch of its own over the state they store.  A request whose
-// groups may be evaluated expanded is queued twice: on expanded groups and step by
-// step, and the launch that its pulse's sums do not pick returns at once.
+// groups may be evaluated expanded is queued on expanded groups with that projection
+// behind it, and step by step as if there were no groups; the launches that its pulse's
+// sums do not pick return at once.
 cudaError_t launch_requests(const std::vector<ReqDesc> &given, int precision, cudaStream_t stream)
 {
     std::vector<ReqDesc> steps, grouped, after;
@@ -689,13 +690,18 @@ cudaError_t launch_requests(const std::vector<ReqDesc> &given, int precision, cu
             continue;
         }
         steps.push_back(r);
-        if (precision == DSP_FP64 || r.by_groups) {
-            steps.back().store_state = 1;
-            steps.back().project = 0;
-            if (r.by_groups)
-                grouped.push_back(steps.back());
-            if (r.project)
-                after.push_back(projection_of(r));
+        if (precision != DSP_FP64 && !r.by_groups)
+            continue;
+        ReqDesc stored = r;
+        stored.store_state = 1;
+        stored.project = 0;
+        if (precision == DSP_FP64)
+            steps.back() = stored;
+        else
+            grouped.push_back(stored);
+        if (r.project) {
+            after.push_back(projection_of(r));
+            after.back().by_groups = r.by_groups;
         }
     }
     // (a launch's 27 KB of parameters cost ~0.5 us to allocate and clear: a projection

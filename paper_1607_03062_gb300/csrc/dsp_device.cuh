@@ -514,10 +514,22 @@ __device__ __forceinline__ GroupPick pick_plan(const GroupTable &t)
     return {kNumGroupSizes, kGroupWide};
 }
 // A step-by-step kernel leaves a request of a pair to the expanded groups where the
-// plan picked them.
+// plan picked them: whether pick_plan finds a size, its sums loaded side by side.
 __device__ __forceinline__ bool left_to_groups(const ReqDesc &R)
 {
-    return R.by_groups && pick_plan(R.groups).size < kNumGroupSizes;
+    if (!R.by_groups)
+        return false;
+    constexpr unsigned long long budget =
+        static_cast<unsigned long long>(kPlanBudget / kPlanUnit);
+    unsigned long long sum[kNumGroupSizes];
+#pragma unroll
+    for (int i = 0; i < kNumGroupSizes; ++i)
+        sum[i] = __ldg(&R.groups.sums->wide[i]);
+    bool any = false;
+#pragma unroll
+    for (int i = 0; i < kNumGroupSizes; ++i)
+        any = any || (i >= R.groups.first && R.groups.n_steps >= group_size(i) && sum[i] <= budget);
+    return any;
 }
 
 // Bounds-check builds verify a CTA's or a warp's tile index; a bad one sets kErrBounds.

@@ -175,8 +175,9 @@ struct ReqDesc {
                          // (host only; see split_last_wave)
     int64_t table_steps;          // entries in the table (checked by bounds-check builds)
     GroupTable groups;   // FP32_MIXED expanded groups (entries null: none)
-    int32_t by_groups;   // 1: this launch is one of a pair, on expanded groups or step by
-                         // step: the kernel that the plan does not pick does nothing
+    int32_t by_groups;   // 1: this launch is on expanded groups (or projects behind them)
+                         // or the same steps one by one: what the plan does not pick does
+                         // nothing
     int32_t rows;  // rows per warp asked for by the tiling hook (4, 1); 0: by size
 };
 

@@ -161,6 +161,18 @@ __global__ void __launch_bounds__(ProjShape<PREC>::threads, 1)
     const int total = args.total_tiles * kGranPerTile;  // granules of the launch
     // granules go to the CTAs in turn, so that a small grid's spread over the SMs
     const int wid = w * gridDim.x + blockIdx.x, nw = gridDim.x * Sh::warps;
+    // A request that went step by step has been projected there: nothing to load or to do.
+    // (Looked up once per request: granules of one follow each other.  A warp's first
+    // granule is loaded meanwhile, whatever comes of it.)
+    int seen = -1;
+    bool wanted = true;
+    const auto to_project = [&](int r) {
+        if (r != seen) {
+            seen = r;
+            wanted = !args.r[r].by_groups || left_to_groups(args.r[r]);
+        }
+        return wanted;
+    };
     if (lane == 0) {
         for (int b = 0; b < NB; ++b)
             mbar_init(&bars[b], 1);
@@ -168,15 +180,18 @@ __global__ void __launch_bounds__(ProjShape<PREC>::threads, 1)
     }
     __syncwarp();
     // lane 0 queues both planes of granule Gi into buffer b (whole 16-byte points);
-    // a granule past the end of its grid completes its phase empty
-    const auto issue = [&](int Gi, int b) {
+    // a granule past the end of its grid, or of a request that is not to be projected,
+    // completes its phase empty
+    const auto issue = [&](int Gi, int b, bool first) {
         const int T = Gi / kGranPerTile;
-        const ReqDesc &R = args.r[find_request(args, T)];
+        const int r = find_request(args, T);
+        const ReqDesc &R = args.r[r];
         const int64_t base = static_cast<int64_t>(T - R.tile_begin) * kTilePoints +
                              static_cast<int64_t>(Gi % kGranPerTile) * kGranule;
         const int64_t left = R.n_points - base;
         const uint32_t bytes =
-            left <= 0 ? 0u : 16u * static_cast<uint32_t>(left < kGranule ? left : kGranule);
+            left <= 0 || !(first || to_project(r))
+                ? 0u : 16u * static_cast<uint32_t>(left < kGranule ? left : kGranule);
         mbar_arrive_expect_tx(&bars[b], 2 * bytes);
         if (bytes > 0) {
             const unsigned char *st = static_cast<const unsigned char *>(R.state);
@@ -188,12 +203,14 @@ __global__ void __launch_bounds__(ProjShape<PREC>::threads, 1)
     if (lane == 0)
         for (int b = 0; b < NB; ++b)
             if (wid + b * nw < total)
-                issue(wid + b * nw, b);
+                issue(wid + b * nw, b, true);
     int k = 0;
     for (int Gi = wid; Gi < total; Gi += nw, ++k) {
         const int b = k % NB;
         const int T = Gi / kGranPerTile;
-        const ReqDesc &R = args.r[find_request(args, T)];
+        const int r = find_request(args, T);
+        const ReqDesc &R = args.r[r];
+        const bool project = to_project(r);
         const bool arrived = mbar_wait_bounded(&bars[b], (k / NB) & 1);
         if (!__all_sync(0xffffffffu, arrived)) {
             if (lane == 0) {  // flag it; give the copies still queued a bounded chance to
@@ -206,7 +223,7 @@ __global__ void __launch_bounds__(ProjShape<PREC>::threads, 1)
             return;
         }
         const int tile = T - R.tile_begin;
-        if (tile_ok(R, tile, R.err)) {
+        if (project && tile_ok(R, tile, R.err)) {
             const int64_t gbase = static_cast<int64_t>(tile) * kTilePoints +
                                   static_cast<int64_t>(Gi % kGranPerTile) * kGranule;
             // column and row of the granule's first point (one division per granule)
@@ -286,7 +303,7 @@ __global__ void __launch_bounds__(ProjShape<PREC>::threads, 1)
         }
         __syncwarp();  // the warp is done with buffer b
         if (lane == 0 && Gi + NB * nw < total)
-            issue(Gi + NB * nw, b);
+            issue(Gi + NB * nw, b, false);
     }
 }
 
