@@ -274,7 +274,8 @@ dsp_status dsp_get_cursor(const dsp_grid *g, int64_t *cursor, int64_t *n_steps);
  * operator of 16, 8 or 4 aligned steps at once, from the expansion of their
  * product in what A changes inside the group (its coefficients are formed once
  * per pulse), as long as the terms it drops, summed over the run, stay below
- * 4e-6; pulses too rough for that take the steps one by one as above. */
+ * 4e-6; pulses too rough for that, or too short to gain by it (by nx, the full
+ * grid's size and n_steps alone), take the steps one by one as above. */
 typedef struct {
     int32_t nx, ny, precision, scheme, valley;
     int32_t cos_degree, sinc_degree;

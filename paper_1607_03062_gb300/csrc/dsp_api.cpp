@@ -1029,28 +1029,75 @@ dsp_status create_grid_impl(int32_t nx, int32_t ny, double px_min, double px_max
     return DSP_OK;
 }
 
+// Steps below which a pulse of the grid is not worth expanding.  Expanding adds a launch
+// (10 us) to setting a pulse and two to a solve, and a write and a read of the state for the
+// projection, which the step-by-step kernels make in place.  Solve alone, step by step and
+// expanded (us): row strips 256^2 x 256 57 and 61, x 512 66 and 62, 1024^2 x 4 170 and 178, x 64
+// 191 and 183, 4096^2 x 16 1890 and 2020, x 32 2030 and 2025, x 64 2210 and 2037; contiguous
+// tiles 64^2 x 4 63 and 50, 1000 x 750 x 4 140 and 136.  (The full grid's rows: a band takes the
+// same way.)
+int64_t least_steps(const dsp_grid *g)
+{
+    const int64_t points = static_cast<int64_t>(g->nx) * g->ny_total;
+    if (g->nx % dsp::kStripWidth != 0)
+        return points >= (1 << 20) ? 32 : 1;
+    return std::min<int64_t>(512, std::max<int64_t>(32, (1 << 25) / points));
+}
+
 // Whether the grid's pulse may be evaluated on expanded groups: its step groups (the
 // piece rule of dsp_evolve) allow it, a group size is within the expansion's angle, the
 // rows fill a good part of the kernel's 32 columns (below 8 columns the step-by-step
-// kernels' contiguous tiles do less work than a quarter-filled warp), and the memory
-// (68 bytes a step and less) stays small.
+// kernels' contiguous tiles do less work than a quarter-filled warp), it is long enough,
+// and the memory (68 bytes a step and less) stays small.
 bool may_expand(const dsp_grid *g)
 {
-    return g->group > 1 && g->nx >= 8 &&
+    return g->group > 1 && g->nx >= 8 && g->n_steps >= least_steps(g) &&
            first_group_size(g->theta_max) < dsp::kNumGroupSizes &&
            GroupMemory(g).total() <= (static_cast<size_t>(4) << 30);
 }
 
-// What follows from a pulse's length and theta_max: series degrees, step groups, and
-// whether they may be evaluated expanded.
-void choose_steps(dsp_grid *g, int64_t n_steps, double theta_max)
+// Whether a pulse is so rough throughout that its expansion is sure to be refused, from at
+// most 32 of its groups of 4: half of them are each over twice their share of the budget
+// by two of the terms that the device sums up for every group (expand_group: second and third
+// order in how A changes inside the group).  Such a pulse then costs what it did without
+// groups (64^2 x 500 steps of noise, set and solved: 142 us with the launches that return,
+// 128 without).  Rough places that are few are left to the device's sums.
+bool rough_throughout(const dsp_grid *g, const double *a_mid)
+{
+    const int per = samples_per_step(g->scheme);
+    const int64_t groups = g->n_steps / 4, stride = std::max<int64_t>(1, groups / 32);
+    const double share = 2.0 * dsp::kPlanBudget / static_cast<double>(std::max<int64_t>(groups, 1));
+    const double x = 16.0 * g->theta_max * g->theta_max, scale = g->dt / per;
+    int seen = 0, over = 0;
+    for (int64_t k = 0; k < groups; k += stride, ++seen) {
+        const double *a = a_mid + 8 * per * k;
+        double d[4][2], odd = 0.0, even = 0.0;
+        for (int c = 0; c < 2; ++c) {
+            for (int n = 0; n < 4; ++n)
+                d[n][c] = scale * (a[2 * per * n + c] + (per == 2 ? a[2 * per * n + 2 + c] : 0.0));
+            const double mean = 0.25 * (d[0][c] + d[1][c] + d[2][c] + d[3][c]);
+            odd += std::fabs(d[2][c] - d[1][c]) + std::fabs(d[3][c] - d[0][c]);
+            even += std::fabs(d[2][c] + d[1][c] - 2.0 * mean) +
+                    std::fabs(d[3][c] + d[0][c] - 2.0 * mean);
+        }
+        const double s = odd + even;
+        if (0.25 * x * odd * even + s * s * s / 24.0 > share)
+            ++over;
+    }
+    return seen > 0 && 2 * over >= seen;
+}
+
+// What follows from a pulse and its theta_max: series degrees, step groups, and whether
+// they may be evaluated expanded.
+void choose_steps(dsp_grid *g, const double *a_mid, int64_t n_steps, double dt, double theta_max)
 {
     g->n_steps = n_steps;
+    g->dt = dt;
     g->theta_max = theta_max;
     g->level = choose_level(g->precision, theta_max, n_steps);
     g->tdeg = g->precision == DSP_FP32_MIXED ? choose_tan_degree(g->scheme, theta_max, n_steps) : 0;
     g->group = choose_group(g->precision, g->scheme, g->tdeg, theta_max);
-    g->by_groups = g->expand && may_expand(g);
+    g->by_groups = g->expand && may_expand(g) && !rough_throughout(g, a_mid);
 }
 
 // Host part of setting a pulse: validates, fills the grid's pulse fields, and lays out
@@ -1068,12 +1115,11 @@ dsp_status prepare_pulse(dsp_grid *g, const double *a_mid, int64_t n_steps, doub
         return s;
     g->has_pulse = true;
     g->cursor = 0;
-    g->dt = dt;
     g->a_in[0] = a_in[0];
     g->a_in[1] = a_in[1];
     g->a_out[0] = a_out[0];
     g->a_out[1] = a_out[1];
-    choose_steps(g, n_steps, tmax);
+    choose_steps(g, a_mid, n_steps, dt, tmax);
     g->fresh = true;
     g->projected = false;
     g->state_stale = false;
@@ -2161,7 +2207,7 @@ dsp_status dsp_server_submit(dsp_server *s, const dsp_request *req, const double
         return st;
     // The request's own footprint and the budget decide whether its groups may be expanded,
     // not what else is active: its result is the same alone and in any mix.
-    choose_steps(&probe, p.n_steps, tmax);
+    choose_steps(&probe, a_mid, p.n_steps, p.dt, tmax);
     size_t footprint = RequestMemory(probe).total;
     if (probe.by_groups && footprint > static_cast<size_t>(s->budget)) {
         probe.by_groups = probe.expand = false;

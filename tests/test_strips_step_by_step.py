@@ -88,13 +88,17 @@ def test_bands_and_valleys_on_strips():
         assert np.array_equal(band[0], ref[0][7:19])
 
 
+# noise in every group is seen on the host; jumps in a quarter of them only in the groups' sums
+@pytest.mark.parametrize("kind", ["noise", "jumps"])
 @pytest.mark.parametrize("size", [(512, 10), (512, 700), (300, 9)])
 @pytest.mark.parametrize("keep", [True, False])
-def test_tables_that_the_expansion_refuses(orc, size, keep):
-    """Noise over the expansion's bound, expansion on: the run goes step by step, with the bits it has
-    when the expansion is off, the final state kept or not."""
+def test_tables_that_the_expansion_refuses(orc, size, keep, kind):
+    """Tables over the expansion's bound, expansion on: the run goes step by step, as it does when the
+    expansion is off, the final state kept or not."""
     rng = np.random.default_rng(4)
     a = rng.standard_normal((3001, 2)).clip(-3, 3)
+    if kind == "jumps":
+        a = np.repeat(rng.choice([-2.0, 2.0], (3001 // 16 + 1, 2)), 16, axis=0)[1:3002]
     tab = (a, np.zeros(2), np.array([0.5, 0.0]), 0.002)
     ref, info = solve(size, tab)
     assert info["group_steps"] > 1
@@ -120,3 +124,22 @@ def test_tables_that_the_expansion_refuses(orc, size, keep):
             g.project()
         assert e.value.code == -4
     g.close()
+
+
+@pytest.mark.parametrize("size,steps,expanded", [
+    ((256, 256), 511, False), ((256, 256), 512, True), ((1024, 512), 63, False),
+    ((1024, 512), 64, True), ((512, 2), 511, False), ((512, 2), 512, True), ((64, 64), 4, True),
+    ((1100, 1000), 31, False), ((1100, 1000), 32, True)])
+def test_pulses_too_short_to_expand(size, steps, expanded):
+    """The line by grid and length, and a band on the full grid's side of it, bit for bit."""
+    a, a_in, a_out, _ = sample("exact", steps)
+    out = []
+    for rows in (None, (1, 2)):
+        g = B.Grid(size[0], size[1], (-4.0, 4.0), (-4.0, 4.0), "fp32_mixed", rows=rows)
+        g.set_pulse(a, 0.002, a_in, a_out)
+        assert (B.get_groups(g.h)[0] > 0) == expanded
+        m, _ = g.solve()
+        torch.cuda.synchronize()
+        out.append(m.cpu().numpy().copy())
+        g.close()
+    assert np.array_equal(out[1], out[0][1:2])
