@@ -574,10 +574,10 @@ int64_t f64_tiles(const ReqDesc &r, int lanes)
     return lanes == 0 ? row_tiles(r, 4) : (r.n_points + 32 / lanes - 1) / (32 / lanes);
 }
 
-// A tile's share of a busy scheduler per step of an FP64 launch (launch_evolve_f64's
-// lanes), in units of 33 ns: its FP64 instructions and, for pairs, the waits between the
-// two warps; n = the series' degrees together.  Measured on grids of 16^2 to 512^2, 1000
-// steps, n of 6 to 12, to within 1%.  EXACT forms its series in FP32: no n.
+// A tile's share of a busy scheduler in an FP64 launch (launch_evolve_f64's lanes), in
+// units of 33 ns: its FP64 instructions and, for pairs, the waits between the two warps;
+// n = the series' degrees together.  Measured on grids of 16^2 to 512^2, 1000 steps, n of 6
+// to 12, to within 1%.  EXACT forms its series in FP32: no n.
 double f64_cost(const ReqDesc &r, int lanes)
 {
     const int n = dsp::kLevelsF64[r.level].dc + dsp::kLevelsF64[r.level].ds;
@@ -587,12 +587,20 @@ double f64_cost(const ReqDesc &r, int lanes)
         return lanes == 1 ? 20.9 + 2.23 * n : lanes == 0 ? 60.6 + 1.25 * n : 5.3 + 0.555 * n;
     return lanes == 1 ? 26.4 + 1.12 * n : 6.7 + 0.28 * n;
 }
+// The same of what a tile does besides its steps: the initial spinors, once per lane (a
+// pair forms each point's four times; launches of one step on 512^2: 43, 43 and 171 us).
+double f64_setup(const ReqDesc &r, int lanes)
+{
+    const double spinors = lanes == 1 ? 60.0 : lanes == 0 ? 210.0 : 70.0;
+    return 10.0 + (r.fresh && !r.init_identity ? spinors : 0.0);
+}
 
 // Shape of an FP64 launch by the FP64 work of its fullest scheduler (dsp_f64.cu): 32
-// points flat, 4 rows x 32 columns (EXACT, STRANG_XY), or 8 points on a warp pair.
-// `alone` is what an EXACT step takes when a scheduler has one tile, whose operators then
-// wait for its own updates (the other schemes' operators are FP64 work themselves, in
-// f64_cost).
+// points flat, 4 rows x 32 columns (EXACT, STRANG_XY), or 8 points on a warp pair (whose
+// operators are formed for 16 steps at a time).  `alone` is what an EXACT step takes when
+// a scheduler has one tile, whose operators then wait for its own updates (the other
+// schemes' operators are FP64 work themselves, in f64_cost).  A new state on 256^2: no step
+// 77 us on pairs, 44 flat; 16 steps 106, 78; 64 steps 207, 187.
 int f64_lanes(const std::vector<ReqDesc> &reqs, int scheme)
 {
     constexpr int shapes[3] = {1, 0, 4};
@@ -604,15 +612,20 @@ int f64_lanes(const std::vector<ReqDesc> &reqs, int scheme)
         if (lanes == 0 && scheme == DSP_SCHEME_MAGNUS4)
             continue;
         int64_t tiles = 0;
-        double work = 0.0;
+        double work = 0.0, longest = 0.0;
         for (const ReqDesc &r : reqs) {
+            const int64_t n = r.step_end - r.step_begin;
+            const double steps = static_cast<double>(lanes == 4 ? (n + 15) / 16 * 16 : n);
+            const double setup = f64_setup(r, lanes);
             tiles += f64_tiles(r, lanes);
-            work += static_cast<double>(f64_tiles(r, lanes)) * f64_cost(r, lanes);
+            work += static_cast<double>(f64_tiles(r, lanes)) * (f64_cost(r, lanes) * steps + setup);
+            if (scheme == DSP_SCHEME_EXACT)
+                longest = std::max(longest, alone[k] * steps + setup);
         }
         if (tiles == 0)
             break;
-        const double t = std::max(scheme == DSP_SCHEME_EXACT ? alone[k] : 0.0,
-                                  launch_time(tiles, work / static_cast<double>(tiles)));
+        const double t =
+            std::max(longest, launch_time(tiles, work / static_cast<double>(tiles)));
         if (lanes == 1 || t < 0.99 * best_t) {
             best = lanes;
             best_t = t;
