@@ -226,8 +226,8 @@ dsp_status dsp_solve(dsp_grid *g, void *map_dev, double *n_host);
  * conj(a)]], so the column (a, b) determines it), then the segments are
  * multiplied onto v(p + A_in) in time order in FP64.  Same steps, same results
  * as dsp_solve up to rounding (not bitwise).  segments = 0 picks enough to fill
- * the chip (at least 16 steps per segment); segments of 32 steps and more start
- * on multiples of 16 steps; needs cursor == 0
+ * the chip (at least 16 steps per segment, 96 segments); FP32_MIXED segments of 32
+ * steps and more start on multiples of 16 steps; needs cursor == 0
  * (DSP_E_STATE otherwise).  Scratch: segments * 32 bytes per point, allocated
  * by the library (at most 16 GB, else DSP_E_INVALID).  map_dev and n_host as
  * in dsp_solve. */

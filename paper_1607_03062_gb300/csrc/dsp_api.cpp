@@ -601,7 +601,8 @@ double f64_setup(const ReqDesc &r, int lanes)
 // a scheduler has one tile, whose operators then wait for its own updates (the other
 // schemes' operators are FP64 work themselves, in f64_cost).  A new state on 256^2: no step
 // 77 us on pairs, 44 flat; 16 steps 106, 78; 64 steps 207, 187.
-int f64_lanes(const std::vector<ReqDesc> &reqs, int scheme)
+// *time, when given, receives the launch's.
+int f64_lanes(const std::vector<ReqDesc> &reqs, int scheme, double *time = nullptr)
 {
     constexpr int shapes[3] = {1, 0, 4};
     constexpr double alone[3] = {26.6, 84.6, 5.5};
@@ -634,6 +635,8 @@ int f64_lanes(const std::vector<ReqDesc> &reqs, int scheme)
     for (const ReqDesc &r : reqs)
         if (r.rows > 0)
             best = r.rows == 4 && scheme != DSP_SCHEME_MAGNUS4 ? 0 : 1;
+    if (time)
+        *time = best_t;
     return best;
 }
 
@@ -1287,6 +1290,45 @@ dsp_status run_one(dsp_grid *g, int64_t end, bool project, void *map)
     return DSP_OK;
 }
 
+// Time segments for dsp_solve_segmented: at most what one launch carries, of at least 16
+// steps.  A segment has one warp per 32 points.  FP32_MIXED: one warp per scheduler, each
+// with a short run left and few columns to combine (64^2 x 2000 steps: 62 us with 2 to 5
+// segments, 74 with 1, 77 with 16, launches included; 2^2 x 20000 184 with 76, 198 with 96).
+// FP64: of the counts that fill the
+// schedulers evenly, the one with the least time of the fullest scheduler (f64_lanes' costs)
+// and of combining, a chain of FP64 operations of about 1.1 us a segment.  Measured (us, the
+// rule's count first; 38 and 41 are a count that fills them and one that does not):
+// 64^2 x 2000 324 (14), 322 (38), 358 (41); 128^2 x 20000 8990 (19), 9840 (39); 32^2 x 5000 246
+// (19), 372 (104); 16^2 x 50000 551 (76), 1680 (1041, in eleven launches).
+int64_t segment_count(const dsp_grid *g)
+{
+    const int64_t warps = (g->n_points + 31) / 32, schedulers = 4 * static_cast<int64_t>(sm_count());
+    const int64_t most = std::max<int64_t>(
+        1, std::min<int64_t>(dsp::kMaxReqPerLaunch, g->n_steps / 16));
+    if (g->precision != DSP_FP64)
+        return std::max<int64_t>(1, std::min({most, static_cast<int64_t>(sm_count() / 2),
+                                              (schedulers + warps - 1) / warps}));
+    int64_t best = 1, last = 0;
+    double best_t = 0.0;
+    for (int64_t fill = 0; fill <= 40; ++fill) {
+        const int64_t S = std::max<int64_t>(1, std::min<int64_t>(most, fill * schedulers / warps));
+        if (S == last)
+            continue;
+        last = S;
+        ReqDesc r = make_desc(g, 0, (g->n_steps + S - 1) / S, false, nullptr);
+        r.init_identity = 1;
+        double t = 0.0;
+        f64_lanes(std::vector<ReqDesc>(static_cast<size_t>(S), r), g->scheme, &t);
+        t += 33.0 * static_cast<double>(S) *
+             std::max(1.0, static_cast<double>(warps) / static_cast<double>(schedulers));
+        if (fill == 0 || t < best_t) {
+            best = S;
+            best_t = t;
+        }
+    }
+    return best;
+}
+
 dsp_status ensure_own_map(dsp_grid *g)
 {
     if (g->own_map)
@@ -1448,19 +1490,8 @@ dsp_status dsp_solve_segmented(dsp_grid *g, int32_t segments, void *map_dev, dou
     if (g->n_steps == 0)
         return dsp_solve(g, map_dev, n_host);
     int64_t S = segments;
-    if (S == 0) {
-        // A segment has one warp per 32 points.  FP32_MIXED: one warp per scheduler, each
-        // with a short run left and few columns to combine (64^2 x 2000 steps: 62 us with
-        // 2 to 5 segments, 74 with 1, 77 with 16, launches included).  FP64: 16, so that the
-        // fullest scheduler is close to the average, in segments of 48 steps and more
-        // (64^2 x 2000: 343 us with 38, 401 with 6, 464 with 5; 128^2 x 20000: 9.0 ms with 19,
-        // 12.4 with 5).
-        const int64_t warps = (g->n_points + 31) / 32;
-        const bool f64 = g->precision == DSP_FP64;
-        const int64_t want = (f64 ? 64 : 4) * static_cast<int64_t>(sm_count());
-        S = (want + warps - 1) / warps;
-        S = std::min<int64_t>(S, g->n_steps / (f64 ? 48 : 16));
-    }
+    if (S == 0)
+        S = segment_count(g);
     S = std::max<int64_t>(1, std::min<int64_t>(S, g->n_steps));
     const size_t slab = 32 * static_cast<size_t>(g->n_points);
     if (S > 65536 || static_cast<double>(S) * static_cast<double>(slab) > 16.0e9)
@@ -1494,10 +1525,11 @@ dsp_status dsp_solve_segmented(dsp_grid *g, int32_t segments, void *map_dev, dou
     std::vector<ReqDesc> descs;
     descs.reserve(static_cast<size_t>(S));
     for (int64_t k = 0; k < S; ++k) {
-        // long segments start on whole step groups
+        // long segments start on whole step groups (FP64 has none: even lengths)
         const auto start = [&](int64_t i) {
             const int64_t n = i * g->n_steps / S;
-            return i < S && g->n_steps / S >= 2 * dsp::kGroupMax ? n - n % dsp::kGroupMax : n;
+            return i < S && g->precision == DSP_FP32_MIXED && g->n_steps / S >= 2 * dsp::kGroupMax
+                       ? n - n % dsp::kGroupMax : n;
         };
         ReqDesc d = make_desc(g, start(k), start(k + 1), false, nullptr);
         d.state = static_cast<unsigned char *>(g->seg_buf) + static_cast<size_t>(k) * slab;
