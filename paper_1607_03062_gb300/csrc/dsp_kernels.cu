@@ -146,7 +146,8 @@ __device__ __forceinline__ void project_pair(const ReqDesc &R, const unsigned ch
                                                granule_spinor<0>(src, l + 32)));
 }
 
-template <int PREC>
+// GROUPS: the launch has requests that may have gone step by step (ReqDesc::by_groups).
+template <int PREC, bool GROUPS>
 __global__ void __launch_bounds__(ProjShape<PREC>::threads, 1)
     project_kernel(const __grid_constant__ EvolveArgs args)
 {
@@ -159,15 +160,20 @@ __global__ void __launch_bounds__(ProjShape<PREC>::threads, 1)
     uint64_t *bars = reinterpret_cast<uint64_t *>(proj_dyn + Sh::warps * Sh::warp_bytes) + NB * w;
     constexpr int kGranPerTile = kTilePoints / kGranule;
     const int total = args.total_tiles * kGranPerTile;  // granules of the launch
-    // granules go to the CTAs in turn, so that a small grid's spread over the SMs
-    const int wid = w * gridDim.x + blockIdx.x, nw = gridDim.x * Sh::warps;
+    // Granules go to the CTAs in turn, so that a small grid's spread over the SMs and the
+    // last round's over all of them; a large FP32_MIXED grid keeps neighbouring granules on
+    // one SM (us a launch, in turn and neighbours: 100 x 75 6.1 and 7.6, 1024^2 8.4 and 10.4,
+    // 2048^2 32.5 and 32.0, 4096^2 101.4 and 99.0).
+    const int nw = gridDim.x * Sh::warps;
+    const int wid = PREC == 0 || total < 4 * nw ? w * gridDim.x + blockIdx.x
+                                                : blockIdx.x * Sh::warps + w;
     // A request that went step by step has been projected there: nothing to load or to do.
     // (Looked up once per request: granules of one follow each other.  A warp's first
     // granule is loaded meanwhile, whatever comes of it.)
     int seen = -1;
     bool wanted = true;
     const auto to_project = [&](int r) {
-        if (r != seen) {
+        if (GROUPS && r != seen) {
             seen = r;
             wanted = !args.r[r].by_groups || left_to_groups(args.r[r]);
         }
@@ -441,6 +447,19 @@ cudaError_t launch_evolve_strip(const EvolveArgs &args, int scheme, int strip_h,
     return half ? launch_evolve_strip_s2_np1(args, stream) : launch_evolve_strip_s2_np2(args, stream);
 }
 
+template <int PREC, bool GROUPS>
+static cudaError_t launch_project(const EvolveArgs &args, int grid, cudaStream_t stream)
+{
+    using Sh = ProjShape<PREC>;
+    // the warps' rings are above the 48 KB a kernel gets without asking
+    const cudaError_t e = cudaFuncSetAttribute(
+        project_kernel<PREC, GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::smem);
+    if (e != cudaSuccess)
+        return e;
+    project_kernel<PREC, GROUPS><<<grid, Sh::threads, Sh::smem, stream>>>(args);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_project(const EvolveArgs &args, int precision, cudaStream_t stream)
 {
     if (args.nreq <= 0 || args.total_tiles <= 0)
@@ -449,23 +468,17 @@ cudaError_t launch_project(const EvolveArgs &args, int precision, cudaStream_t s
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess)
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    // the warps' rings are above the 48 KB a kernel gets without asking
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(project_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 ProjShape<1>::smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(project_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 ProjShape<0>::smem);
     if (e != cudaSuccess)
         return e;
+    bool groups = false;
+    for (int i = 0; i < args.nreq; ++i)
+        groups = groups || args.r[i].by_groups;
     // one CTA per SM, no more CTAs than granules
     const int granules = args.total_tiles * (kTilePoints / kGranule);
     const int grid = granules < sms ? granules : sms;
-    if (precision == 1)
-        project_kernel<1><<<grid, ProjShape<1>::threads, ProjShape<1>::smem, stream>>>(args);
-    else
-        project_kernel<0><<<grid, ProjShape<0>::threads, ProjShape<0>::smem, stream>>>(args);
-    return cudaGetLastError();
+    return precision != 1 ? launch_project<0, false>(args, grid, stream)
+           : groups       ? launch_project<1, true>(args, grid, stream)
+                          : launch_project<1, false>(args, grid, stream);
 }
 
 cudaError_t launch_finalize(const FinalizeArgs &args, cudaStream_t stream)
