@@ -285,13 +285,16 @@ typedef struct {
     int32_t group_steps;
     int32_t row_begin;  /* first global row (0 unless the grid is a band)      */
     int32_t ny_total;   /* rows of the full grid (ny unless the grid is a band) */
-    int32_t row_strips; /* 1: evolve launches that go step by step tile the grid in
-                           row strips of 4 rows x 256 columns (nx a multiple of 256;
-                           FP32_MIXED every scheme, FP64 EXACT and STRANG_XY),
+    int32_t row_strips; /* 1: nx is a multiple of 256 (FP32_MIXED every scheme, FP64
+                           EXACT and STRANG_XY): FP32_MIXED launches that go step by
+                           step tile the grid in row strips of 4 rows x 256 columns,
                            sharing each step's momentum work across a strip; 0: in
                            contiguous tiles of 1024 points.  n_tiles counts those
-                           tiles.  Launches on expanded groups take 32 columns x 1,
-                           2 or 4 rows per warp on any grid. */
+                           tiles.  Launches on expanded groups (32 columns x 1, 2 or 4
+                           rows per warp) and FP64 launches (32 columns x 4 rows or 32
+                           points per warp, or 8 points on a pair, by what fills the
+                           chip) take their own tiles on any grid; for them the two
+                           fields only say how the grid divides. */
     int32_t tan_degree; /* see above */
 } dsp_grid_info;
 /* Fills *info for the grid's current pulse (the fields above; bookkeeping,
@@ -315,13 +318,14 @@ dsp_status dsp_get_groups(dsp_grid *g, int32_t *steps, int32_t *level);
 dsp_status dsp_test_withhold_next_copy(dsp_grid *g);
 
 /* Test hook (not in the paper) on the tiling of the grid's evolve launches.
- * Grids whose nx is a multiple of 256 (FP32_MIXED every scheme, FP64 EXACT and
- * STRANG_XY) evolve on row strips: a CTA owns 4 rows x 256 columns and shares
- * the per-step momentum work across them; a launch of one such grid whose last
- * wave of CTAs would be at most half full runs its last strips 2 rows high.
- * Expanded step groups evolve on warps of 4, 2 or 1 rows, by what fills the chip.
- * tiling = 1: those automatic choices (the default); 0: contiguous 1024-point
- * tiles, warps of 1 row; 2: row strips and warps, all 4 rows high.  Every tiling gives bitwise the same
+ * FP32_MIXED grids whose nx is a multiple of 256 go step by step on row strips: a CTA
+ * owns 4 rows x 256 columns and shares the per-step momentum work across them; a
+ * launch of one such grid whose last wave of CTAs would be at most half full runs its
+ * last strips 2 rows high.  Expanded step groups evolve on warps of 4, 2 or 1 rows,
+ * FP64 on warps of 4 rows x 32 columns or 32 points or on warp pairs, by what fills
+ * the chip.  tiling = 1: those automatic choices (the default); 0: contiguous
+ * 1024-point tiles, warps of 1 row (FP64: of 32 points); 2: row strips and warps, all 4
+ * rows high.  Every tiling gives bitwise the same
  * map and density; the hook exists so that a test can show it. */
 dsp_status dsp_test_tiling(dsp_grid *g, int32_t tiling);
 
