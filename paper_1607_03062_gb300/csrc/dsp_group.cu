@@ -592,7 +592,7 @@ static_assert(kGroupWarps * sizeof(WarpSmem) <= 48 * 1024, "dynamic shared memor
 // and kinks, and for MAGNUS4 of noise in D alone: at most 0.7 of the estimate (EXACT
 // 1.2 where a group drops less than 1e-9).
 //
-// One thread per group, and one per 16 steps for the per-step table (dt A rounded
+// One thread per group, and two per 16 steps for the per-step table (dt A rounded
 // to FP32 so that its running sum keeps to the exact one, dsp_steptable.h); FP64 only
 // where those sums and the group's mean need it.  A 1e5-step table takes microseconds, where the host took 18 ns a step.
 // ---------------------------------------------------------------------------
@@ -623,15 +623,18 @@ struct StepA {
     double x, y;
     F2 D;
 };
+__device__ __forceinline__ float gauss_difference(const PrepArgs &a, double p, double q)
+{
+    constexpr double kappa = -0.28867513459481288225;  // -sqrt(3)/6
+    return static_cast<float>(kappa * (a.sdt * (q - p)));
+}
 __device__ __forceinline__ StepA step_potential(const PrepArgs &a, int64_t n)
 {
     if (a.scheme == 2) {
         const double2 p = reinterpret_cast<const double2 *>(a.raw)[2 * n];
         const double2 q = reinterpret_cast<const double2 *>(a.raw)[2 * n + 1];
-        constexpr double kappa = -0.28867513459481288225;  // -sqrt(3)/6
         return {a.sdt * (0.5 * (p.x + q.x)), a.sdt * (0.5 * (p.y + q.y)),
-                {static_cast<float>(kappa * (a.sdt * (q.x - p.x))),
-                 static_cast<float>(kappa * (a.sdt * (q.y - p.y)))}};
+                {gauss_difference(a, p.x, q.x), gauss_difference(a, p.y, q.y)}};
     }
     const double2 p = reinterpret_cast<const double2 *>(a.raw)[n];
     return {a.sdt * p.x, a.sdt * p.y, {0.0f, 0.0f}};
@@ -799,21 +802,30 @@ __global__ void __launch_bounds__(kPrepThreads) prep_groups_kernel(const __grid_
         add_estimate(&a.sums->lite[what], lite);
         return;
     }
-    // dt A per step, rounded to FP32 (table_block)
-    if (kTableBlock * g >= a.n_steps)
+    // dt A per step, rounded to FP32 (table_block): a thread per 16 steps and coordinate, so
+    // that the chain of FP64 operations is half as long (prep of 12000 MAGNUS4 steps 24.6
+    // us with one thread for both, 18.4 with the residual dropped every 16 steps)
+    const int64_t block = g >> 1;
+    const int c = static_cast<int>(g & 1);
+    if (kTableBlock * block >= a.n_steps)
         return;
     const double half = a.scheme == 2 ? 0.5 * a.sdt : a.sdt;  // times the sum of the samples
-    const double2 s0 = reinterpret_cast<const double2 *>(a.prefix)[g];
-    const double2 s1 = reinterpret_cast<const double2 *>(a.prefix)[g + 1];
-    table_block(g, a.n_steps, __dmul_rn(half, s0.x), __dmul_rn(half, s0.y),
-                __dmul_rn(half, s1.x), __dmul_rn(half, s1.y),
-                [&](int64_t k) { return step_potential(a, k); },
-                [&](int64_t k, const StepA &s, float fx, float fy) {
-                    if (a.scheme == 2)
-                        static_cast<float4 *>(a.table)[k] = make_float4(fx, fy, s.D.x, s.D.y);
-                    else
-                        static_cast<float2 *>(a.table)[k] = make_float2(fx, fy);
-                });
+    const double s0 = a.prefix[2 * block + c], s1 = a.prefix[2 * block + 2 + c];
+    float *out = static_cast<float *>(a.table) + c;
+    if (a.scheme == 2) {
+        table_block(block, a.n_steps, __dmul_rn(half, s0), __dmul_rn(half, s1),
+                    [&](int64_t k) {
+                        return a.sdt * (0.5 * (a.raw[4 * k + c] + a.raw[4 * k + 2 + c]));
+                    },
+                    [&](int64_t k, float f) {
+                        out[4 * k] = f;
+                        out[4 * k + 2] = gauss_difference(a, a.raw[4 * k + c], a.raw[4 * k + 2 + c]);
+                    });
+    } else {
+        table_block(block, a.n_steps, __dmul_rn(half, s0), __dmul_rn(half, s1),
+                    [&](int64_t k) { return a.sdt * a.raw[2 * k + c]; },
+                    [&](int64_t k, float f) { out[2 * k] = f; });
+    }
 }
 
 }  // namespace

@@ -73,33 +73,23 @@ DSP_HD double table_sum(double s, double v, double w)
     return add_rn(add_rn(s, magic), -magic);
 }
 
-// Entries of the steps [16 g, 16 g + 16) of a table of n steps.  step(k) is s dt A of step
-// k (also called for the steps just before and after the block), as a type with x and y;
-// (x0, y0) and (x1, y1) the running sums before the block and after it; put(k, step(k),
-// fx, fy) takes the entry.
+// Entries of the steps [16 g, 16 g + 16) of a table of n steps, one coordinate.  step(k) is
+// s dt A of step k (also called for the steps just before and after the block), s0 and s1
+// the running sums before the block and after it; put(k, f) takes the entry.
 template <typename Step, typename Put>
-DSP_HD void table_block(int64_t g, int64_t n, double x0, double y0, double x1, double y1,
-                        Step step, Put put)
+DSP_HD void table_block(int64_t g, int64_t n, double s0, double s1, Step step, Put put)
 {
     const int64_t first = kTableBlock * g;
     const int64_t end = first + kTableBlock < n ? first + kTableBlock : n;
-    auto v = step(first);
-    double fx = 0.0, fy = 0.0, lx = 0.0, ly = 0.0;  // lx, ly: the sum inside the block
-    if (first > 0) {
-        const auto u = step(first - 1);
-        fx = table_sum(x0, u.x, v.x);
-        fy = table_sum(y0, u.y, v.y);
-    }
+    double v = step(first), inside = 0.0;  // inside: the sum in the block
+    double f = first > 0 ? table_sum(s0, step(first - 1), v) : 0.0;
     for (int64_t k = first; k < end; ++k) {
-        const auto w = step(k + 1 < n ? k + 1 : k);  // (past the end: the last step again)
-        lx = add_rn(lx, v.x);
-        ly = add_rn(ly, v.y);
+        const double w = step(k + 1 < n ? k + 1 : k);  // (past the end: the last step again)
+        inside = add_rn(inside, v);
         // (the next block starts from the same sum)
-        const double x = k + 1 < end ? add_rn(x0, lx) : x1, y = k + 1 < end ? add_rn(y0, ly) : y1;
-        const double hx = table_sum(x, v.x, w.x), hy = table_sum(y, v.y, w.y);
-        put(k, v, static_cast<float>(add_rn(hx, -fx)), static_cast<float>(add_rn(hy, -fy)));
-        fx = hx;
-        fy = hy;
+        const double h = table_sum(k + 1 < end ? add_rn(s0, inside) : s1, v, w);
+        put(k, static_cast<float>(add_rn(h, -f)));
+        f = h;
         v = w;
     }
 }

@@ -12,7 +12,6 @@ from paper_1607_03062_gb300 import build as Bd
 
 SHIM = r"""
 #include "dsp_steptable.h"
-struct S { double x, y; };
 extern "C" void table(const double *a, int64_t n, int per, double sdt, float *out)
 {
     const int64_t blocks = (n + dsp::kTableBlock - 1) / dsp::kTableBlock;
@@ -21,16 +20,14 @@ extern "C" void table(const double *a, int64_t n, int per, double sdt, float *ou
     dsp::copy_with_prefix(a, n, per, copy, pre);
     a = copy;
     const double h = per == 2 ? 0.5 * sdt : sdt;
-    const auto step = [&](int64_t k) {
-        return per == 2 ? S{sdt * (0.5 * (a[4 * k] + a[4 * k + 2])), sdt * (0.5 * (a[4 * k + 1] + a[4 * k + 3]))}
-                        : S{sdt * a[2 * k], sdt * a[2 * k + 1]};
-    };
-    for (int64_t g = blocks - 1; g >= 0; --g)  // any order
-        dsp::table_block(g, n, h * pre[2 * g], h * pre[2 * g + 1], h * pre[2 * g + 2],
-                         h * pre[2 * g + 3], step, [&](int64_t k, const S &, float x, float y) {
-                             out[2 * k] = x;
-                             out[2 * k + 1] = y;
-                         });
+    for (int c = 0; c < 2; ++c)
+        for (int64_t g = blocks - 1; g >= 0; --g)  // any order
+            dsp::table_block(g, n, h * pre[2 * g + c], h * pre[2 * g + 2 + c],
+                             [&](int64_t k) {
+                                 return per == 2 ? sdt * (0.5 * (a[4 * k + c] + a[4 * k + 2 + c]))
+                                                 : sdt * a[2 * k + c];
+                             },
+                             [&](int64_t k, float f) { out[2 * k + c] = f; });
     delete[] pre;
     delete[] copy;
 }
