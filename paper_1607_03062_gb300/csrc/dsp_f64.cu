@@ -610,7 +610,8 @@ __global__ void __launch_bounds__(32 * kF64Warps, ROWS ? 4 : 5)
 
 // Warp pairs, kF64Warps / 2 of them or one per CTA.  The CTAs are dealt to the SMs in
 // turn, so that swapping the warps' roles from one round of SMs to the next puts both
-// kinds on every scheduler.
+// kinds on every scheduler.  One kernel per scheme.
+template <int SCHEME>
 __global__ void __launch_bounds__(32 * kF64Warps, 4)
     evolve_f64_pair_kernel(const __grid_constant__ EvolveArgs args, int sms)
 {
@@ -634,8 +635,9 @@ __global__ void __launch_bounds__(32 * kF64Warps, 4)
     if (!tile_ok(R, tile, R.err) || !table_range_ok(R, R.step_begin, R.err))
         return;
     const bool forms = (w & 1) != ((blockIdx.x / sms) & 1);
-    dispatch_f64<true>(R, [&](auto scheme, auto dc, auto ds) {
-        body_pair<decltype(scheme)::value, decltype(dc)::value, decltype(ds)::value>(R, tile, sm, R.err, forms);
+    dispatch_level<SCHEME, 0>(R, [&](auto scheme, auto dc, auto ds) {
+        body_pair<decltype(scheme)::value, decltype(dc)::value, decltype(ds)::value>(R, tile, sm,
+                                                                                     R.err, forms);
     });
 }
 
@@ -653,8 +655,14 @@ cudaError_t launch_evolve_f64(const EvolveArgs &args, int lanes, int warps, cuda
         if (e != cudaSuccess)
             return e;
         const int pairs = warps > 1 ? warps / 2 : 1;
-        evolve_f64_pair_kernel<<<(args.total_tiles + pairs - 1) / pairs, 64 * pairs, 0, stream>>>(
-            args, sms);
+        const int grid = (args.total_tiles + pairs - 1) / pairs;
+        const int scheme = args.r[0].scheme;
+        if (scheme == 0)
+            evolve_f64_pair_kernel<0><<<grid, 64 * pairs, 0, stream>>>(args, sms);
+        else if (scheme == 1)
+            evolve_f64_pair_kernel<1><<<grid, 64 * pairs, 0, stream>>>(args, sms);
+        else
+            evolve_f64_pair_kernel<2><<<grid, 64 * pairs, 0, stream>>>(args, sms);
         return cudaGetLastError();
     }
     const int grid = (args.total_tiles + warps - 1) / warps;
