@@ -150,7 +150,8 @@ def kernel_source_sha256():
     headers it includes)."""
     import hashlib
     h = hashlib.sha256()
-    for name in ("dsp_group.cu", "dsp_device.cuh", "dsp_internal.h", "dsp_df.cuh"):
+    for name in ("dsp_group.cu", "dsp_device.cuh", "dsp_internal.h", "dsp_df.cuh",
+                 "dsp_steptable.h"):
         with open(os.path.join(ROOT, "paper_1607_03062_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()
@@ -246,10 +247,10 @@ def ops_strang(dc, ds, group=1, strips=False, tdeg=0):
 
 def ops_groups(steps, level, strang=False):
     """FP32 lane instructions per spinor-step of expanded groups of `steps` steps: per
-    group 42 (level 0), 64 (1) or 75 (2) for the operator and the compensated update, 11
+    group 42 (level 0), 64 (1) or 76 (2) for the operator and the compensated update, 11
     more for STRANG_XY's momentum, and the column part (9 scalar ops per lane) shared by
     its 4 rows."""
-    return ((42, 64, 75)[level] + (11 if strang else 0) + 9 / 4.0) / steps
+    return ((42, 64, 76)[level] + (11 if strang else 0) + 9 / 4.0) / steps
 
 
 def ops_fp64(dc, ds, strips=False):
@@ -431,10 +432,12 @@ def run_gpu(args):
         dist.all_reduce(t, op=dist.ReduceOp.MAX)
         e2e_tot = float(t.item())
     e2e = {"value": work_per_solve * args.steps * world / e2e_tot, "unit": METRIC,
-           # the caller's FP64 table, from which the device makes the rest, 64 bytes of
-           # zeroed sums and the projection nodes (hi/lo float pairs of every column
-           # and row); step by step the FP32 table that the host builds instead
-           "h2d_bytes_per_step": ((16 * nsteps + 64) if expanded else 8 * nsteps) + 8 * (n + n),
+           # the caller's FP64 table, from which the device makes the rest, its running
+           # sums every 16 steps, 64 bytes of zeroed sums and the projection nodes (hi/lo
+           # float pairs of every column and row); step by step the FP32 table that the
+           # host builds instead
+           "h2d_bytes_per_step": ((16 * nsteps + 16 * (-(-nsteps // 16) + 1) + 64) if expanded
+                                  else 8 * nsteps) + 8 * (n + n),
            "d2h_bytes_per_step": 4 * n * n + 16,
            "note": "dsp_solve_host: host midpoint table in, host |c+|^2 map (pinned) and density out"}
 

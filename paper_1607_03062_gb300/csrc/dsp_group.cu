@@ -33,7 +33,7 @@ namespace {
 //   wide  also applies S and the small rest of w apart, because at large group angles
 //         the rounding of their sum would show.
 //
-// What bounds it: FP32 issue.  Per spinor and group 42 (lite), 64 (full) or 75 (wide)
+// What bounds it: FP32 issue.  Per spinor and group 42 (lite), 64 (full) or 76 (wide)
 // lane operations plus a column part shared by the warp's rows, against 9 and more per
 // spinor and STEP of the chains.  FMA pipe 83% busy (lite; packed instructions hold it
 // two cycles), issue 50%, DRAM idle.
@@ -47,7 +47,7 @@ namespace {
 // The projection is the projection kernel's, on the state this kernel leaves.
 //
 // Measured (GB300, whole solves, step by step -> expanded): 2048^2 x 1e5 sin^2 pulse
-// 209.2 -> 35.2 ms (lite, G = 16); 1024^2 x 3e4 Gaussian pulse 22.6 -> 5.00 ms (wide,
+// 209.2 -> 35.2 ms (lite, G = 16); 1024^2 x 3e4 Gaussian pulse 22.6 -> 5.05 ms (wide,
 // 16); 1000 x 750 x 2e4 two colours 10.36 -> 2.46 ms (wide, 16; contiguous tiles
 // before); 512^2 x 12000 MAGNUS4 3.14 -> 0.575 ms (full); 256^2 x 2e4 paper pulse 1.42
 // -> 0.375 ms; 512 x 384 x 12000 STRANG_XY 1.79 -> 0.55 ms (full).  2-norm error of
@@ -275,12 +275,15 @@ __device__ __forceinline__ void group_step(GroupPoint<V> &p, const GroupCol &c,
             return;
         }
         const V Tx = vadd(Sx, vx), Ty = vadd(Sy, vy);
-        const V x = vfma(vadd(Sx, Tx), vx, vfma(vadd(Sy, Ty), vy, vfma(wz, wz, x0)));
+        const V x = vfma(Tx, Tx, vfma(Ty, Ty, vmul(wz, wz)));
         const V s = vmul(vhorner<V, kWideDS, 1, 1>(x), x);
-        // q = S + (v + s (S + v)), the outer sum left unrounded for the update
+        // q = S + (v + s (S + v)), the outer sum left unrounded for the update; q.q from that
+        // sum, rounded (from x (1 + s)^2, one operation less, the error against 64 bits is
+        // up to half as large again)
         const V qx = vfma(s, Tx, vx), qy = vfma(s, Ty, vy), qz = vfma(s, wz, wz);
-        const V u = vfma(x, s, x);  // q.q = x (1 + s)^2
-        const V m = cos1(vmul(vhorner<V, kWideDC, 1, 0>(x), x), vfma(u, s, u));
+        const V fx = vadd(Sx, qx), fy = vadd(Sy, qy);
+        const V m = cos1(vmul(vhorner<V, kWideDC, 1, 0>(x), x),
+                         vfma(fx, fx, vfma(fy, fy, vmul(qz, qz))));
         const V nqx = vneg(qx), nqy = vneg(qy), nqz = vneg(qz), nSx = vneg(Sx), nSy = vneg(Sy);
         V dar = vfma(m, p.ar, vfma(qz, p.ai, vfma(nqy, p.br, vfma(qx, p.bi, p.lar))));
         V dai = vfma(m, p.ai, vfma(nqz, p.ar, vfma(nqy, p.bi, vfma(nqx, p.br, p.lai))));
