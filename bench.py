@@ -140,8 +140,8 @@ class ClockSampler:
 # means the counters are stale and the traffic is reported as null.
 KERNEL_TRAFFIC = {
     "evolve_group_kernel": {
-        "bytes": 76466688,
-        "source_sha256": "c9310a7057b83593eeebe4005f2bef4b96db229a8769beb6396996a3a65e5c28"},
+        "bytes": 74987776,
+        "source_sha256": "e2e42bd21c6fa1c942fb32eb33eb875c76845e6017d417f1b717942c2083234e"},
 }
 
 
