@@ -601,8 +601,9 @@ double f64_setup(const ReqDesc &r, int lanes)
 // a scheduler has one tile, whose operators then wait for its own updates (the other
 // schemes' operators are FP64 work themselves, in f64_cost).  A new state on 256^2: no step
 // 77 us on pairs, 44 flat; 16 steps 106, 78; 64 steps 207, 187.
-// *time, when given, receives the launch's.
-int f64_lanes(const std::vector<ReqDesc> &reqs, int scheme, double *time = nullptr)
+// *time, when given, receives the launch's; `copies` of every request.
+int f64_lanes(const std::vector<ReqDesc> &reqs, int scheme, int64_t copies = 1,
+              double *time = nullptr)
 {
     constexpr int shapes[3] = {1, 0, 4};
     constexpr double alone[3] = {26.6, 84.6, 5.5};
@@ -618,8 +619,9 @@ int f64_lanes(const std::vector<ReqDesc> &reqs, int scheme, double *time = nullp
             const int64_t n = r.step_end - r.step_begin;
             const double steps = static_cast<double>(lanes == 4 ? (n + 15) / 16 * 16 : n);
             const double setup = f64_setup(r, lanes);
-            tiles += f64_tiles(r, lanes);
-            work += static_cast<double>(f64_tiles(r, lanes)) * (f64_cost(r, lanes) * steps + setup);
+            tiles += copies * f64_tiles(r, lanes);
+            work += static_cast<double>(copies * f64_tiles(r, lanes)) *
+                    (f64_cost(r, lanes) * steps + setup);
             if (scheme == DSP_SCHEME_EXACT)
                 longest = std::max(longest, alone[k] * steps + setup);
         }
@@ -1293,13 +1295,13 @@ dsp_status run_one(dsp_grid *g, int64_t end, bool project, void *map)
 // Time segments for dsp_solve_segmented: at most what one launch carries, of at least 16
 // steps.  A segment has one warp per 32 points.  FP32_MIXED: one warp per scheduler, each
 // with a short run left and few columns to combine (64^2 x 2000 steps: 62 us with 2 to 5
-// segments, 74 with 1, 77 with 16, launches included; 2^2 x 20000 184 with 76, 198 with 96).
-// FP64: of the counts that fill the
-// schedulers evenly, the one with the least time of the fullest scheduler (f64_lanes' costs)
-// and of combining, a chain of FP64 operations of about 1.1 us a segment.  Measured (us, the
-// rule's count first; 38 and 41 are a count that fills them and one that does not):
-// 64^2 x 2000 324 (14), 322 (38), 358 (41); 128^2 x 20000 8990 (19), 9840 (39); 32^2 x 5000 246
-// (19), 372 (104); 16^2 x 50000 551 (76), 1680 (1041, in eleven launches).
+// segments, 74 with 1, 77 with 16, launches included; 2^2 x 20000 184 with 76, 198 with
+// 96).  FP64: of the counts that fill the schedulers evenly, the one with the least time of
+// the fullest scheduler (f64_lanes' costs) and of combining, a chain of FP64 operations of
+// about 1.1 us a segment.  Measured (us, segments in brackets, the rule's first; 41 and 39
+// do not fill them evenly): 64^2 x 2000 324 (14), 322 (38), 358 (41); 128^2 x 20000 8990
+// (19), 9840 (39); 32^2 x 5000 246 (19), 372 (104); 16^2 x 50000 551 (76), 1680 (1041, in
+// eleven launches).
 int64_t segment_count(const dsp_grid *g)
 {
     const int64_t warps = (g->n_points + 31) / 32, schedulers = 4 * static_cast<int64_t>(sm_count());
@@ -1308,6 +1310,8 @@ int64_t segment_count(const dsp_grid *g)
     if (g->precision != DSP_FP64)
         return std::max<int64_t>(1, std::min({most, static_cast<int64_t>(sm_count() / 2),
                                               (schedulers + warps - 1) / warps}));
+    std::vector<ReqDesc> segment(1, make_desc(g, 0, 0, false, nullptr));
+    segment[0].fresh = segment[0].init_identity = 1;
     int64_t best = 1, last = 0;
     double best_t = 0.0;
     for (int64_t fill = 0; fill <= 40; ++fill) {
@@ -1315,10 +1319,9 @@ int64_t segment_count(const dsp_grid *g)
         if (S == last)
             continue;
         last = S;
-        ReqDesc r = make_desc(g, 0, (g->n_steps + S - 1) / S, false, nullptr);
-        r.init_identity = 1;
+        segment[0].step_end = (g->n_steps + S - 1) / S;
         double t = 0.0;
-        f64_lanes(std::vector<ReqDesc>(static_cast<size_t>(S), r), g->scheme, &t);
+        f64_lanes(segment, g->scheme, S, &t);
         t += 33.0 * static_cast<double>(S) *
              std::max(1.0, static_cast<double>(warps) / static_cast<double>(schedulers));
         if (fill == 0 || t < best_t) {
