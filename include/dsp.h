@@ -54,11 +54,11 @@ typedef int32_t dsp_status;
                               built with -DDSP_BOUNDS_CHECK (accesses are skipped) */
 
 /* Arithmetic of the evolution. */
-#define DSP_FP64 0       /* the spinor and its update in FP64; STRANG_XY and MAGNUS4 all
-                            in FP64; EXACT's small parts cos(theta) - 1 and
-                            sin(theta)/theta - 1 in double-float FP32 arithmetic,
-                            within 2^-46 of themselves: below theta^2 2^-47 a step
-                            (7e-17 at theta = 0.1, an ulp of the state at 0.18)     */
+#define DSP_FP64 0       /* the spinor and its update in FP64.  EXACT's small parts
+                            cos(theta) - 1 and sin(theta)/theta - 1 in double-float FP32
+                            arithmetic, within 2^-46 of themselves: below theta^2 2^-47 a
+                            step (7e-17 at theta = 0.1, an ulp of the state at 0.18);
+                            STRANG_XY's and MAGNUS4's to FP64 rounding              */
 #define DSP_FP32_MIXED 1 /* spinor in compensated FP32 (hi + lo); dt P_n formed as
                             dt p_hi + (dt A_n + dt p_lo) with dt p an FP32 hi/lo
                             pair and dt A_n one FP32 per step, rounded so that

@@ -574,18 +574,33 @@ int64_t f64_tiles(const ReqDesc &r, int lanes)
     return lanes == 0 ? row_tiles(r, 4) : (r.n_points + 32 / lanes - 1) / (32 / lanes);
 }
 
-// A tile's share of a busy scheduler in an FP64 launch (launch_evolve_f64's lanes), in
-// units of 33 ns: its FP64 instructions and, for pairs, the waits between the two warps;
-// n = the series' degrees together.  Measured on grids of 16^2 to 512^2, 1000 steps, n of 6
-// to 12, to within 1%.  EXACT forms its series in FP32: no n.
-double f64_cost(const ReqDesc &r, int lanes)
+// What an FP64 step of a tile takes (launch_evolve_f64's lanes), in units of 33 ns:
+// `busy` its share of a busy scheduler, its FP64 instructions and, for pairs, the waits between
+// the two warps; `alone` on a scheduler with no other tile, where its operators, partly FP32
+// work, wait for its own updates.  n = the series' degrees together; EXACT forms its series in
+// FP32, the others up to kF64TailDegree but for their first terms: no n.  Measured on grids
+// of 16^2 to 512^2, 1000 steps, n of 6 to 12, to within 1%.
+struct F64Cost {
+    double busy, alone;
+};
+F64Cost f64_cost(const ReqDesc &r, int lanes)
 {
-    const int n = dsp::kLevelsF64[r.level].dc + dsp::kLevelsF64[r.level].ds;
-    if (r.scheme == DSP_SCHEME_EXACT)
-        return lanes == 1 ? 18.0 : lanes == 0 ? 64.2 : 4.55;
-    if (r.scheme == DSP_SCHEME_STRANG_XY)
-        return lanes == 1 ? 20.9 + 2.23 * n : lanes == 0 ? 60.6 + 1.25 * n : 5.3 + 0.555 * n;
-    return lanes == 1 ? 26.4 + 1.12 * n : 6.7 + 0.28 * n;
+    const dsp::SeriesLevel lv = dsp::kLevelsF64[r.level];
+    const int n = lv.dc + lv.ds;
+    const int k = lanes == 1 ? 0 : lanes == 0 ? 1 : 2;
+    if (r.scheme == DSP_SCHEME_EXACT) {
+        constexpr F64Cost c[3] = {{18.0, 26.6}, {64.2, 84.6}, {4.55, 5.5}};
+        return c[k];
+    }
+    if (lv.dc <= dsp::kF64TailDegree) {
+        constexpr F64Cost strang[3] = {{31.9, 42.0}, {67.5, 74.0}, {8.0, 9.5}};
+        constexpr F64Cost magnus[3] = {{31.7, 37.0}, {0.0, 0.0}, {8.0, 8.9}};
+        return r.scheme == DSP_SCHEME_STRANG_XY ? strang[k] : magnus[k];
+    }
+    const double strang[3] = {20.9 + 2.23 * n, 60.6 + 1.25 * n, 5.3 + 0.555 * n};
+    const double magnus[3] = {26.4 + 1.12 * n, 0.0, 6.7 + 0.28 * n};
+    const double busy = r.scheme == DSP_SCHEME_STRANG_XY ? strang[k] : magnus[k];
+    return {busy, busy};
 }
 // The same of what a tile does besides its steps: the initial spinors, once per lane (a
 // pair forms each point's four times; launches of one step on 512^2: 43, 43 and 171 us).
@@ -597,16 +612,13 @@ double f64_setup(const ReqDesc &r, int lanes)
 
 // Shape of an FP64 launch by the FP64 work of its fullest scheduler (dsp_f64.cu): 32
 // points flat, 4 rows x 32 columns (EXACT, STRANG_XY), or 8 points on a warp pair (whose
-// operators are formed for 16 steps at a time).  `alone` is what an EXACT step takes when
-// a scheduler has one tile, whose operators then wait for its own updates (the other
-// schemes' operators are FP64 work themselves, in f64_cost).  A new state on 256^2: no step
-// 77 us on pairs, 44 flat; 16 steps 106, 78; 64 steps 207, 187.
+// operators are formed for 16 steps at a time).  A new state on 256^2: no step 77 us on
+// pairs, 59 flat; 4 steps 95, 61; 16 steps 108, 95.
 // *time, when given, receives the launch's; `copies` of every request.
 int f64_lanes(const std::vector<ReqDesc> &reqs, int scheme, int64_t copies = 1,
               double *time = nullptr)
 {
     constexpr int shapes[3] = {1, 0, 4};
-    constexpr double alone[3] = {26.6, 84.6, 5.5};
     int best = 1;
     double best_t = 0.0;
     for (int k = 0; k < 3; ++k) {
@@ -619,11 +631,11 @@ int f64_lanes(const std::vector<ReqDesc> &reqs, int scheme, int64_t copies = 1,
             const int64_t n = r.step_end - r.step_begin;
             const double steps = static_cast<double>(lanes == 4 ? (n + 15) / 16 * 16 : n);
             const double setup = f64_setup(r, lanes);
+            const F64Cost cost = f64_cost(r, lanes);
             tiles += copies * f64_tiles(r, lanes);
             work += static_cast<double>(copies * f64_tiles(r, lanes)) *
-                    (f64_cost(r, lanes) * steps + setup);
-            if (scheme == DSP_SCHEME_EXACT)
-                longest = std::max(longest, alone[k] * steps + setup);
+                    (cost.busy * steps + setup);
+            longest = std::max(longest, cost.alone * steps + setup);
         }
         if (tiles == 0)
             break;

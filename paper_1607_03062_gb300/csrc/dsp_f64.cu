@@ -103,21 +103,49 @@ __device__ __forceinline__ double horner_f64(double x)
         return fma(horner_f64<D, K + 1, ODD>(x), x, c);
 }
 
+// cos and sinc of STRANG_XY and MAGNUS4 from x = theta^2 in FP64.  Up to cosine degree
+// kF64TailDegree (theta below ~0.16) the terms from x^2 on are summed in double-float beside the
+// FP64 work: at most theta^4/24, they are off by less than 1e-20 at theta 0.1, so cos and
+// sinc are rounded as in the FP64 series (measured on the CPU over random theta: cos the
+// same, sinc theta 0.8 of its error), for 2 FP64 operations each, whatever the degree.  (All
+// of cos - 1 and sinc - 1 as pairs of floats, 1 each, is off by ~2^-50 of theta^2/2 with one
+// sign: 1e5 steps at theta 0.06 put 1.6e-13 into the state instead of 1.7e-14.)
+// c = cos - 1 + 1 and s1 = sinc - 1 (DC <= kF64TailDegree).
+template <int DC, int DS>
+__device__ __forceinline__ void cos_sinc_f64(double x, double &c, double &s1)
+{
+    float xh, xl, x2h, x2l, th, tl, uh, ul;
+    split_f64(x, xh, xl);
+    df_mul(xh, xl, xh, xl, x2h, x2l);
+    horner_df<DC, 2, 0>(xh, xl, th, tl);
+    df_mul(x2h, x2l, th, tl, uh, ul);
+    c = 1.0 + fma(x, -0.5, df_to_f64(uh, ul));
+    horner_df<DS, 2, 1>(xh, xl, th, tl);
+    df_mul(x2h, x2l, th, tl, uh, ul);
+    s1 = fma(x, -1.0 / 6.0, df_to_f64(uh, ul));
+}
+
 // The FP64 MAGNUS4 step's operator: n = (dt Pbar, n_z), n_z = Pbar x D; c = cos|n|, q and
-// qz = sinc|n| n, all in FP64: 26 + dc + ds FP64 operations a step.  (Its small parts as
-// pairs of floats, 26, are off by ~2^-50 of theta^2/2 with one sign: 1e5 steps at theta
-// 0.06 put 1.6e-13 into the state instead of 1.7e-14.)
+// qz = sinc|n| n: 31 FP64 operations a step with the update, 26 + dc + ds above kF64TailDegree.
 template <int DC, int DS>
 __device__ __forceinline__ void operator_f64_magnus(double Px, double Py, double2 d, double &c,
                                                     double &qr, double &qi, double &qz)
 {
     const double nz = fma(Px, d.y, -(Py * d.x));
     const double x = fma(Px, Px, fma(Py, Py, nz * nz));
-    c = horner_f64<DC, 0, 0>(x);
-    const double sn = horner_f64<DS, 0, 1>(x);
-    qr = sn * Py;
-    qi = sn * Px;
-    qz = sn * nz;
+    if constexpr (DC <= kF64TailDegree) {
+        double s1;
+        cos_sinc_f64<DC, DS>(x, c, s1);
+        qr = fma(s1, Py, Py);
+        qi = fma(s1, Px, Px);
+        qz = fma(s1, nz, nz);
+    } else {
+        c = horner_f64<DC, 0, 0>(x);
+        const double sn = horner_f64<DS, 0, 1>(x);
+        qr = sn * Py;
+        qi = sn * Px;
+        qz = sn * nz;
+    }
 }
 template <int DC, int DS>
 __device__ __forceinline__ void step_f64_magnus(F64Point &s, double Px, double Py, double2 d)
@@ -143,15 +171,20 @@ __device__ __forceinline__ void apply_f64(F64Point &s, double c, double qr, doub
     s.ar = nar; s.ai = nai; s.br = nbr; s.bi = nbi;
 }
 
-// STRANG_XY's parts of one coordinate, {cos P, sin P}, in FP64 (as MAGNUS4's; pairs of
-// floats put 1.6e-13 instead of 2.2e-14 into the state there); and its step from those of
-// x and y, c = cos y cos x, q = sin y + i cos y sin x.  20 + 2 dc + 2 ds FP64 operations;
-// on row tiles the parts of a row and of a column are formed once.
+// STRANG_XY's parts of one coordinate, {cos P, sin P}; and its step from those of x and y,
+// c = cos y cos x, q = sin y + i cos y sin x.  30 FP64 operations a step, 20 + 2 dc + 2 ds
+// above kF64TailDegree; on row tiles the parts of a row and of a column are formed once.
 template <int DC, int DS>
 __device__ __forceinline__ double2 strang_part(double P)
 {
     const double x = P * P;
-    return make_double2(horner_f64<DC, 0, 0>(x), P * horner_f64<DS, 0, 1>(x));
+    if constexpr (DC <= kF64TailDegree) {
+        double c, s1;
+        cos_sinc_f64<DC, DS>(x, c, s1);
+        return make_double2(c, fma(s1, P, P));
+    } else {
+        return make_double2(horner_f64<DC, 0, 0>(x), P * horner_f64<DS, 0, 1>(x));
+    }
 }
 __device__ __forceinline__ void step_f64_strang(F64Point &s, double2 x, double2 y)
 {
@@ -221,12 +254,12 @@ __device__ __forceinline__ void strip64_step(F64Point (&pt)[H], double tx, doubl
 // Warps (in one shape, pairs of warps) work alone: their own double-buffered bulk copies
 // of the table with bounded waits, no CTA-wide barrier, and the host picks the shape that
 // loads the fullest scheduler least (f64_lanes in dsp_api.cpp).  FP64 instructions per
-// step of a tile (EXACT; STRANG_XY and MAGNUS4 at series degrees 4 and 3) and its points:
+// step of a tile (EXACT; STRANG_XY and MAGNUS4 up to kF64TailDegree) and its points:
 //   rows   32 columns x 4 rows: the dt P_x part once per lane, the dt P_y part once per
-//          row and step in a shared table                       65, 67, - for 128
-//   flat   32 consecutive points, a lane each                   18, 34, 33 for 32
+//          row and step in a shared table                       65, 65, - for 128
+//   flat   32 consecutive points, a lane each                   18, 30, 31 for 32
 //   pair   8 points, a lane per real component in one warp, the operators of four
-//          steps at once in the other                           4.5, 8.5, 8.3 for 8
+//          steps at once in the other                           4.5, 7.5, 7.8 for 8
 // Every FP64 operation of a point is the same in every shape (same operands, same
 // rounding), so its result is bitwise the same.  The projection is the projection
 // kernel's, on the state these leave.

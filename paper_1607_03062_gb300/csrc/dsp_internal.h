@@ -39,6 +39,10 @@ constexpr SeriesLevel kLevelsF32[kNumLevels] = {{2, 1}, {2, 2}, {3, 2}, {3, 3},
 constexpr SeriesLevel kLevelsF64[kNumLevels] = {{3, 3}, {4, 3}, {4, 4}, {5, 5},
                                                  {6, 6}, {8, 8}, {11, 11}, {16, 16}};
 
+// FP64 STRANG_XY and MAGNUS4 sum their series' terms from theta^4 on in double-float up to
+// this cosine degree (cos_sinc_f64 in dsp_f64.cu).
+constexpr int kF64TailDegree = 5;
+
 // FP32_MIXED step groups of EXACT and STRANG_XY divide each step by its real
 // diagonal (the tan-normalised chain of the kernels) and need, in x = theta^2,
 //   tan(theta)/theta = sum_k kTanSeries[k] x^k   (4^(k+1) (4^(k+1) - 1) |B_(2k+2)| / (2k+2)!)
