@@ -140,8 +140,8 @@ class ClockSampler:
 # means the counters are stale and the traffic is reported as null.
 KERNEL_TRAFFIC = {
     "evolve_group_kernel": {
-        "bytes": 74987776,
-        "source_sha256": "e2e42bd21c6fa1c942fb32eb33eb875c76845e6017d417f1b717942c2083234e"},
+        "bytes": 76638464,
+        "source_sha256": "4434aaa16cb2c5b086efb16d08fd26d77335b682bb6db66e91fb9a9495989b1e"},
 }
 
 
