@@ -378,9 +378,13 @@ ReqDesc make_desc(const dsp_grid *g, int64_t begin, int64_t end, bool project, v
     r.tdeg = g->tdeg;
     r.withhold_first_copy = g->withhold_next ? 1 : 0;
     r.table_steps = g->table_cap;
-    // (a launch without one whole group of the smallest size has no use for them)
+    // A launch without one whole group of the smallest size has no use for them, unless it
+    // is the end of a run cut on a multiple of 16: in one launch those steps are taken by
+    // the group kernel, alone, and the pieces promise the same bits.
     constexpr int64_t least = dsp::group_size(dsp::kNumGroupSizes - 1);
-    if (g->by_groups && (begin + least - 1) / least < end / least) {
+    const bool whole = (begin + least - 1) / least < end / least;
+    const bool tail = begin < end && end == g->n_steps && begin % dsp::kGroupMax == 0;
+    if (g->by_groups && (whole || tail)) {
         const GroupMemory m(g);
         r.by_groups = 1;
         const unsigned char *base = static_cast<const unsigned char *>(g->groups);
