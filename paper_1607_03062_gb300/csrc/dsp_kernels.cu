@@ -147,7 +147,9 @@ __device__ __forceinline__ void project_pair(const ReqDesc &R, const unsigned ch
 }
 
 // GROUPS: the launch has requests that may have gone step by step (ReqDesc::by_groups).
-template <int PREC, bool GROUPS>
+// NEAR: neighbouring granules go to one SM; else they go to the CTAs in turn, so that a small
+// grid's spread over the SMs and the last round's over all of them (see launch_project).
+template <int PREC, bool GROUPS, bool NEAR>
 __global__ void __launch_bounds__(ProjShape<PREC>::threads, 1)
     project_kernel(const __grid_constant__ EvolveArgs args)
 {
@@ -160,13 +162,8 @@ __global__ void __launch_bounds__(ProjShape<PREC>::threads, 1)
     uint64_t *bars = reinterpret_cast<uint64_t *>(proj_dyn + Sh::warps * Sh::warp_bytes) + NB * w;
     constexpr int kGranPerTile = kTilePoints / kGranule;
     const int total = args.total_tiles * kGranPerTile;  // granules of the launch
-    // Granules go to the CTAs in turn, so that a small grid's spread over the SMs and the
-    // last round's over all of them; a large FP32_MIXED grid keeps neighbouring granules on
-    // one SM (us a launch, in turn and neighbours: 100 x 75 6.1 and 7.6, 1024^2 8.4 and 10.4,
-    // 2048^2 32.5 and 32.0, 4096^2 101.4 and 99.0).
     const int nw = gridDim.x * Sh::warps;
-    const int wid = PREC == 0 || total < 4 * nw ? w * gridDim.x + blockIdx.x
-                                                : blockIdx.x * Sh::warps + w;
+    const int wid = NEAR ? blockIdx.x * Sh::warps + w : w * gridDim.x + blockIdx.x;
     // A request that went step by step has been projected there: nothing to load or to do.
     // (Looked up once per request: granules of one follow each other.  A warp's first
     // granule is loaded meanwhile, whatever comes of it.)
@@ -447,16 +444,16 @@ cudaError_t launch_evolve_strip(const EvolveArgs &args, int scheme, int strip_h,
     return half ? launch_evolve_strip_s2_np1(args, stream) : launch_evolve_strip_s2_np2(args, stream);
 }
 
-template <int PREC, bool GROUPS>
+template <int PREC, bool GROUPS, bool NEAR>
 static cudaError_t launch_project(const EvolveArgs &args, int grid, cudaStream_t stream)
 {
     using Sh = ProjShape<PREC>;
     // the warps' rings are above the 48 KB a kernel gets without asking
     const cudaError_t e = cudaFuncSetAttribute(
-        project_kernel<PREC, GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::smem);
+        project_kernel<PREC, GROUPS, NEAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::smem);
     if (e != cudaSuccess)
         return e;
-    project_kernel<PREC, GROUPS><<<grid, Sh::threads, Sh::smem, stream>>>(args);
+    project_kernel<PREC, GROUPS, NEAR><<<grid, Sh::threads, Sh::smem, stream>>>(args);
     return cudaGetLastError();
 }
 
@@ -470,15 +467,26 @@ cudaError_t launch_project(const EvolveArgs &args, int precision, cudaStream_t s
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess)
         return e;
-    bool groups = false;
-    for (int i = 0; i < args.nreq; ++i)
+    bool groups = false, whole = true;
+    for (int i = 0; i < args.nreq; ++i) {
         groups = groups || args.r[i].by_groups;
+        whole = whole && args.r[i].nx % kGranule == 0;
+    }
     // one CTA per SM, no more CTAs than granules
     const int granules = args.total_tiles * (kTilePoints / kGranule);
     const int grid = granules < sms ? granules : sms;
-    return precision != 1 ? launch_project<0, false>(args, grid, stream)
-           : groups       ? launch_project<1, true>(args, grid, stream)
-                          : launch_project<1, false>(args, grid, stream);
+    if (precision != 1)
+        return launch_project<0, false, false>(args, grid, stream);
+    // Rows of whole granules, four or more of them a warp: neighbours on one SM (us a launch on
+    // buffers not in L2, in turn and neighbours: 2048^2 32.7 and 32.5, 3072 x 2000 44.3 and 43.4,
+    // 4096^2 101.9 and 100.2).  Fewer or ragged ones in turn (100 x 75 6.1 and 7.6, 1024^2 8.4
+    // and 10.4, 1801 x 2001 31.1 and 31.6); the order as a constant, since one picked in the
+    // kernel costs every grid up to 1% (1500^2 22.6 and 22.9).
+    if (whole && granules >= 4 * grid * ProjShape<1>::warps)
+        return groups ? launch_project<1, true, true>(args, grid, stream)
+                      : launch_project<1, false, true>(args, grid, stream);
+    return groups ? launch_project<1, true, false>(args, grid, stream)
+                  : launch_project<1, false, false>(args, grid, stream);
 }
 
 cudaError_t launch_finalize(const FinalizeArgs &args, cudaStream_t stream)
